@@ -111,7 +111,8 @@ enum { SS_C1 = 0, SS_R, SS_C3, SS_AV, SS_TAU, SCS };
 // <= -2 interface record (-2 - r).
 constexpr int32_t NB_BOUNDARY = -1;
 
-constexpr int MAX_TARGETS = 4;
+constexpr int MAX_TARGETS = 6;        // of a stage launch: the adjoint of an accepted tableau may need six
+constexpr int MAX_PLAN_TARGETS = 4;   // of a forward tableau's stage (build_plan)
 constexpr int MAX_SOURCES = 8;
 
 // Simulation clock read by graph-replayed stage kernels: the time of stage
@@ -160,10 +161,28 @@ struct StageArgsT {
     double shot_f0, shot_t0, shot_amp;
 };
 
-// MODE_RAW writes the rate before the per-cell material factors (and, in
-// solids, before the stress mixing): the derivative of the rate with respect
-// to those factors, used by the adjoint gradient.
-enum { MODE_TRACES = 0, MODE_STAGE = 1, MODE_APPLY = 2, MODE_RAW = 3 };
+// MODE_GRAD forms the rate before the per-cell material factors (and, in
+// solids, before the stress mixing), which is the derivative of the rate with
+// respect to those factors, and accumulates one backward stage's share of the
+// adjoint gradients from it (GradArgsT).
+enum { MODE_TRACES = 0, MODE_STAGE = 1, MODE_APPLY = 2, MODE_GRAD = 3 };
+
+// The adjoint side of a MODE_GRAD launch: the adjoint stage value z with its
+// traces under the coupling-reversed operator, and the gradient sums.  The
+// stage's adjoint is mu = w S M z (adjoint.cu).
+template <class T>
+struct GradArgsT {
+    const T* z;
+    const T* tr_z;
+    const double* if_coef_z;   // interface coefficients of the coupling-reversed operator
+    double w;
+    const double* mass_f;      // [2][Nf]: rho h^2, h^2/kappa
+    const double* mass_s;      // [4][Ns]: h^2 compliance (3), rho h^2
+    double* grad_f;            // [2][Nf]: d/d(1/(rho h)), d/d(kappa/h)
+    double* grad_s;            // [4][Ns]: d/d(c1, r, c3, 1/(rho h))
+    double* gstab;             // [Nf + Ns]: sum of face integrals of the jump products
+    double* wgrad;             // [n_src]: mu^T g (may be null)
+};
 
 // ERK plan (stage.cu): row i of the extended tableau (a_{s+1,:} = b) is the
 // partial sum P_i = U^{n-1} + dt sum_j a_ij k_j.
@@ -188,6 +207,10 @@ void launch_stage_f64(const hho_ops* ops, int mode, StageArgsT<double>& a, int n
                       bool sources, void* stream);
 void launch_stage_f32(const hho_ops* ops, int mode, StageArgsT<float>& a, int n_shots, double tn, int j, double cdt,
                       bool sources, void* stream);
+void launch_grad_f64(const hho_ops* ops, StageArgsT<double>& a, const GradArgsT<double>& g, double tn, int j, double cdt,
+                     void* stream);
+void launch_grad_f32(const hho_ops* ops, StageArgsT<float>& a, const GradArgsT<float>& g, double tn, int j, double cdt,
+                     void* stream);
 void launch_record_f64(const hho_ops* ops, const double* state, double* out, void* stream);
 // nsteps ERK steps of one FP32 state (the batched FP32 path with one shot)
 int erk_steps_f32(hho_ops* ops, const hho_tableau* tab, double t0, double dt, int64_t nsteps, float* d_state,

@@ -526,6 +526,277 @@ __device__ __forceinline__ T shot_src_value(const StageArgsT<T>& A) {
     return T(ricker_dev(stage_time(A.clock, A.dt, A.c_stage), A.shot_f0, A.shot_t0, A.shot_amp));
 }
 
+// ---- adjoint gradients (MODE_GRAD) ---------------------------------------------------
+// Sums of products in at least FP64 accuracy for FP64 values, and exact
+// products with double-float sums for FP32 values (FP32 pipes; an FP64 sum of
+// FP32 products would spend most of its time in conversions on the FP64 pipe).
+template <class T>
+struct Wide {
+    using type = double;
+};
+template <>
+struct Wide<float> {
+    using type = f2x;
+};
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ f2x widen(float x) { return f2x(x, 0.0f); }
+template <class T>
+struct WideData;   // operator data in the wide type
+template <>
+struct WideData<double> {
+    __device__ static const double* beta_f(const DevOps& o) { return o.beta_f; }
+    __device__ static const double* beta_s(const DevOps& o) { return o.beta_s; }
+    __device__ static const double* cls(const DevOps& o) { return o.cls_dbl; }
+};
+template <>
+struct WideData<float> {
+    __device__ static const f2x* beta_f(const DevOps& o) { return o.beta_f_x; }
+    __device__ static const f2x* beta_s(const DevOps& o) { return o.beta_s_x; }
+    __device__ static const f2x* cls(const DevOps& o) { return o.cls_x; }
+};
+
+// M0's parity pattern on rectangles: it couples equal parities of both exponents.
+__host__ __device__ constexpr bool mass_nz(int i, int j) {
+    return ((ea(i) + ea(j)) & 1) == 0 && ((eb(i) + eb(j)) & 1) == 0;
+}
+// y = M0 x with the class mass matrix (stored n x n, rows unpadded), in the
+// wide type: mu = S M z is a difference of large terms where M0 is badly
+// conditioned, so FP32 matrix entries or sums would cost the FP32 gradient
+// about a factor of two in accuracy.
+template <class T, int K, bool RECT, class W>
+__device__ __forceinline__ void mass_apply(const W* __restrict__ M0, const T* x, W* y) {
+    constexpr int n = Dims<K>::n;
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+        W s(0);
+#pragma unroll
+        for (int j = 0; j < n; ++j)
+            if (!RECT || mass_nz(i, j)) s = fma(__ldg(M0 + i * n + j), widen(x[j]), s);
+        y[i] = s;
+    }
+}
+template <class T, int K, class W>
+__device__ __forceinline__ void mass_apply(const W* __restrict__ M0, bool rect, const T* x, W* y) {
+    if (rect) mass_apply<T, K, true>(M0, x, y);
+    else mass_apply<T, K, false>(M0, x, y);
+}
+template <class T, int K, class W>
+__device__ __forceinline__ W coef_dot(const T* x, const W* y) {
+    W s(0);
+#pragma unroll
+    for (int i = 0; i < Dims<K>::n; ++i) s = fma(widen(x[i]), y[i], s);
+    return s;
+}
+
+// acc + z^T M0 g in the wide type for one field of a cell (z with stride N):
+// the source cells of the wavelet gradient only.
+template <class T, int K>
+__device__ __noinline__ typename Wide<T>::type wide_form(const DevOps& op, const int* ci, const T* z, int N,
+                                                         const T* g, typename Wide<T>::type acc) {
+    using W = typename Wide<T>::type;
+    constexpr int n = Dims<K>::n;
+    const W* M0 = WideData<T>::cls(op) + __ldg(ci + CI_DOFF);
+    for (int i = 0; i < n; ++i) {
+        W y(0);
+        for (int j = 0; j < n; ++j) y = fma(M0[i * n + j], widen(z[(size_t)j * N]), y);
+        acc = fma(y, widen(g[i]), acc);
+    }
+    return acc;
+}
+
+// The integral over a face of unit length of the product of two functions
+// given by their face coefficients:
+// (psi_l, psi_m) = rho0^(l+m) / (l+m+1) on a face of unit length for even
+// l + m, else 0 (constants of the unrolled sums).
+__host__ __device__ constexpr double face_gram(int l, int m) {
+    if ((l + m) & 1) return 0.0;
+    double r = 1.0;
+    for (int e = 0; e < l + m; ++e) r *= FACE_RHO;
+    return r / (l + m + 1);
+}
+// a gram entry in the wide type; called with unrolled constants, so that the
+// double-float split is folded and issues no FP64 instruction
+template <class W>
+__device__ __forceinline__ W gram_const(double v) {
+    return W(v);
+}
+template <int K, class W>
+__device__ __forceinline__ W face_inner(const W* a, const W* b, W acc) {
+    constexpr int f = Dims<K>::f;
+#pragma unroll
+    for (int l = 0; l < f; ++l) {
+        W t = l == 0 ? b[l] : gram_const<W>(face_gram(l, l)) * b[l];   // (psi_0, psi_0) = 1
+#pragma unroll
+        for (int m = 0; m < f; ++m)
+            if (m != l && ((l + m) & 1) == 0) t = fma(gram_const<W>(face_gram(l, m)), b[m], t);
+        acc = fma(a[l], t, acc);
+    }
+    return acc;
+}
+
+// Jump of the primal trace on local face j in the wide type, from the
+// published traces tr (fluid part then solid part) and interface
+// coefficients `co6`; NC = 1 component in a fluid cell, 2 in a solid cell.
+template <class T, int K, int NC, class W>
+__device__ __forceinline__ void wide_jump(const DevOps& op, const T* __restrict__ tr, const double* __restrict__ co6,
+                                          int slot, int nb, W* jmp) {
+    constexpr int f = Dims<K>::f;
+    const size_t S = NC == 1 ? op.SF : op.SS;
+    const T* trf = tr;
+    const T* trs = tr + (size_t)2 * f * op.SF;
+    const T* own = NC == 1 ? trf : trs;
+#pragma unroll
+    for (int i = 0; i < NC * f; ++i) jmp[i] = widen(__ldg(own + (NC * f + i) * S + slot));
+    if (nb >= 0) {
+        const W be = __ldg((NC == 1 ? WideData<T>::beta_f(op) : WideData<T>::beta_s(op)) + slot);
+#pragma unroll
+        for (int i = 0; i < NC * f; ++i) {
+            const W w = widen(__ldg(own + i * S + nb));
+            jmp[i] = ((i % f) & 1) ? fma(-be, w, jmp[i]) : fma(be, w, jmp[i]);
+        }
+    } else if (nb < NB_BOUNDARY) {
+        const int r = -2 - nb;
+        const int no = __ldg(op.if_nb + r);
+        const double* co = co6 + 6 * r;
+        if constexpr (NC == 1) {
+            const W bx(__ldg(co + 1)), by(__ldg(co + 2));
+#pragma unroll
+            for (int l = 0; l < f; ++l) {
+                const W ws = fma(bx, widen(__ldg(trs + (size_t)l * op.SS + no)), by * widen(__ldg(trs + (size_t)(f + l) * op.SS + no)));
+                jmp[l] = (l & 1) ? jmp[l] - ws : jmp[l] + ws;
+            }
+        } else {
+            const W b0(__ldg(co + 4)), b1(__ldg(co + 5));
+#pragma unroll
+            for (int l = 0; l < f; ++l) {
+                const W w = widen(__ldg(trf + (size_t)l * op.SF + no));
+                jmp[l] = (l & 1) ? fma(-b0, w, jmp[l]) : fma(b0, w, jmp[l]);
+                jmp[f + l] = (l & 1) ? fma(-b1, w, jmp[f + l]) : fma(b1, w, jmp[f + l]);
+            }
+        }
+    }
+}
+
+// Stabilisation-weight part of one backward stage: gstab += w sum_F |F|/h
+// (jump of Y, jump of z)_F over the cell's faces.
+template <class T, int K, int NC>
+__device__ __forceinline__ void tau_grad(const StageArgsT<T>& A, const GradArgsT<T>& G, const CellCtx<T>& c,
+                                         const int* ci, int g) {
+    using W = typename Wide<T>::type;
+    constexpr int f = Dims<K>::f, FS = Dims<K>::FS;
+    const DevOps& op = A.op;
+    const double* cd = op.cls_dbl + __ldg(ci + CI_DOFF) + Dims<K>::M0P;
+    double acc = 0.0;
+#pragma unroll 1
+    for (int j = 0; j < c.nF; ++j) {
+        const int slot = c.sbase + j * c.npad + c.lq;
+        const int nb = __ldg((NC == 1 ? op.nb_f : op.nb_s) + slot);
+        W jy[NC * f], jz[NC * f];
+        wide_jump<T, K, NC, W>(op, A.tr_in, op.if_coef, slot, nb, jy);
+        wide_jump<T, K, NC, W>(op, G.tr_z, G.if_coef_z, slot, nb, jz);
+        W sum(0);
+#pragma unroll
+        for (int e = 0; e < NC; ++e) sum = face_inner<K, W>(jy + e * f, jz + e * f, sum);
+        acc = fma(__ldg(cd + j * FS + 2), double(sum), acc);   // |F| / h
+    }
+    G.gstab[g] = fma(G.w, acc, G.gstab[g]);
+}
+
+// Gradients of one fluid cell: U holds the raw rates [grad p (2), div m].
+// With mu = w S M z, mu^T raw is a sum of z^T M0 raw per field.
+template <class T, int K>
+__device__ __forceinline__ void fluid_grad(const StageArgsT<T>& A, const GradArgsT<T>& G, const CellCtx<T>& c,
+                                           const int* ci, bool rect, const T* U) {
+    constexpr int n = Dims<K>::n;
+    using W = typename Wide<T>::type;
+    const int q = c.q;
+    const W* M0 = WideData<T>::cls(A.op) + __ldg(ci + CI_DOFF);
+    W qf[3];
+#pragma unroll
+    for (int fld = 0; fld < 3; ++fld) {
+        T u[n], z[n];
+        W y[n];
+#pragma unroll
+        for (int i = 0; i < n; ++i) u[i] = U[fld * n + i];
+        mass_apply<T, K>(M0, rect, u, y);
+        load_state<n>(G.z, c.N, q, fld * n, z);
+        qf[fld] = coef_dot<T, K, W>(z, y);
+    }
+    const double cm = G.mass_f[q], cp = G.mass_f[c.N + q];
+    G.grad_f[q] = fma(-G.w * cm, double(qf[0]) + double(qf[1]), G.grad_f[q]);
+    G.grad_f[c.N + q] = fma(G.w * cp, double(qf[2]), G.grad_f[c.N + q]);
+    if (G.wgrad)
+        for (int s = 0; s < A.n_src; ++s)
+            if (A.src_dom[s] == 0 && A.src_q[s] == q) {
+                const W acc = wide_form<T, K>(A.op, ci, G.z + (size_t)2 * n * c.N + q, c.N,
+                                              A.src_g + (size_t)s * 2 * n, W(0));
+                G.wgrad[s] = G.w * cp * double(acc);
+            }
+    tau_grad<T, K, 1>(A, G, c, ci, q);
+}
+
+// Gradients of one solid cell: U holds the raw rates [e_xx, e_yy, e_xy, div s (2)].
+template <class T, int K>
+__device__ __forceinline__ void solid_grad(const StageArgsT<T>& A, const GradArgsT<T>& G, const CellCtx<T>& c,
+                                           const int* ci, bool rect, const T* U) {
+    constexpr int n = Dims<K>::n;
+    using W = typename Wide<T>::type;
+    const int q = c.q;
+    const size_t N = c.N;
+    const W* M0 = WideData<T>::cls(A.op) + __ldg(ci + CI_DOFF);
+    const T* zb = G.z + (size_t)3 * n * A.op.Nf;
+    W q00, q01, q10, q11, q22, qv;   // q_ab = z_a^T M0 raw_b
+    {
+        T u[n], z[n];
+        W y0[n], y1[n];
+#pragma unroll
+        for (int i = 0; i < n; ++i) u[i] = U[i];
+        mass_apply<T, K>(M0, rect, u, y0);
+#pragma unroll
+        for (int i = 0; i < n; ++i) u[i] = U[n + i];
+        mass_apply<T, K>(M0, rect, u, y1);
+        load_state<n>(zb, c.N, q, 0, z);
+        q00 = coef_dot<T, K, W>(z, y0);
+        q01 = coef_dot<T, K, W>(z, y1);
+        load_state<n>(zb, c.N, q, n, z);
+        q10 = coef_dot<T, K, W>(z, y0);
+        q11 = coef_dot<T, K, W>(z, y1);
+    }
+    W qs[3];
+#pragma unroll
+    for (int fld = 2; fld < 5; ++fld) {
+        T u[n], z[n];
+        W y[n];
+#pragma unroll
+        for (int i = 0; i < n; ++i) u[i] = U[fld * n + i];
+        mass_apply<T, K>(M0, rect, u, y);
+        load_state<n>(zb, c.N, q, fld * n, z);
+        qs[fld - 2] = coef_dot<T, K, W>(z, y);
+    }
+    q22 = qs[0];
+    qv = qs[1] + qs[2];
+    const double d0 = G.mass_s[q], d1 = G.mass_s[N + q], d2 = G.mass_s[2 * N + q], rv = G.mass_s[3 * N + q];
+    const double c1 = A.op.scal_s[SS_C1 * N + q], r = A.op.scal_s[SS_R * N + q];
+    // mu_xx = -(d0 z_xx + d1 z_yy), mu_yy = -(d1 z_xx + d0 z_yy), mu_xy = -d2 z_xy (times M0 and w)
+    const double xx_xx = d0 * double(q00) + d1 * double(q10), xx_yy = d0 * double(q01) + d1 * double(q11);
+    const double yy_xx = d1 * double(q00) + d0 * double(q10), yy_yy = d1 * double(q01) + d0 * double(q11);
+    const double w = G.w;
+    G.grad_s[q] = fma(-w, xx_xx + r * xx_yy + yy_yy + r * yy_xx, G.grad_s[q]);          // d/dc1
+    G.grad_s[N + q] = fma(-w * c1, xx_yy + yy_xx, G.grad_s[N + q]);                     // d/dr
+    G.grad_s[2 * N + q] = fma(-w * d2, double(q22), G.grad_s[2 * N + q]);               // d/dc3
+    G.grad_s[3 * N + q] = fma(w * rv, double(qv), G.grad_s[3 * N + q]);                 // d/d(1/(rho h))
+    if (G.wgrad)
+        for (int s = 0; s < A.n_src; ++s)
+            if (A.src_dom[s] == 1 && A.src_q[s] == q) {
+                W acc(0);
+                for (int e = 0; e < 2; ++e)
+                    acc = wide_form<T, K>(A.op, ci, zb + (size_t)(3 + e) * n * N + q, c.N,
+                                          A.src_g + ((size_t)s * 2 + e) * n, acc);
+                G.wgrad[s] = w * rv * double(acc);
+            }
+    tau_grad<T, K, 2>(A, G, c, ci, A.op.Nf + q);
+}
+
 // ---- fluid cells -------------------------------------------------------------------
 // Lift the face jump of one face into the raw rate accumulators
 // (kmx, kmy: grad p part; kp: div m part, tau folded).
@@ -695,7 +966,8 @@ __device__ __forceinline__ void fluid_rect_traces(const StageArgsT<T>& A, const 
 }
 
 template <class T, int K, int MODE>
-__device__ __forceinline__ void fluid_cell(const StageArgsT<T>& A, int q, int shot, const T* cd_smem, T* acc_smem) {
+__device__ __forceinline__ void fluid_cell(const StageArgsT<T>& A, int q, int shot, const T* cd_smem, T* acc_smem,
+                                           const GradArgsT<T>* G = nullptr) {
     constexpr int n = Dims<K>::n, f = Dims<K>::f;
     const DevOps& op = A.op;
     const int cls = __ldg(op.warp_class + (q >> 5));
@@ -729,7 +1001,7 @@ __device__ __forceinline__ void fluid_cell(const StageArgsT<T>& A, int q, int sh
         T* kmy = U + n;
         T* kp = U + 2 * n;
         if constexpr (L2Prefetch<T, K>::mask != 0)
-            prefetch_cell<T, K, 3 * n, f, 0, MODE != MODE_RAW>(A, c, soff, c.trf_in, c.SF, op.nb_f,
+            prefetch_cell<T, K, 3 * n, f, 0, MODE != MODE_GRAD>(A, c, soff, c.trf_in, c.SF, op.nb_f,
                                                             OpData<T>::beta_f(op), rect ? 4 : c.nF);
         {
             T u[n];
@@ -742,7 +1014,7 @@ __device__ __forceinline__ void fluid_cell(const StageArgsT<T>& A, int q, int sh
             add_ddy<T, K>(u, kp);
         }
         if constexpr (L2Prefetch<T, K>::mask != 0)
-            prefetch_cell<T, K, 3 * n, f, 1, MODE != MODE_RAW>(A, c, soff, c.trf_in, c.SF, op.nb_f,
+            prefetch_cell<T, K, 3 * n, f, 1, MODE != MODE_GRAD>(A, c, soff, c.trf_in, c.SF, op.nb_f,
                                                             OpData<T>::beta_f(op), rect ? 4 : c.nF);
         if (rect) {
             // faces 0 (s = -1) and 2 (s = +1) are horizontal, 1 (s = +1) and 3 (s = -1) vertical
@@ -774,10 +1046,8 @@ __device__ __forceinline__ void fluid_cell(const StageArgsT<T>& A, int q, int sh
 #pragma unroll
             for (int i = 0; i < n; ++i) kp[i] = fma(w, g[i], kp[i]);
         }
-        if constexpr (MODE == MODE_RAW) {
-            T* dst = A.tgt[0].dst + soff;
-#pragma unroll
-            for (int i = 0; i < 3 * n; ++i) dst[(size_t)i * c.N + q] = norm(U[i]);
+        if constexpr (MODE == MODE_GRAD) {
+            fluid_grad<T, K>(A, *G, c, ci, rect, U);
             return;
         }
         const T sc[3] = {Am, Ap, T(0)};
@@ -967,7 +1237,8 @@ __device__ __forceinline__ void solid_rect_traces(const StageArgsT<T>& A, const 
 }
 
 template <class T, int K, int MODE>
-__device__ __forceinline__ void solid_cell(const StageArgsT<T>& A, int q, int shot, const T* cd_smem, T* acc_smem) {
+__device__ __forceinline__ void solid_cell(const StageArgsT<T>& A, int q, int shot, const T* cd_smem, T* acc_smem,
+                                           const GradArgsT<T>* G = nullptr) {
     constexpr int n = Dims<K>::n, f = Dims<K>::f;
     const DevOps& op = A.op;
     const int cls = __ldg(op.warp_class + op.n_warps_f + (q >> 5));
@@ -1004,7 +1275,7 @@ __device__ __forceinline__ void solid_cell(const StageArgsT<T>& A, int q, int sh
         T* kvx = U + 3 * n;
         T* kvy = U + 4 * n;
         if constexpr (L2Prefetch<T, K>::mask != 0)
-            prefetch_cell<T, K, 5 * n, 2 * f, 0, MODE != MODE_RAW>(A, c, soff, c.trs_in, c.SS, op.nb_s,
+            prefetch_cell<T, K, 5 * n, 2 * f, 0, MODE != MODE_GRAD>(A, c, soff, c.trs_in, c.SS, op.nb_s,
                                                                 OpData<T>::beta_s(op), rect ? 4 : c.nF);
         {
             T u[n];
@@ -1023,7 +1294,7 @@ __device__ __forceinline__ void solid_cell(const StageArgsT<T>& A, int q, int sh
             add_ddx<T, K>(u, kvy);
         }
         if constexpr (L2Prefetch<T, K>::mask != 0)
-            prefetch_cell<T, K, 5 * n, 2 * f, 1, MODE != MODE_RAW>(A, c, soff, c.trs_in, c.SS, op.nb_s,
+            prefetch_cell<T, K, 5 * n, 2 * f, 1, MODE != MODE_GRAD>(A, c, soff, c.trs_in, c.SS, op.nb_s,
                                                                 OpData<T>::beta_s(op), rect ? 4 : c.nF);
         if (rect) {
             if (kind == KIND_SQUARE) {
@@ -1039,7 +1310,7 @@ __device__ __forceinline__ void solid_cell(const StageArgsT<T>& A, int q, int sh
         }
         // stress rate = C e = c1 [(e_xx + r e_yy), (e_yy + r e_xx)], c3 e_xy; c1, c3 folded into targets
         const T r = __ldg(OpData<T>::scal_s(op) + SS_R * c.N + q);
-        if constexpr (MODE != MODE_RAW) {
+        if constexpr (MODE != MODE_GRAD) {
 #pragma unroll
             for (int i = 0; i < n; ++i) {
                 const T a = exx[i], b = eyy[i];
@@ -1068,10 +1339,8 @@ __device__ __forceinline__ void solid_cell(const StageArgsT<T>& A, int q, int sh
                 kvy[i] = fma(w, g[n + i], kvy[i]);
             }
         }
-        if constexpr (MODE == MODE_RAW) {
-            T* dst = A.tgt[0].dst + soff;
-#pragma unroll
-            for (int i = 0; i < 5 * n; ++i) dst[(size_t)i * c.N + q] = norm(U[i]);
+        if constexpr (MODE == MODE_GRAD) {
+            solid_grad<T, K>(A, *G, c, ci, rect, U);
             return;
         }
         const T sc[3] = {__ldg(OpData<T>::scal_s(op) + SS_C1 * c.N + q), __ldg(OpData<T>::scal_s(op) + SS_C3 * c.N + q), Av};
@@ -1143,6 +1412,22 @@ __global__ void __launch_bounds__(128, MinBlocks<T, K>::value) stage_kernel(cons
         fluid_cell<T, K, MODE>(A, gq, shot, cd, acc);
     else if (gq < A.op.Nf + A.op.Ns)
         solid_cell<T, K, MODE>(A, gq - A.op.Nf, shot, cd, acc);
+}
+
+// One backward stage's gradients (MODE_GRAD): the stage kernel's rate of the
+// forward stage value, taken straight into the gradient sums instead of being
+// stored.
+template <class T, int K>
+__global__ void __launch_bounds__(128, MinBlocks<T, K>::value)
+    grad_stage_kernel(const StageArgsT<T> A, const GradArgsT<T> G) {
+    extern __shared__ __align__(16) unsigned char stage_smem[];
+    const int gq = blockIdx.x * blockDim.x + threadIdx.x;
+    T* acc = nullptr;
+    if constexpr (AccSmem<T, K>::value) acc = reinterpret_cast<T*>(stage_smem) + threadIdx.x * acc_stride<K>();
+    if (gq < A.op.Nf)
+        fluid_cell<T, K, MODE_GRAD>(A, gq, 0, nullptr, acc, &G);
+    else if (gq < A.op.Nf + A.op.Ns)
+        solid_cell<T, K, MODE_GRAD>(A, gq - A.op.Nf, 0, nullptr, acc, &G);
 }
 
 // canonical (AoS, input cell order, FP64) <-> device layout (SoA by class, T);
@@ -1365,32 +1650,42 @@ __global__ void record_kernel(DevOps op, int n_rec, const int32_t* __restrict__ 
     for (int j = 0; j < 5; ++j) ob[j] = TO(o[j]);
 }
 
+// Per function and device: the opt-in above 48 KB of dynamic shared memory
+// (the largest size set is remembered), and the largest carveout where the
+// accumulators live in shared memory, for the resident blocks that the
+// register budget allows.  `Tag` makes one state per kernel.
+template <class Tag, class F>
+void stage_smem_attributes(F* kernel, size_t smem, bool carve) {
+    static size_t opted[64] = {};
+    static bool carved[64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const bool known = dev >= 0 && dev < 64;
+    if (smem > 48 * 1024 && (!known || opted[dev] < smem)) {
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (known) opted[dev] = smem;
+    }
+    if (carve && (!known || !carved[dev])) {
+        cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             (int)cudaSharedmemCarveoutMaxShared);
+        if (known) carved[dev] = true;
+    }
+}
+template <class T, int K, int MODE>
+struct StageTag {};
+
 template <class T, int K, int MODE>
 void launch_kk(const StageArgsT<T>& a, dim3 grid, cudaStream_t s) {
     const size_t smem = stage_smem_bytes<T, K>(a.op.max_nf);
-    if (smem > 48 * 1024) {
-        // the opt-in is per function and device; remember the largest size set
-        static size_t opted[64] = {};
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (dev < 0 || dev >= 64 || opted[dev] < smem) {
-            cudaFuncSetAttribute(stage_kernel<T, K, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (dev >= 0 && dev < 64) opted[dev] = smem;
-        }
-    }
-    if constexpr (AccSmem<T, K>::value) {
-        // the accumulators need the largest shared-memory carveout for the
-        // resident blocks the register budget allows
-        static bool carved[64] = {};
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (dev < 0 || dev >= 64 || !carved[dev]) {
-            cudaFuncSetAttribute(stage_kernel<T, K, MODE>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 (int)cudaSharedmemCarveoutMaxShared);
-            if (dev >= 0 && dev < 64) carved[dev] = true;
-        }
-    }
+    stage_smem_attributes<StageTag<T, K, MODE>>(stage_kernel<T, K, MODE>, smem, AccSmem<T, K>::value);
     stage_kernel<T, K, MODE><<<grid, 128, smem, s>>>(a);
+}
+
+template <class T, int K>
+void launch_grad_k(const StageArgsT<T>& a, const GradArgsT<T>& g, unsigned grid, cudaStream_t s) {
+    const size_t smem = stage_smem_bytes<T, K>(a.op.max_nf);
+    stage_smem_attributes<StageTag<T, K, MODE_GRAD>>(grad_stage_kernel<T, K>, smem, AccSmem<T, K>::value);
+    grad_stage_kernel<T, K><<<grid, 128, smem, s>>>(a, g);
 }
 
 template <class T, int MODE>
@@ -1465,7 +1760,7 @@ int build_plan(const hho_tableau* tab, std::vector<StagePlan>& plan, int* n_buf)
         for (int i = j + 2; i <= s; ++i) {
             const double a = coef(i, j);
             if (a == 0.0) continue;
-            if (P.n_tgt >= MAX_TARGETS) return HHO_EINVAL;
+            if (P.n_tgt >= MAX_PLAN_TARGETS) return HHO_EINVAL;
             if (buf[i] < 0) buf[i] = nb++;
             TargetPlan t;
             t.src = touched[i] ? buf[i] : SRC_STATE;
@@ -1640,7 +1935,7 @@ static int erk_run(hho_ops* ops, const hho_tableau* tab, double t0, double dt, i
     std::vector<StagePlan> plan;
     int nb = 0;
     if (build_plan(tab, plan, &nb) != HHO_OK) {
-        hho_set_error("%s: unsupported tableau (s <= 6, at most %d partial sums per stage)", who, MAX_TARGETS);
+        hho_set_error("%s: unsupported tableau (s <= 6, at most %d partial sums per stage)", who, MAX_PLAN_TARGETS);
         return HHO_EINVAL;
     }
     if (nsteps == 0) return HHO_OK;
@@ -2616,7 +2911,7 @@ void launch_stage_f64(const hho_ops* ops, int mode, StageArgsT<double>& a, int n
         case MODE_TRACES: launch_k<double, MODE_TRACES>(ops->k, a, grid, st); break;
         case MODE_STAGE: launch_k<double, MODE_STAGE>(ops->k, a, grid, st); break;
         case MODE_APPLY: launch_k<double, MODE_APPLY>(ops->k, a, grid, st); break;
-        default: launch_k<double, MODE_RAW>(ops->k, a, grid, st); break;
+        default: break;
     }
 }
 
@@ -2639,8 +2934,30 @@ void launch_stage_f32(const hho_ops* ops, int mode, StageArgsT<float>& a, int n_
         case MODE_TRACES: launch_k<float, MODE_TRACES>(ops->k, a, grid, st); break;
         case MODE_STAGE: launch_k<float, MODE_STAGE>(ops->k, a, grid, st); break;
         case MODE_APPLY: launch_k<float, MODE_APPLY>(ops->k, a, grid, st); break;
-        default: launch_k<float, MODE_RAW>(ops->k, a, grid, st); break;
+        default: break;
     }
+}
+
+template <class T>
+static void launch_grad_t(const hho_ops* ops, StageArgsT<T>& a, const GradArgsT<T>& g, double tn, int j, double cdt,
+                          void* stream) {
+    const unsigned grid = (unsigned)((ops->dev.Nf + ops->dev.Ns + 127) / 128);
+    if (grid == 0) return;
+    a.state_stride = ops->n_state;
+    a.trace_stride = ops->trace_doubles;
+    fill_sources<T>(ops, a, tn, j, cdt, 1);
+    cudaStream_t st = (cudaStream_t)stream;
+    if (ops->k == 1) launch_grad_k<T, 1>(a, g, grid, st);
+    else if (ops->k == 2) launch_grad_k<T, 2>(a, g, grid, st);
+    else launch_grad_k<T, 3>(a, g, grid, st);
+}
+void launch_grad_f64(const hho_ops* ops, StageArgsT<double>& a, const GradArgsT<double>& g, double tn, int j, double cdt,
+                     void* stream) {
+    launch_grad_t<double>(ops, a, g, tn, j, cdt, stream);
+}
+void launch_grad_f32(const hho_ops* ops, StageArgsT<float>& a, const GradArgsT<float>& g, double tn, int j, double cdt,
+                     void* stream) {
+    launch_grad_t<float>(ops, a, g, tn, j, cdt, stream);
 }
 
 int erk_steps_f32(hho_ops* ops, const hho_tableau* tab, double t0, double dt, int64_t nsteps, float* d_state,

@@ -264,3 +264,64 @@ def test_fp32_adjoint_against_fp64(lib):
     et = np.linalg.norm(t32 - t64) / np.linalg.norm(t64)
     print("FP32 adjoint vs FP64: materials %.2e, wavelet %.2e, tau %.2e" % (eg, ew, et))
     assert eg <= 1e-3 and ew <= 1e-3 and et <= 1e-3
+
+
+def _tableau(hho, a, b):
+    """An explicit tableau from the rows below its diagonal and its weights."""
+    t = hho.Tableau()
+    t.s = len(b)
+    for i, row in enumerate(a):
+        for j, v in enumerate(row):
+            t.a[i][j] = v
+        t.c[i] = sum(row)
+    for j, v in enumerate(b):
+        t.b[j] = v
+    return t
+
+
+@pytest.mark.parametrize("name, a, b", [
+    ("one stage", [[]], [1.0]),
+    ("first weight zero", [[], [0.5]], [0.0, 1.0]),
+    ("last weight zero", [[], [0.5], [0.25, 0.25]], [0.5, 0.5, 0.0]),
+    ("small weight", [[], [0.5], [-1.0, 2.0]], [1e-6, 1.0 - 2e-6, 1e-6]),
+    ("last row full", [[], [0.2], [0.0, 0.3], [0.0, 0.0, 0.4], [0.0, 0.0, 0.0, 0.5], [0.1, 0.2, -0.1, 0.3, 0.25]],
+     [0.1, 0.2, 0.1, 0.2, 0.15, 0.25])])
+def test_vjp_of_unusual_tableaux_is_the_derivative(lib, name, a, b):
+    """The backward step is an explicit scheme scaled by the weights b_i, with
+    other scalings where a weight vanishes or is small and up to six targets a
+    stage: for each of these tableaux the wavelet gradient is the derivative
+    of the (linear) map from the wavelet to the traces.  The traces are exactly
+    linear in the samples, so both sides agree to rounding: 1e-11 is a
+    thousand times the FP64 error of the two runs."""
+    hho, _ = lib
+    md = synth.hybrid_grid(6, 6, 0.0, 1.0, 0.0, 1.0, 0.7, 0.5)
+    media = synth.layered_media(md)
+    tab = _tableau(hho, a, b)
+    dt, nsteps, s = 0.002, 7, len(b)
+    rec = [(0.31, 0.72), (0.47, 0.5), (0.83, 0.21)]
+    mesh = hho.hho_mesh_create(md.xy, md.cell_ptr, md.cell_vtx, md.cell_domain)
+    ops = hho.hho_operators_build(mesh, 2, *media)
+    hho.hho_mesh_destroy(mesh)
+    rng = np.random.default_rng(3)
+    hho.hho_receivers_set(ops, rec)
+    lay = hho.hho_state_layout(ops)
+    G = torch.as_tensor(rng.standard_normal((nsteps, len(rec), 5))).cuda()
+    dw = rng.standard_normal((1, nsteps, s))
+    work = torch.empty(hho.hho_work_size(ops, tab), dtype=torch.float64, device="cuda")
+    out = []
+    for w in (dw, np.zeros_like(dw)):
+        hho.hho_sources_set_samples(ops, [(0.41, 0.23)], [(0.6, 0.8)], 0.0, dt, w)
+        x = torch.zeros(lay.n_state, dtype=torch.float64, device="cuda")
+        seis = torch.zeros((nsteps, len(rec), 5), dtype=torch.float64, device="cuda")
+        hho.hho_erk_step_record(ops, tab, 0.0, dt, nsteps, x.data_ptr(), work.data_ptr(), seis.data_ptr())
+        out.append(float((seis * G).sum()))
+    x0 = torch.zeros(lay.n_state, dtype=torch.float64, device="cuda")
+    for every in (3, 7):
+        nw = hho.hho_adjoint_work_size(ops, tab, nsteps, every)
+        aw = torch.empty(nw, dtype=torch.float64, device="cuda")
+        _, gw = hho.hho_adjoint_vjp(ops, tab, 0.0, dt, nsteps, every, x0.data_ptr(), G.data_ptr(), aw.data_ptr(), nw,
+                                    md.n_cells, n_src=1)
+        got = float((gw[:, :, 0] * dw[0]).sum())
+        scale = float(np.abs(gw[:, :, 0] * dw[0]).sum())
+        assert abs(got - (out[0] - out[1])) <= 1e-11 * scale, (name, every, got, out)
+    hho.hho_ops_destroy(ops)
