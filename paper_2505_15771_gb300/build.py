@@ -15,7 +15,10 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(ROOT, "_build")
 LIB = os.path.join(HERE, "libhho.so")
 PROBE_LIB = os.path.join(HERE, "libhho_probe.so")
-SOURCES = ["mesh.cpp", "operators.cpp", "stage.cu", "adjoint.cu", "sdirk.cu", "tc.cu", "f2x_check.cu", "probe.cu"]
+# the translation units that stage_tuning.h reaches
+STAGE_SOURCES = ["stage_f64.cu", "stage_f32.cu", "stage_f2x.cu", "stage_tc.cu"]
+SOURCES = STAGE_SOURCES + ["mesh.cpp", "operators.cpp", "stage.cu", "adjoint.cu", "sdirk.cu", "tc.cu", "f2x_check.cu",
+                           "probe.cu"]
 
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
@@ -54,10 +57,10 @@ def build(verbose=False):
 
 
 def build_stage_variant(tuning_header: str, out_dir: str) -> str:
-    """Builds <out_dir>/libhho.so with stage.cu compiled against the given
-    stage_tuning.h text (a candidate of tune.py) and the other translation
-    units taken from the in-tree build, which must exist."""
-    objs = [os.path.join(OBJ, s + ".o") for s in SOURCES if s not in ("stage.cu", "probe.cu")]
+    """Builds <out_dir>/libhho.so with the stage kernels compiled against the
+    given stage_tuning.h text (a candidate of tune.py) and the other
+    translation units taken from the in-tree build, which must exist."""
+    objs = [os.path.join(OBJ, s + ".o") for s in SOURCES if s not in STAGE_SOURCES + ["probe.cu"]]
     missing = [o for o in objs if not os.path.exists(o)]
     if missing:
         raise RuntimeError("in-tree objects missing (%s); run build() first" % ", ".join(missing))
@@ -69,14 +72,15 @@ def build_stage_variant(tuning_header: str, out_dir: str) -> str:
                 b.write(a.read())
     with open(os.path.join(src, "stage_tuning.h"), "w") as f:
         f.write(tuning_header)
-    obj = os.path.join(out_dir, "stage.cu.o")
     flags = [x for x in FLAGS if x != "-I" + CSRC] + ["-I" + src]
-    r = subprocess.run([NVCC] + ARCH + flags + ["-c", os.path.join(src, "stage.cu"), "-o", obj],
-                       capture_output=True, text=True)
-    if r.returncode != 0:
-        raise RuntimeError("nvcc failed for the stage variant in %s:\n%s" % (out_dir, r.stderr))
+    mine = [os.path.join(out_dir, s + ".o") for s in STAGE_SOURCES]
+    jobs = [subprocess.Popen([NVCC] + ARCH + flags + ["-c", os.path.join(src, s), "-o", o], stdout=subprocess.PIPE,
+                             stderr=subprocess.STDOUT, text=True) for s, o in zip(STAGE_SOURCES, mine)]
+    logs = [j.communicate()[0] for j in jobs]
+    if any(j.returncode != 0 for j in jobs):
+        raise RuntimeError("nvcc failed for the stage variant in %s:\n%s" % (out_dir, "\n".join(logs)))
     lib = os.path.join(out_dir, "libhho.so")
-    r = subprocess.run([NVCC] + ARCH + ["-shared", "-o", lib, obj] + objs, capture_output=True, text=True)
+    r = subprocess.run([NVCC] + ARCH + ["-shared", "-o", lib] + mine + objs, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError("link failed for the stage variant in %s:\n%s" % (out_dir, r.stderr))
     return lib

@@ -1,6 +1,6 @@
 // Batched FP32 stage with its dense local products on the tcgen05 tensor
-// cores in split BF16 (HHO_BF16X3).  Included by stage.cu (uses its cell
-// helpers, in its anonymous namespace).
+// cores in split BF16 (HHO_BF16X3).  Included by stage_tc.cu after
+// stage_kernels.cuh, whose cell helpers it uses.
 //
 // A block is 128 (cell, shot) rows: C = 32 consecutive cells of one class
 // (class runs are padded to 32 cells, so they share a class and a domain)
