@@ -110,6 +110,63 @@ __device__ __forceinline__ f2x __ldg(const f2x* p) {
 // Renormalised pair (hi = RN(hi + lo)), applied where a value is stored.
 __device__ __forceinline__ f2x norm(f2x x) { return f2x_fast_two_sum(x.hi, x.lo); }
 
+// ---- conversions off the FP64 pipe -----------------------------------------------
+// GB300 converts between FP32 and FP64 on its FP64 unit (two lanes a clock per
+// SM), so a split into a pair (three conversions and a subtraction) cost more
+// than the memory traffic of the arrays it converts: 92 us for the 12.6 M values
+// of the 1024 x 512, k = 2 bilayer state, whose 200 MB take 30 us.  These
+// forms work on the bit patterns in the integer pipes; results are those of
+// the plain conversions, bit for bit.  Zeros, infinities, NaNs and the ends of the
+// exponent range take the plain conversion.
+
+// (double)x
+__device__ __forceinline__ double f32_to_f64(float x) {
+    const uint32_t u = __float_as_uint(x), m = u & 0x7fffffffu;
+    if (m - 0x00800000u >= 0x7f000000u) {   // zero, subnormal, infinity or NaN
+        if (m == 0u) return __hiloint2double((int)u, 0);
+        return (double)x;
+    }
+    return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+}
+
+// f2x(v): hi = RN(v), lo = RN(v - hi)
+__device__ __forceinline__ f2x f64_to_pair(double v) {
+    const uint32_t h = (uint32_t)__double2hiint(v), l = (uint32_t)__double2loint(v);
+    const uint32_t e = (h >> 20) & 0x7ffu;   // biased exponent; plain path outside 2^-70 .. 2^126
+    if (e - 953u > 196u) {
+        if (((h << 1) | l) == 0u) return f2x(__uint_as_float(h), 0.0f);
+        return f2x(v);
+    }
+    // 23 leading mantissa bits, and 29 trailing ones as a signed remainder in (-2^28, 2^28]
+    uint32_t q = ((h & 0x000fffffu) << 3) | (l >> 29);
+    int32_t r = (int32_t)(l & 0x1fffffffu);
+    if (r > 0x10000000 || (r == 0x10000000 && (q & 1u))) {   // round half to even
+        ++q;                                                  // a carry out of the mantissa raises the exponent
+        r -= 0x20000000;
+    }
+    const uint32_t sign = h & 0x80000000u;
+    const float hi = __uint_as_float(sign | (((e - 896u) << 23) + q));
+    // v - hi = +-r 2^(e - 1023 - 52): r rounds once, the scaling is exact (no subnormal results here)
+    const float scale = __uint_as_float(sign | ((e - 948u) << 23));
+    return f2x(hi, __fadd_rn(__fmul_rn(__int2float_rn(r), scale), 0.0f));   // + 0: never -0, as RN(v - hi)
+}
+__device__ __forceinline__ float f64_to_f32(double v) { return f64_to_pair(v).hi; }
+
+// double(x): one FP64 addition left of two conversions and one
+__device__ __forceinline__ double pair_to_f64(f2x x) { return f32_to_f64(x.hi) + f32_to_f64(x.lo); }
+
+template <class T>
+__device__ __forceinline__ T from_f64(double v);
+template <>
+__device__ __forceinline__ double from_f64<double>(double v) { return v; }
+template <>
+__device__ __forceinline__ float from_f64<float>(double v) { return f64_to_f32(v); }
+template <>
+__device__ __forceinline__ f2x from_f64<f2x>(double v) { return f64_to_pair(v); }
+__device__ __forceinline__ double to_f64(double v) { return v; }
+__device__ __forceinline__ double to_f64(float v) { return f32_to_f64(v); }
+__device__ __forceinline__ double to_f64(f2x v) { return pair_to_f64(v); }
+
 // Scalar helpers shared by the FP64, FP32 and double-float instantiations.
 __device__ __forceinline__ double norm(double x) { return x; }
 __device__ __forceinline__ float norm(float x) { return x; }

@@ -19,40 +19,89 @@ namespace {
 
 // canonical (AoS, input cell order, FP64) <-> device layout (SoA by class, T);
 // y = shot: canonical shot stride n_canon, state shot stride n_state.
-template <class T>
-__global__ void pack_kernel(const int32_t* __restrict__ dev2orig, const int64_t* __restrict__ canon_off, int Nf,
-                            int Ns, int n, int64_t n_canon, int64_t n_state, const double* __restrict__ canon,
-                            T* __restrict__ state) {
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= Nf + Ns) return;
-    const bool fl = g < Nf;
-    const int q = fl ? g : g - Nf;
-    const int N = fl ? Nf : Ns;
-    const int nv = (fl ? 3 : 5) * n;
-    T* st = state + (size_t)blockIdx.y * n_state + (fl ? 0 : (size_t)3 * n * Nf);
-    const int c = dev2orig[g];
-    if (c < 0) {
-        for (int i = 0; i < nv; ++i) st[(size_t)i * N + q] = T(0);
-        return;
+// A block of 128 threads moves 32 consecutive device slots (a class run is
+// padded to 32, so one domain) through shared memory: the device side in
+// 32-element rows, the canonical side in the cells' own runs, which are
+// adjacent where the class's cells are.  Bound by memory; one thread a cell
+// walking its run took 152 us to unpack the 1024 x 512, k = 2 state (200 MB) and
+// 2265 us for 16 FP32 shots of the 680 x 340, k = 3 hybrid mesh (2.2 GB).
+constexpr int PACK_THREADS = 128;
+template <class T, int NV, bool PACK>
+__device__ __forceinline__ void pack_block(const int32_t* __restrict__ dev2orig, const int64_t* __restrict__ canon_off,
+                                           int N, int q0, typename std::conditional<PACK, const double, double>::type* canon,
+                                           typename std::conditional<PACK, T, const T>::type* st, T* run) {
+    constexpr int LD = NV | 1;   // odd stride: a column of the tile has no bank conflicts
+    __shared__ int64_t off[32];
+    if (threadIdx.x < 32) {
+        const int c = dev2orig[threadIdx.x];
+        off[threadIdx.x] = c < 0 ? -1 : canon_off[c];
     }
-    const double* cv = canon + (size_t)blockIdx.y * n_canon + canon_off[c];
-    for (int i = 0; i < nv; ++i) st[(size_t)i * N + q] = T(cv[i]);
+    const int lane = threadIdx.x & 31, row0 = threadIdx.x >> 5;
+    if constexpr (!PACK) {
+#pragma unroll 8
+        for (int i = row0; i < NV; i += PACK_THREADS / 32) run[lane * LD + i] = st[(size_t)i * N + q0 + lane];
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int e = threadIdx.x; e < 32 * NV; e += PACK_THREADS) {
+        const int cell = e / NV, i = e - cell * NV;
+        const int64_t o = off[cell];
+        if constexpr (PACK) run[cell * LD + i] = o < 0 ? T(0) : from_f64<T>(canon[o + i]);
+        else if (o >= 0) canon[o + i] = to_f64(run[cell * LD + i]);
+    }
+    if constexpr (PACK) {
+        __syncthreads();
+#pragma unroll 8
+        for (int i = row0; i < NV; i += PACK_THREADS / 32) st[(size_t)i * N + q0 + lane] = run[lane * LD + i];
+    }
+}
+template <class T, int K>
+__global__ void __launch_bounds__(PACK_THREADS)
+    pack_kernel(const int32_t* __restrict__ dev2orig, const int64_t* __restrict__ canon_off, int Nf, int Ns,
+                int64_t n_canon, int64_t n_state, const double* __restrict__ canon, T* __restrict__ state) {
+    constexpr int n = (K + 1) * (K + 2) / 2;
+    __shared__ T run[32 * ((5 * n) | 1)];
+    const int g = blockIdx.x * 32;
+    const double* cv = canon + (size_t)blockIdx.y * n_canon;
+    T* st = state + (size_t)blockIdx.y * n_state;
+    if (g < Nf) pack_block<T, 3 * n, true>(dev2orig + g, canon_off, Nf, g, cv, st, run);
+    else pack_block<T, 5 * n, true>(dev2orig + g, canon_off, Ns, g - Nf, cv, st + (size_t)3 * n * Nf, run);
+}
+template <class T, int K>
+__global__ void __launch_bounds__(PACK_THREADS)
+    unpack_kernel(const int32_t* __restrict__ dev2orig, const int64_t* __restrict__ canon_off, int Nf, int Ns,
+                  int64_t n_canon, int64_t n_state, const T* __restrict__ state, double* __restrict__ canon) {
+    constexpr int n = (K + 1) * (K + 2) / 2;
+    __shared__ T run[32 * ((5 * n) | 1)];
+    const int g = blockIdx.x * 32;
+    double* cv = canon + (size_t)blockIdx.y * n_canon;
+    const T* st = state + (size_t)blockIdx.y * n_state;
+    if (g < Nf) pack_block<T, 3 * n, false>(dev2orig + g, canon_off, Nf, g, cv, st, run);
+    else pack_block<T, 5 * n, false>(dev2orig + g, canon_off, Ns, g - Nf, cv, st + (size_t)3 * n * Nf, run);
+}
+template <class T, int K>
+void launch_pack(const hho_ops* ops, int n_shots, const double* canon, T* state, cudaStream_t st) {
+    const dim3 grid((ops->dev.Nf + ops->dev.Ns) / 32, n_shots);
+    pack_kernel<T, K><<<grid, PACK_THREADS, 0, st>>>(ops->d_dev2orig, ops->d_canon_off, ops->dev.Nf, ops->dev.Ns,
+                                                     ops->n_canonical, ops->n_state, canon, state);
+}
+template <class T, int K>
+void launch_unpack(const hho_ops* ops, int n_shots, const T* state, double* canon, cudaStream_t st) {
+    const dim3 grid((ops->dev.Nf + ops->dev.Ns) / 32, n_shots);
+    unpack_kernel<T, K><<<grid, PACK_THREADS, 0, st>>>(ops->d_dev2orig, ops->d_canon_off, ops->dev.Nf, ops->dev.Ns,
+                                                       ops->n_canonical, ops->n_state, state, canon);
 }
 template <class T>
-__global__ void unpack_kernel(const int32_t* __restrict__ dev2orig, const int64_t* __restrict__ canon_off, int Nf,
-                              int Ns, int n, int64_t n_canon, int64_t n_state, const T* __restrict__ state,
-                              double* __restrict__ canon) {
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= Nf + Ns) return;
-    const bool fl = g < Nf;
-    const int q = fl ? g : g - Nf;
-    const int N = fl ? Nf : Ns;
-    const int nv = (fl ? 3 : 5) * n;
-    const T* st = state + (size_t)blockIdx.y * n_state + (fl ? 0 : (size_t)3 * n * Nf);
-    const int c = dev2orig[g];
-    if (c < 0) return;
-    double* cv = canon + (size_t)blockIdx.y * n_canon + canon_off[c];
-    for (int i = 0; i < nv; ++i) cv[i] = double(st[(size_t)i * N + q]);
+void launch_pack(const hho_ops* ops, int n_shots, const double* canon, void* state, cudaStream_t st) {
+    if (ops->k == 1) launch_pack<T, 1>(ops, n_shots, canon, (T*)state, st);
+    else if (ops->k == 2) launch_pack<T, 2>(ops, n_shots, canon, (T*)state, st);
+    else launch_pack<T, 3>(ops, n_shots, canon, (T*)state, st);
+}
+template <class T>
+void launch_unpack(const hho_ops* ops, int n_shots, const void* state, double* canon, cudaStream_t st) {
+    if (ops->k == 1) launch_unpack<T, 1>(ops, n_shots, (const T*)state, canon, st);
+    else if (ops->k == 2) launch_unpack<T, 2>(ops, n_shots, (const T*)state, canon, st);
+    else launch_unpack<T, 3>(ops, n_shots, (const T*)state, canon, st);
 }
 
 // Canonical vector in host memory (pinned, mapped into the device's address
@@ -97,7 +146,7 @@ __global__ void __launch_bounds__(STAGED_CELLS) pack_host_kernel(const int32_t* 
     T* st = state + (fl ? 0 : (size_t)3 * n * Nf);
     const double* v = run + (canon_off[c] - e0);
     const int nv = (fl ? 3 : 5) * n;
-    for (int i = 0; i < nv; ++i) st[(size_t)i * N + q] = T(v[i]);
+    for (int i = 0; i < nv; ++i) st[(size_t)i * N + q] = from_f64<T>(v[i]);
 }
 template <class T>
 __global__ void __launch_bounds__(STAGED_CELLS) unpack_host_kernel(const int32_t* __restrict__ cell_dom,
@@ -119,7 +168,7 @@ __global__ void __launch_bounds__(STAGED_CELLS) unpack_host_kernel(const int32_t
         const T* st = state + (fl ? 0 : (size_t)3 * n * Nf);
         double* v = run + (canon_off[c] - e0);
         const int nv = (fl ? 3 : 5) * n;
-        for (int i = 0; i < nv; ++i) v[i] = double(st[(size_t)i * N + q]);
+        for (int i = 0; i < nv; ++i) v[i] = to_f64(st[(size_t)i * N + q]);
     }
     __syncthreads();
     for (int e = threadIdx.x; e < len; e += STAGED_CELLS) canon[e0 + e] = run[e];
@@ -617,11 +666,11 @@ static int64_t work_f64_part(const hho_ops* ops, int nb) {
 namespace {
 __global__ void to_pairs_kernel(const double* __restrict__ x, f2x* __restrict__ y, int64_t n) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        y[i] = f2x(x[i]);
+        y[i] = f64_to_pair(x[i]);
 }
 __global__ void from_pairs_kernel(const f2x* __restrict__ x, double* __restrict__ y, int64_t n) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        y[i] = double(x[i]);
+        y[i] = pair_to_f64(x[i]);
 }
 int pairs_grid(int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, 152 * 16); }
 }  // namespace
@@ -924,19 +973,11 @@ extern "C" int hho_batch_pack(const hho_ops* ops, int32_t n_shots, int32_t preci
         if (ops) hho_set_error("hho_batch_pack: bad arguments");
         return HHO_EINVAL;
     }
-    const int tot = ops->dev.Nf + ops->dev.Ns;
-    if (tot == 0) return HHO_OK;
-    const dim3 grid((tot + 127) / 128, n_shots);
+    if (ops->dev.Nf + ops->dev.Ns == 0) return HHO_OK;
     cudaStream_t st = (cudaStream_t)stream;
-    if (precision == HHO_F64)
-        pack_kernel<double><<<grid, 128, 0, st>>>(ops->d_dev2orig, ops->d_canon_off, ops->dev.Nf, ops->dev.Ns, ops->n,
-                                                  ops->n_canonical, ops->n_state, d_canonical, (double*)d_state);
-    else if (precision == HHO_F32X2)
-        pack_kernel<f2x><<<grid, 128, 0, st>>>(ops->d_dev2orig, ops->d_canon_off, ops->dev.Nf, ops->dev.Ns, ops->n,
-                                               ops->n_canonical, ops->n_state, d_canonical, (f2x*)d_state);
-    else
-        pack_kernel<float><<<grid, 128, 0, st>>>(ops->d_dev2orig, ops->d_canon_off, ops->dev.Nf, ops->dev.Ns, ops->n,
-                                                 ops->n_canonical, ops->n_state, d_canonical, (float*)d_state);
+    if (precision == HHO_F64) launch_pack<double>(ops, n_shots, d_canonical, d_state, st);
+    else if (precision == HHO_F32X2) launch_pack<f2x>(ops, n_shots, d_canonical, d_state, st);
+    else launch_pack<float>(ops, n_shots, d_canonical, d_state, st);
     return check_launch("hho_batch_pack");
 }
 
@@ -946,19 +987,11 @@ extern "C" int hho_batch_unpack(const hho_ops* ops, int32_t n_shots, int32_t pre
         if (ops) hho_set_error("hho_batch_unpack: bad arguments");
         return HHO_EINVAL;
     }
-    const int tot = ops->dev.Nf + ops->dev.Ns;
-    if (tot == 0) return HHO_OK;
-    const dim3 grid((tot + 127) / 128, n_shots);
+    if (ops->dev.Nf + ops->dev.Ns == 0) return HHO_OK;
     cudaStream_t st = (cudaStream_t)stream;
-    if (precision == HHO_F64)
-        unpack_kernel<double><<<grid, 128, 0, st>>>(ops->d_dev2orig, ops->d_canon_off, ops->dev.Nf, ops->dev.Ns, ops->n,
-                                                    ops->n_canonical, ops->n_state, (const double*)d_state, d_canonical);
-    else if (precision == HHO_F32X2)
-        unpack_kernel<f2x><<<grid, 128, 0, st>>>(ops->d_dev2orig, ops->d_canon_off, ops->dev.Nf, ops->dev.Ns, ops->n,
-                                                 ops->n_canonical, ops->n_state, (const f2x*)d_state, d_canonical);
-    else
-        unpack_kernel<float><<<grid, 128, 0, st>>>(ops->d_dev2orig, ops->d_canon_off, ops->dev.Nf, ops->dev.Ns, ops->n,
-                                                   ops->n_canonical, ops->n_state, (const float*)d_state, d_canonical);
+    if (precision == HHO_F64) launch_unpack<double>(ops, n_shots, d_state, d_canonical, st);
+    else if (precision == HHO_F32X2) launch_unpack<f2x>(ops, n_shots, d_state, d_canonical, st);
+    else launch_unpack<float>(ops, n_shots, d_state, d_canonical, st);
     return check_launch("hho_batch_unpack");
 }
 
