@@ -167,10 +167,24 @@ __device__ __forceinline__ double to_f64(double v) { return v; }
 __device__ __forceinline__ double to_f64(float v) { return f32_to_f64(v); }
 __device__ __forceinline__ double to_f64(f2x v) { return pair_to_f64(v); }
 
+// Comparisons of class-matrix entries (FP64 ones on the bits: a DSETP would
+// take an FP64 slot).
+__device__ __forceinline__ bool is_zero(double x) { return (__double_as_longlong(x) << 1) == 0; }
+__device__ __forceinline__ bool is_zero(float x) { return x == 0.0f; }
+__device__ __forceinline__ bool is_zero(f2x x) { return x.hi == 0.0f; }
+__device__ __forceinline__ bool is_negative(double x) { return __double2hiint(x) < 0; }
+__device__ __forceinline__ bool is_negative(float x) { return x < 0.0f; }
+__device__ __forceinline__ bool is_negative(f2x x) { return x.hi < 0.0f; }
+
 // Scalar helpers shared by the FP64, FP32 and double-float instantiations.
 __device__ __forceinline__ double norm(double x) { return x; }
 __device__ __forceinline__ float norm(float x) { return x; }
-__device__ __forceinline__ double mulc(float c, double x) { return (double)c * x; }
-__device__ __forceinline__ float mulc(float c, float x) { return c * x; }
+// A product that stays rounded: contracted into a following addition (or not)
+// it would depend on the code around it.
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ f2x mul_rn(f2x a, f2x b) { return a * b; }
+__device__ __forceinline__ double mulc(float c, double x) { return mul_rn((double)c, x); }
+__device__ __forceinline__ float mulc(float c, float x) { return mul_rn(c, x); }
 __device__ __forceinline__ double fmac(float c, double x, double z) { return fma((double)c, x, z); }
 __device__ __forceinline__ float fmac(float c, float x, float z) { return fmaf(c, x, z); }

@@ -55,7 +55,9 @@ struct hho_mesh {
 };
 
 // Per-class integer record on the device (stride CI_STRIDE ints).
-enum { CI_DOMAIN = 0, CI_NF, CI_START, CI_COUNT, CI_NPAD, CI_SLOT, CI_DOFF, CI_KIND, CI_STRIDE };
+// CI_HOR, CI_VER: bit j set where local face j < 32 is horizontal (n_x = 0) or
+// vertical (n_y = 0).
+enum { CI_DOMAIN = 0, CI_NF, CI_START, CI_COUNT, CI_NPAD, CI_SLOT, CI_DOFF, CI_KIND, CI_HOR, CI_VER, CI_STRIDE };
 
 // Class kinds: generic polygon (dense class matrices) or axis-aligned
 // rectangle with faces ordered bottom, right, top, left, whose trace and
@@ -75,6 +77,7 @@ struct DevOps {
     int32_t SF, SS;          // face-side slots per domain
     int32_t n_warps_f, n_warps_s;
     int32_t max_nf;              // most faces of any class
+    int32_t n_warps_rect;        // warps whose class is a rectangle
     const int32_t* warp_class;   // [n_warps_f + n_warps_s]
     const int32_t* cls_int;      // [n_classes][CI_STRIDE]
     const double* cls_dbl;       // class matrices, see operators.cpp

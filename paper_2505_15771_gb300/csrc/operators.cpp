@@ -720,6 +720,10 @@ extern "C" int hho_operators_build_tau(const hho_mesh* m, int32_t k, const doubl
         r[CI_SLOT] = cls_slot[cl];
         r[CI_DOFF] = cls_doff[cl];
         r[CI_KIND] = cls_kind[cl];
+        for (int j = 0; j < std::min(cls_nf[cl], 32); ++j) {
+            if (ops->class_normals[cl][2 * j] == 0.0) r[CI_HOR] |= (int32_t)(1u << j);
+            if (ops->class_normals[cl][2 * j + 1] == 0.0) r[CI_VER] |= (int32_t)(1u << j);
+        }
     }
 
     // ---- per-cell scalars ----------------------------------------------------------
@@ -874,6 +878,9 @@ extern "C" int hho_operators_build_tau(const hho_mesh* m, int32_t k, const doubl
         std::vector<StageClock> clk(1, StageClock{0.0, 0});
         ops->d_clock = dev_upload(ops, clk, &err);
     }
+    D.n_warps_rect = 0;
+    for (int32_t w : warp_class)
+        if (cls_kind[w] != KIND_GENERIC) ++D.n_warps_rect;
     D.max_nf = 0;
     for (int32_t cl = 0; cl < (int32_t)(cls_int.size() / CI_STRIDE); ++cl)
         D.max_nf = std::max(D.max_nf, cls_int[(size_t)cl * CI_STRIDE + CI_NF]);

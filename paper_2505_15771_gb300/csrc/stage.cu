@@ -287,16 +287,16 @@ __global__ void record_kernel(DevOps op, int n_rec, const int32_t* __restrict__ 
 }
 
 template <class T, int MODE>
-void launch_k(int k, const StageArgsT<T>& a, dim3 grid, cudaStream_t s) {
-    if (k == 1) hho_stage::launch_stage<T, 1, MODE>(a, grid, s);
-    else if (k == 2) hho_stage::launch_stage<T, 2, MODE>(a, grid, s);
-    else hho_stage::launch_stage<T, 3, MODE>(a, grid, s);
+void launch_k(int k, const StageArgsT<T>& a, int n_shots, cudaStream_t s) {
+    if (k == 1) hho_stage::launch_stage<T, 1, MODE>(a, n_shots, s);
+    else if (k == 2) hho_stage::launch_stage<T, 2, MODE>(a, n_shots, s);
+    else hho_stage::launch_stage<T, 3, MODE>(a, n_shots, s);
 }
 
 // A stage launch of erk_run: the tensor-core stage when the batched call
 // asked for HHO_BF16X3, else the stage kernel of the arithmetic.
 template <class T, int MODE>
-void launch_stage(const hho_ops* ops, const StageArgsT<T>& a, dim3 grid, int n_shots, cudaStream_t s) {
+void launch_stage(const hho_ops* ops, const StageArgsT<T>& a, int n_shots, cudaStream_t s) {
     if constexpr (std::is_same<T, float>::value) {
         if (ops->tc_on) {
             if (ops->k == 1) hho_stage::launch_tc<1, MODE>(ops, a, n_shots, s);
@@ -305,7 +305,7 @@ void launch_stage(const hho_ops* ops, const StageArgsT<T>& a, dim3 grid, int n_s
             return;
         }
     }
-    launch_k<T, MODE>(ops->k, a, grid, s);
+    launch_k<T, MODE>(ops->k, a, n_shots, s);
 }
 
 }  // namespace
@@ -535,7 +535,7 @@ static int erk_run(hho_ops* ops, const hho_tableau* tab, double t0, double dt, i
         !ops->prof_on && ops->d_clock && !ops->src_sampled &&
         (ops->launch_mode == HHO_LAUNCH_GRAPH ||
          (ops->launch_mode == HHO_LAUNCH_AUTO && (int64_t)grid.x * n_shots <= 2048 && nsteps >= 8));
-    launch_stage<T, MODE_TRACES>(ops, a, grid, n_shots, st);
+    launch_stage<T, MODE_TRACES>(ops, a, n_shots, st);
     int rc = check_launch(who);
     if (rc) return rc;
     int cur = 0;
@@ -595,7 +595,7 @@ static int erk_run(hho_ops* ops, const hho_tableau* tab, double t0, double dt, i
                     hho_set_error("%s: stream capture failed to start", who);
                     return HHO_ECUDA;
                 }
-                for (int j = 0; j < tab->s; ++j) launch_stage<T, MODE_STAGE>(ops, args[j], grid, n_shots, cs);
+                for (int j = 0; j < tab->s; ++j) launch_stage<T, MODE_STAGE>(ops, args[j], n_shots, cs);
                 if (rec)
                     record_kernel<T, TS><<<rgrid, 64, 0, cs>>>(ops->dev, ops->n_rec, ops->d_rec_int, ops->d_rec_dbl,
                                                              d_state, ops->n_state, d_seis, ops->d_clock);
@@ -640,7 +640,7 @@ static int erk_run(hho_ops* ops, const hho_tableau* tab, double t0, double dt, i
             fill_sources<T>(ops, a, tn, j, tab->c[j] * dt, n_shots);
             const bool prof = ops->prof_on && 2 * ops->prof_n + 1 < (int)ops->prof_events.size();
             if (prof) cudaEventRecord((cudaEvent_t)ops->prof_events[2 * ops->prof_n], st);
-            launch_stage<T, MODE_STAGE>(ops, a, grid, n_shots, st);
+            launch_stage<T, MODE_STAGE>(ops, a, n_shots, st);
             if (prof) cudaEventRecord((cudaEvent_t)ops->prof_events[2 * ops->prof_n++ + 1], st);
             rc = check_launch(who);
             if (rc) return rc;
@@ -837,7 +837,7 @@ extern "C" int hho_erk_traces(hho_ops* ops, const hho_tableau* tab, const double
     a.trace_stride = ops->trace_doubles;
     a.inp = d_state;
     a.tr_out = d_work + ops->n_state * (1 + nb);
-    launch_k<double, MODE_TRACES>(ops->k, a, grid, (cudaStream_t)stream);
+    launch_k<double, MODE_TRACES>(ops->k, a, 1, (cudaStream_t)stream);
     return check_launch("hho_erk_traces");
 }
 
@@ -880,7 +880,7 @@ extern "C" int hho_erk_stage(hho_ops* ops, const hho_tableau* tab, int64_t n, in
         a.tgt[t].coef = P.t[t].a * dt;
     }
     fill_sources<double>(ops, a, tn, j, tab->c[j] * dt, 1);
-    launch_k<double, MODE_STAGE>(ops->k, a, grid, (cudaStream_t)stream);
+    launch_k<double, MODE_STAGE>(ops->k, a, 1, (cudaStream_t)stream);
     return check_launch("hho_erk_stage");
 }
 
@@ -1088,16 +1088,18 @@ extern "C" int hho_stage_cost(const hho_ops* ops, const hho_tableau* tab, int64_
     }
     const int K = ops->k, n = ops->n, f = ops->f;
     const int64_t dsm = (int64_t)K * (K - 1) / 2, dvalid = (int64_t)K * (K + 1) / 2;
-    // entries of the rectangle parity patterns (the same count on every face);
-    // a square's trace takes K(K+1)/2 multiply-adds (trace_square)
-    int64_t rect_tr = 0, rect_lift = 0, square_lift = 0;
-    const int64_t square_tr = (int64_t)K * (K + 1) / 2;
+    // entries of the rectangle parity patterns (the same count on every face),
+    // of an axis-aligned face's trace, and of a general face; a square's trace
+    // takes K(K+1)/2 multiply-adds (trace_square)
+    int64_t rect_tr = 0, rect_lift = 0, square_lift = 0, axis_tr = 0;
+    const int64_t square_tr = (int64_t)K * (K + 1) / 2, full = (int64_t)f * n;
     for (int i = 0; i < n; ++i) {
         const int e = ea(i);
         for (int l = 0; l < f; ++l) {
             rect_tr += (e == l);
             rect_lift += (((e + l) % 2) == 0);
             square_lift += (((e + l) % 2) == 0) && e - l != 2;
+            axis_tr += e >= l;
         }
     }
     int64_t ops_total = 0, bytes_k = 0, dofs = 0;
@@ -1107,21 +1109,24 @@ extern "C" int hho_stage_cost(const hho_ops* ops, const hho_tableau* tab, int64_
         const int npad = ci[CI_NPAD], sbase = ci[CI_SLOT];
         const bool rect = ci[CI_KIND] != KIND_GENERIC;
         const int nv = (dom ? 5 : 3) * n, pc = dom ? 2 : 1;   // state values, primal components
-        const int64_t nnzT = ci[CI_KIND] == KIND_SQUARE ? square_tr : rect ? rect_tr : (int64_t)f * n;
-        const int64_t nnzL = ci[CI_KIND] == KIND_SQUARE ? square_lift : rect ? rect_lift : (int64_t)f * n;
+        const int64_t nnzT = ci[CI_KIND] == KIND_SQUARE ? square_tr : rect_tr;
+        const int64_t nnzL = ci[CI_KIND] == KIND_SQUARE ? square_lift : rect_lift;
+        const uint32_t axis = (uint32_t)(ci[CI_HOR] | ci[CI_VER]);
         dofs += (int64_t)count * nv;
         for (int r = 0; r < count; ++r) {
             int64_t rate = dom ? 5 * dsm + 3 * dvalid + 2 * n : 3 * dsm + dvalid;   // derivatives (+ stress mix)
+            if (rect) rate += pc * n;                                               // tau, once per cell
             int64_t traces = 0, bytes_faces = 0;
             for (int j = 0; j < nF; ++j) {
                 const int32_t nb = (dom ? ops->h_nb_s : ops->h_nb_f)[sbase + j * npad + r];
                 const bool bnd = nb == NB_BOUNDARY, ifc = nb < NB_BOUNDARY;
+                const bool ax = j < 32 && ((axis >> j) & 1);
                 rate += bnd ? 0 : (ifc && !dom ? 3 * f : pc * f);                  // jump
-                // lift and the normal / tau combinations; rectangles lift each mirror
-                // pair of faces at once (lift_pair: 4f + 2 nnz(L) per pair and component)
-                rate += rect ? pc * (nnzL + 2 * f) : pc * nnzL + (dom ? 6 * n : 3 * n);
-                traces += dom ? (rect ? 4 * nnzT : 4 * n + 4 * nnzT) + 2 * f + (ifc ? 4 * f : 2 * f)
-                              : (rect ? 2 * nnzT : 2 * n + 2 * nnzT) + 2 * f;
+                // lift and the normal / tau combinations; rectangles lift each mirror pair of
+                // faces at once (lift_pair: 2f + 2 nnz(L) per pair and component)
+                rate += rect ? pc * (nnzL + f) : pc * full + (dom ? (ax ? 4 * n : 6 * n) : (ax ? 2 * n : 3 * n));
+                traces += rect ? 2 * pc * nnzT : ax ? 2 * pc * axis_tr : dom ? 5 * full + 4 * f : 3 * full + 2 * f;
+                traces += dom ? 2 * f + (ifc ? 4 * f : 2 * f) : 2 * f;
                 bytes_faces += 8 * (int64_t)pc * f * (1 + (bnd ? 0 : 1) + 2) + 4 + 8;
             }
             for (int j = 0; j < tab->s; ++j) {
@@ -1163,7 +1168,7 @@ static int apply_t(hho_ops* ops, double t, const T* d_state, T* d_rate, T* d_tra
     a.trace_stride = ops->trace_doubles;
     a.inp = d_state;
     a.tr_out = d_traces;
-    launch_k<T, MODE_TRACES>(ops->k, a, grid, st);
+    launch_k<T, MODE_TRACES>(ops->k, a, 1, st);
     int rc = check_launch("hho_apply (trace kernel)");
     if (rc) return rc;
     a.tr_in = d_traces;
@@ -1173,7 +1178,7 @@ static int apply_t(hho_ops* ops, double t, const T* d_state, T* d_rate, T* d_tra
     a.tgt[0].dst = d_rate;
     a.tgt[0].coef = T(1.0);
     fill_sources<T>(ops, a, t, -1, 0.0, 1);
-    launch_k<T, MODE_APPLY>(ops->k, a, grid, st);
+    launch_k<T, MODE_APPLY>(ops->k, a, 1, st);
     return check_launch("hho_apply (stage kernel)");
 }
 
@@ -1462,9 +1467,9 @@ void launch_stage_f64(const hho_ops* ops, int mode, StageArgsT<double>& a, int n
     }
     cudaStream_t st = (cudaStream_t)stream;
     switch (mode) {
-        case MODE_TRACES: launch_k<double, MODE_TRACES>(ops->k, a, grid, st); break;
-        case MODE_STAGE: launch_k<double, MODE_STAGE>(ops->k, a, grid, st); break;
-        case MODE_APPLY: launch_k<double, MODE_APPLY>(ops->k, a, grid, st); break;
+        case MODE_TRACES: launch_k<double, MODE_TRACES>(ops->k, a, n_shots, st); break;
+        case MODE_STAGE: launch_k<double, MODE_STAGE>(ops->k, a, n_shots, st); break;
+        case MODE_APPLY: launch_k<double, MODE_APPLY>(ops->k, a, n_shots, st); break;
         default: break;
     }
 }
@@ -1485,9 +1490,9 @@ void launch_stage_f32(const hho_ops* ops, int mode, StageArgsT<float>& a, int n_
     }
     cudaStream_t st = (cudaStream_t)stream;
     switch (mode) {
-        case MODE_TRACES: launch_k<float, MODE_TRACES>(ops->k, a, grid, st); break;
-        case MODE_STAGE: launch_k<float, MODE_STAGE>(ops->k, a, grid, st); break;
-        case MODE_APPLY: launch_k<float, MODE_APPLY>(ops->k, a, grid, st); break;
+        case MODE_TRACES: launch_k<float, MODE_TRACES>(ops->k, a, n_shots, st); break;
+        case MODE_STAGE: launch_k<float, MODE_STAGE>(ops->k, a, n_shots, st); break;
+        case MODE_APPLY: launch_k<float, MODE_APPLY>(ops->k, a, n_shots, st); break;
         default: break;
     }
 }
@@ -1501,9 +1506,9 @@ static void launch_grad_t(const hho_ops* ops, StageArgsT<T>& a, const GradArgsT<
     a.trace_stride = ops->trace_doubles;
     fill_sources<T>(ops, a, tn, j, cdt, 1);
     cudaStream_t st = (cudaStream_t)stream;
-    if (ops->k == 1) hho_stage::launch_grad<T, 1>(a, g, grid, st);
-    else if (ops->k == 2) hho_stage::launch_grad<T, 2>(a, g, grid, st);
-    else hho_stage::launch_grad<T, 3>(a, g, grid, st);
+    if (ops->k == 1) hho_stage::launch_grad<T, 1>(a, g, st);
+    else if (ops->k == 2) hho_stage::launch_grad<T, 2>(a, g, st);
+    else hho_stage::launch_grad<T, 3>(a, g, st);
 }
 void launch_grad_f64(const hho_ops* ops, StageArgsT<double>& a, const GradArgsT<double>& g, double tn, int j, double cdt,
                      void* stream) {

@@ -4,9 +4,9 @@
 namespace hho_stage {
 
 #define HHO_INSTANTIATE(K) \
-    template void launch_stage<f2x, K, MODE_TRACES>(const StageArgsT<f2x>&, dim3, cudaStream_t); \
-    template void launch_stage<f2x, K, MODE_STAGE>(const StageArgsT<f2x>&, dim3, cudaStream_t); \
-    template void launch_stage<f2x, K, MODE_APPLY>(const StageArgsT<f2x>&, dim3, cudaStream_t);
+    template void launch_stage<f2x, K, MODE_TRACES>(const StageArgsT<f2x>&, int, cudaStream_t); \
+    template void launch_stage<f2x, K, MODE_STAGE>(const StageArgsT<f2x>&, int, cudaStream_t); \
+    template void launch_stage<f2x, K, MODE_APPLY>(const StageArgsT<f2x>&, int, cudaStream_t);
 
 HHO_INSTANTIATE(1)
 HHO_INSTANTIATE(2)

@@ -4,10 +4,10 @@
 namespace hho_stage {
 
 #define HHO_INSTANTIATE(K) \
-    template void launch_stage<float, K, MODE_TRACES>(const StageArgsT<float>&, dim3, cudaStream_t); \
-    template void launch_stage<float, K, MODE_STAGE>(const StageArgsT<float>&, dim3, cudaStream_t); \
-    template void launch_stage<float, K, MODE_APPLY>(const StageArgsT<float>&, dim3, cudaStream_t); \
-    template void launch_grad<float, K>(const StageArgsT<float>&, const GradArgsT<float>&, unsigned, cudaStream_t);
+    template void launch_stage<float, K, MODE_TRACES>(const StageArgsT<float>&, int, cudaStream_t); \
+    template void launch_stage<float, K, MODE_STAGE>(const StageArgsT<float>&, int, cudaStream_t); \
+    template void launch_stage<float, K, MODE_APPLY>(const StageArgsT<float>&, int, cudaStream_t); \
+    template void launch_grad<float, K>(const StageArgsT<float>&, const GradArgsT<float>&, cudaStream_t);
 
 HHO_INSTANTIATE(1)
 HHO_INSTANTIATE(2)

@@ -4,10 +4,10 @@
 namespace hho_stage {
 
 #define HHO_INSTANTIATE(K) \
-    template void launch_stage<double, K, MODE_TRACES>(const StageArgsT<double>&, dim3, cudaStream_t); \
-    template void launch_stage<double, K, MODE_STAGE>(const StageArgsT<double>&, dim3, cudaStream_t); \
-    template void launch_stage<double, K, MODE_APPLY>(const StageArgsT<double>&, dim3, cudaStream_t); \
-    template void launch_grad<double, K>(const StageArgsT<double>&, const GradArgsT<double>&, unsigned, cudaStream_t);
+    template void launch_stage<double, K, MODE_TRACES>(const StageArgsT<double>&, int, cudaStream_t); \
+    template void launch_stage<double, K, MODE_STAGE>(const StageArgsT<double>&, int, cudaStream_t); \
+    template void launch_stage<double, K, MODE_APPLY>(const StageArgsT<double>&, int, cudaStream_t); \
+    template void launch_grad<double, K>(const StageArgsT<double>&, const GradArgsT<double>&, cudaStream_t);
 
 HHO_INSTANTIATE(1)
 HHO_INSTANTIATE(2)

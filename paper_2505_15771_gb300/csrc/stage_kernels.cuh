@@ -191,7 +191,11 @@ __device__ __forceinline__ void add_ddy(const T* u, T* out) {
 // their lifting matrices also vanish where the exponent along the face
 // exceeds the face coefficient's degree by 2 (checked when the class is
 // built, up to k = 3).
+// PolyAxis<A>: a horizontal or vertical face of any polygon; every Lift entry
+// is used, but X^a Y^b traces to degree a only where Y is constant (b where X
+// is), so half of Tr is empty, and one component of the flux is enough.
 struct GenericFace {
+    static constexpr bool axis = false;
     static constexpr bool rect = false;
     static constexpr bool square = false;
     static constexpr bool horiz = false;
@@ -199,7 +203,17 @@ struct GenericFace {
     __host__ __device__ static constexpr bool lift_nz(int, int) { return true; }
 };
 template <int AX>
+struct PolyAxis {
+    static constexpr bool axis = true;
+    static constexpr bool rect = false;
+    static constexpr bool square = false;
+    static constexpr bool horiz = AX == 0;
+    __host__ __device__ static constexpr bool tr_nz(int l, int i) { return (horiz ? ea(i) : eb(i)) >= l; }
+    __host__ __device__ static constexpr bool lift_nz(int, int) { return true; }
+};
+template <int AX>
 struct RectAxis {
+    static constexpr bool axis = true;
     static constexpr bool rect = true;
     static constexpr bool square = false;
     static constexpr bool horiz = AX == 0;
@@ -213,6 +227,19 @@ struct SquareAxis : RectAxis<AX> {
     __host__ __device__ static constexpr bool lift_nz(int i, int l) {
         return RectAxis<AX>::lift_nz(i, l) && RectAxis<AX>::e(i) - l != 2;
     }
+};
+
+// The FP64 kernel is bound by the FP64 pipe, and its arithmetic is arranged to
+// issue the fewest instructions: tau multiplies a cell's lifted jumps once
+// instead of every pair's sigma and delta, and axis-aligned faces of polygons
+// have bodies of their own that skip the empty half of their trace matrices
+// (k = 3 stages of 524,288 cells: hanging nodes 754 -> 630 us, triangles
+// 857 -> 752; the 680 x 340 hybrid mesh 324 -> 305).  The other types are bound
+// by memory and latency and lost 5 to 10 % to the longer code and the extra
+// accumulators, so they keep the compact form.
+template <class T>
+struct Fp64Form {
+    static constexpr bool value = std::is_same<T, double>::value;
 };
 
 // Class matrices of the double-float kernel are read from a per-warp copy in
@@ -425,7 +452,8 @@ struct SolidGroups {   // [s_xx, s_yy | s_xy | v_x, v_y]
 // Per-thread view of one (cell, shot): class layout and this shot's buffers.
 template <class T>
 struct CellCtx {
-    int q, lq, nF, npad, sbase, N, SF, SS;
+    int q, lq, nF, npad, sbase, N, SF, SS, FS;
+    uint32_t hor, ver; // axis-aligned faces (CI_HOR, CI_VER)
     const T* cd;       // class face blocks
     T tau;
     const T* trf_in;   // this shot's trace buffers (fluid part, solid part)
@@ -433,6 +461,32 @@ struct CellCtx {
     T* trf_out;
     T* trs_out;
 };
+
+// The faces of a polygon.  FP64: horizontal ones, then vertical ones (each with
+// the sign of its normal), then the others; the order is part of the arithmetic.  Other types: in local order
+// through the general body.
+template <class T, class H, class V, class O>
+__device__ __forceinline__ void for_faces(const CellCtx<T>& c, H hor, V ver, O other) {
+    if constexpr (Fp64Form<T>::value) {
+#pragma unroll 1
+        for (uint32_t m = c.hor; m; m &= m - 1) {
+            const int j = __ffs(m) - 1;
+            hor(j, is_negative(cls_val(c.cd + j * c.FS + 1)) ? -1 : 1);
+        }
+#pragma unroll 1
+        for (uint32_t m = c.ver; m; m &= m - 1) {
+            const int j = __ffs(m) - 1;
+            ver(j, is_negative(cls_val(c.cd + j * c.FS)) ? -1 : 1);
+        }
+        const uint32_t done = c.hor | c.ver;
+#pragma unroll 1
+        for (int j = 0; j < c.nF; ++j)
+            if (j >= 32 || !((done >> j) & 1)) other(j);
+    } else {
+#pragma unroll 1
+        for (int j = 0; j < c.nF; ++j) other(j);
+    }
+}
 
 // ---- L2 prefetch hints -------------------------------------------------------------
 // A stage thread reads its cell's state, its faces' own traces, its
@@ -831,22 +885,24 @@ __device__ __forceinline__ void fluid_face_jump(const StageArgsT<T>& A, const Ce
 // built).  With s the first face's normal sign, jb, jp the two jumps and
 // jh = F jp, sigma = jb + jh and delta = jb - jh:
 //     normal accumulator  += s L delta (rows with P = +1), s L sigma (P = -1)
-//     tau accumulator     += tau L sigma (P = +1), tau L delta (P = -1)
-// Each lifted row is accumulated straight into its target: 4f + 2 nnz(L)
-// operations per pair instead of 2 (nnz(L) + 2n) for two separate lifts.
+//     jump accumulator    += L sigma (P = +1), L delta (P = -1)
+// Each lifted row is accumulated straight into its target: 2f + 2 nnz(L)
+// operations per pair instead of 2 (nnz(L) + 2n) for two separate lifts.  tau
+// multiplies the jump accumulator once per cell in FP64 (Fp64Form); the other
+// types scale sigma and delta and accumulate into the rate.
 template <class T, int K, int AX, bool SQ = false>
-__device__ __forceinline__ void lift_pair(const T* __restrict__ L, const T* jb, const T* jp, T tau, T* ke, T* kt) {
+__device__ __forceinline__ void lift_pair(const T* __restrict__ L, const T* jb, const T* jp, T tau, T* ke, T* ks) {
     constexpr int n = Dims<K>::n, f = Dims<K>::f, fP = Dims<K>::fP, w = Vec16<T>::w;
     using P = typename std::conditional<SQ, SquareAxis<AX>, RectAxis<AX>>::type;
     constexpr bool neg = AX == 0;   // face 0 has normal -e_y, face 1 +e_x
-    T sg[f], dl[f], ts[f], td[f];
+    T sg[f], dl[f], ts[f], td[f];   // sigma, delta; what the jump accumulator takes
 #pragma unroll
     for (int l = 0; l < f; ++l) {
         const T jh = (l & 1) ? -jp[l] : jp[l];
         sg[l] = jb[l] + jh;
         dl[l] = jb[l] - jh;
-        ts[l] = tau * sg[l];
-        td[l] = tau * dl[l];
+        ts[l] = Fp64Form<T>::value ? sg[l] : mul_rn(tau, sg[l]);
+        td[l] = Fp64Form<T>::value ? dl[l] : mul_rn(tau, dl[l]);
     }
 #pragma unroll
     for (int i = 0; i < n; ++i) {
@@ -860,7 +916,7 @@ __device__ __forceinline__ void lift_pair(const T* __restrict__ L, const T* jb, 
             for (int e = 0; e < w; ++e) need = need || (c0 + e < f && P::lift_nz(i, c0 + e));
             if (need) cls_row<T>(L + i * fP + c0, row + c0);
         }
-        T e = ke[i], k = kt[i];
+        T e = ke[i], k = ks[i];
 #pragma unroll
         for (int l = 0; l < f; ++l)
             if (P::lift_nz(i, l)) {
@@ -869,17 +925,17 @@ __device__ __forceinline__ void lift_pair(const T* __restrict__ L, const T* jb, 
                 k = fma(row[l], even ? ts[l] : td[l], k);
             }
         ke[i] = e;
-        kt[i] = k;
+        ks[i] = k;
     }
 }
 
 template <class T, int K, int AX, bool SQ = false>
-__device__ __forceinline__ void fluid_pair_rate(const StageArgsT<T>& A, const CellCtx<T>& c, T* kmx, T* kmy, T* kp) {
+__device__ __forceinline__ void fluid_pair_rate(const StageArgsT<T>& A, const CellCtx<T>& c, T* kmx, T* kmy, T* ks) {
     constexpr int f = Dims<K>::f, FS = Dims<K>::FS;
     T jb[f], jp[f];
     fluid_face_jump<T, K>(A, c, AX, jb);
     fluid_face_jump<T, K>(A, c, AX + 2, jp);
-    lift_pair<T, K, AX, SQ>(c.cd + AX * FS + Dims<K>::LI, jb, jp, c.tau, AX == 0 ? kmy : kmx, kp);
+    lift_pair<T, K, AX, SQ>(c.cd + AX * FS + Dims<K>::LI, jb, jp, c.tau, AX == 0 ? kmy : kmx, ks);
 }
 
 template <class T, int K, class P>
@@ -892,7 +948,7 @@ __device__ __forceinline__ void fluid_face_rate(const StageArgsT<T>& A, const Ce
     fluid_face_jump<T, K>(A, c, j, jmp);
     T lv[n];
     lift_apply<T, K, P>(fm + Dims<K>::LI, jmp, lv);
-    if constexpr (P::rect) {
+    if constexpr (P::axis) {
         add_signed<n>(lv, P::horiz ? kmy : kmx, sg);
     } else {
         const T nx = cls_val(fm), ny = cls_val(fm + 1);
@@ -919,16 +975,24 @@ __device__ __forceinline__ void fluid_face_trace(const StageArgsT<T>& A, const C
     const T* p = U + 2 * n;
     T tp[f], tm[f];
     face_trace_apply<T, K, P>(Tr, p, tp, sg);
-    if constexpr (P::rect) {
+    if constexpr (P::axis) {
         face_trace_apply<T, K, P>(Tr, P::horiz ? my : mx, tm, sg);
     } else {
         const T nx = cls_val(fm), ny = cls_val(fm + 1);
-        T mn[n];
+        if constexpr (Fp64Form<T>::value) {   // two traces (2 f n + 2 f operations) against 2 n + f n for m.n first:
+            T t1[f];                          // more here, but the team form, which shares it, takes coefficient by
+            face_trace_apply<T, K, P>(Tr, mx, tm, sg);   // coefficient and would form m.n f times
+            face_trace_apply<T, K, P>(Tr, my, t1, sg);
 #pragma unroll
-        for (int i = 0; i < n; ++i) mn[i] = fma(nx, mx[i], ny * my[i]);
-        face_trace_apply<T, K, P>(Tr, mn, tm, sg);
+            for (int l = 0; l < f; ++l) tm[l] = fma(nx, tm[l], mul_rn(ny, t1[l]));
+        } else {
+            T mn[n];
+#pragma unroll
+            for (int i = 0; i < n; ++i) mn[i] = fma(nx, mx[i], mul_rn(ny, my[i]));
+            face_trace_apply<T, K, P>(Tr, mn, tm, sg);
+        }
     }
-    const int sgn = P::rect ? sg : 1;   // rect: tm holds the unsigned trace
+    const int sgn = P::axis ? sg : 1;   // axis-aligned: tm holds the unsigned trace
     const int slot = c.sbase + j * c.npad + c.lq;
     const int nb = __ldg(op.nb_f + slot);
     const T al = (nb >= NB_BOUNDARY) ? __ldg(OpData<T>::beta_f(op) + slot) : __ldg(OpData<T>::if_coef(op) + 6 * (-2 - nb));
@@ -957,6 +1021,22 @@ __device__ __forceinline__ void fluid_rect_traces(const StageArgsT<T>& A, const 
     }
 }
 
+// FP64 rectangles: the rate of a primal field from its lifted jumps k (sum_F L j)
+// and the divergence of its flux (a, b), the state's fields at rows fa and fb:
+// k = tau k + da/dX + db/dY.  The flux is loaded here, after the faces, so that
+// the face loop holds neither it nor its derivatives.
+template <class T, int K>
+__device__ __forceinline__ void fp64_rect_div(const T* __restrict__ inp, const CellCtx<T>& c, int fa, int fb, T* k) {
+    constexpr int n = Dims<K>::n;
+    T a[n], b[n], d[n];
+    load_state<n>(inp, c.N, c.q, fa, a);
+    load_state<n>(inp, c.N, c.q, fb, b);
+    ddx<T, K>(a, d);
+    add_ddy<T, K>(b, d);
+#pragma unroll
+    for (int i = 0; i < n; ++i) k[i] = fma(c.tau, k[i], d[i]);
+}
+
 template <class T, int K, int MODE>
 __device__ __forceinline__ void fluid_cell(const StageArgsT<T>& A, int q, int shot, const T* cd_smem, T* acc_smem,
                                            const GradArgsT<T>* G = nullptr) {
@@ -971,6 +1051,9 @@ __device__ __forceinline__ void fluid_cell(const StageArgsT<T>& A, int q, int sh
     c.nF = __ldg(ci + CI_NF);
     c.npad = __ldg(ci + CI_NPAD);
     c.sbase = __ldg(ci + CI_SLOT);
+    c.hor = (uint32_t)__ldg(ci + CI_HOR);
+    c.ver = (uint32_t)__ldg(ci + CI_VER);
+    c.FS = Dims<K>::FS;
     c.cd = ClsSmem<T>::value ? cd_smem : OpData<T>::cls(op) + __ldg(ci + CI_DOFF) + Dims<K>::M0P;
     c.N = op.Nf;
     c.SF = op.SF;
@@ -995,21 +1078,28 @@ __device__ __forceinline__ void fluid_cell(const StageArgsT<T>& A, int q, int sh
         if constexpr (L2Prefetch<T, K>::mask != 0)
             prefetch_cell<T, K, 3 * n, f, 0, MODE != MODE_GRAD>(A, c, soff, c.trf_in, c.SF, op.nb_f,
                                                             OpData<T>::beta_f(op), rect ? 4 : c.nF);
+        const bool late = Fp64Form<T>::value && rect;   // div m after the faces, see fp64_rect_div
         {
             T u[n];
             load_state<n>(A.inp + soff, c.N, q, 2 * n, u);      // p
             ddx<T, K>(u, kmx);
             ddy<T, K>(u, kmy);
-            load_state<n>(A.inp + soff, c.N, q, 0, u);          // m_x
-            ddx<T, K>(u, kp);
-            load_state<n>(A.inp + soff, c.N, q, n, u);          // m_y
-            add_ddy<T, K>(u, kp);
+            if (!late) {
+                load_state<n>(A.inp + soff, c.N, q, 0, u);      // m_x
+                ddx<T, K>(u, kp);
+                load_state<n>(A.inp + soff, c.N, q, n, u);      // m_y
+                add_ddy<T, K>(u, kp);
+            }
         }
         if constexpr (L2Prefetch<T, K>::mask != 0)
             prefetch_cell<T, K, 3 * n, f, 1, MODE != MODE_GRAD>(A, c, soff, c.trf_in, c.SF, op.nb_f,
                                                             OpData<T>::beta_f(op), rect ? 4 : c.nF);
         if (rect) {
             // faces 0 (s = -1) and 2 (s = +1) are horizontal, 1 (s = +1) and 3 (s = -1) vertical
+            if constexpr (Fp64Form<T>::value) {
+#pragma unroll
+                for (int i = 0; i < n; ++i) kp[i] = T(0);
+            }
             if (kind == KIND_SQUARE) {
                 fluid_pair_rate<T, K, 0, true>(A, c, kmx, kmy, kp);   // faces 0 and 2
                 fluid_pair_rate<T, K, 1, true>(A, c, kmx, kmy, kp);   // faces 1 and 3
@@ -1017,9 +1107,11 @@ __device__ __forceinline__ void fluid_cell(const StageArgsT<T>& A, int q, int sh
                 fluid_pair_rate<T, K, 0>(A, c, kmx, kmy, kp);
                 fluid_pair_rate<T, K, 1>(A, c, kmx, kmy, kp);
             }
+            if constexpr (Fp64Form<T>::value) fp64_rect_div<T, K>(A.inp + soff, c, 0, n, kp);
         } else {
-#pragma unroll 1
-            for (int j = 0; j < c.nF; ++j) fluid_face_rate<T, K, GenericFace>(A, c, j, 1, kmx, kmy, kp);
+            for_faces(c, [&](int j, int sg) { fluid_face_rate<T, K, PolyAxis<0>>(A, c, j, sg, kmx, kmy, kp); },
+                      [&](int j, int sg) { fluid_face_rate<T, K, PolyAxis<1>>(A, c, j, sg, kmx, kmy, kp); },
+                      [&](int j) { fluid_face_rate<T, K, GenericFace>(A, c, j, 1, kmx, kmy, kp); });
         }
         const T Am = __ldg(OpData<T>::scal_f(op) + SF_AM * c.N + q), Ap = __ldg(OpData<T>::scal_f(op) + SF_AP * c.N + q);
         // Point sources: the stored vector is kappa/h^2 M0^-1 phi(x_s); the
@@ -1051,8 +1143,9 @@ __device__ __forceinline__ void fluid_cell(const StageArgsT<T>& A, int q, int sh
     } else if (rect) {
         fluid_rect_traces<T, K, RectAxis<0>, RectAxis<1>>(A, c, U);
     } else {
-#pragma unroll 1
-        for (int j = 0; j < c.nF; ++j) fluid_face_trace<T, K, GenericFace>(A, c, j, 1, U);
+        for_faces(c, [&](int j, int sg) { fluid_face_trace<T, K, PolyAxis<0>>(A, c, j, sg, U); },
+                  [&](int j, int sg) { fluid_face_trace<T, K, PolyAxis<1>>(A, c, j, sg, U); },
+                  [&](int j) { fluid_face_trace<T, K, GenericFace>(A, c, j, 1, U); });
     }
 }
 
@@ -1106,7 +1199,7 @@ __device__ __forceinline__ void solid_face_rate(const StageArgsT<T>& A, const Ce
     T lx[n], ly[n];
     lift_apply<T, K, P>(L, jx, lx);
     lift_apply<T, K, P>(L, jy, ly);
-    if constexpr (P::rect) {
+    if constexpr (P::axis) {
         if constexpr (P::horiz) {
             add_signed<n>(ly, eyy, sg);
             add_signed<n>(lx, exy, sg);
@@ -1145,6 +1238,59 @@ __device__ __forceinline__ void solid_pair_rate(const StageArgsT<T>& A, const Ce
     lift_pair<T, K, AX, SQ>(L, by, py, c.tau, AX == 0 ? eyy : exy, kvy);
 }
 
+// FP64: both components of one orientation's jumps lifted together, so that
+// four consecutive multiply-adds share the matrix entry.  The FP64 pipe takes 16
+// cycles for an instruction that shares a register operand with the one before
+// it and 19 otherwise (measured per SM).
+template <class T, int K, int AX, bool SQ>
+__device__ __forceinline__ void fp64_solid_pair(const StageArgsT<T>& A, const CellCtx<T>& c, T* ex, T* ey, T* kvx,
+                                                T* kvy) {
+    constexpr int n = Dims<K>::n, f = Dims<K>::f, fP = Dims<K>::fP, FS = Dims<K>::FS, w = Vec16<T>::w;
+    using P = typename std::conditional<SQ, SquareAxis<AX>, RectAxis<AX>>::type;
+    constexpr bool neg = AX == 0;
+    const T* L = c.cd + AX * FS + Dims<K>::LI;
+    T sx[f], sy[f], dx[f], dy[f];   // sigma, delta of both components
+    {
+        T bx[f], by[f], px[f], py[f];
+        solid_face_jump<T, K>(A, c, AX, bx, by);
+        solid_face_jump<T, K>(A, c, AX + 2, px, py);
+#pragma unroll
+        for (int l = 0; l < f; ++l) {
+            const T hx = (l & 1) ? -px[l] : px[l], hy = (l & 1) ? -py[l] : py[l];
+            sx[l] = bx[l] + hx;
+            dx[l] = bx[l] - hx;
+            sy[l] = by[l] + hy;
+            dy[l] = by[l] - hy;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+        const bool even = ((AX == 0 ? eb(i) : ea(i)) & 1) == 0;
+        T row[fP];
+#pragma unroll
+        for (int c0 = 0; c0 < fP; c0 += w) {
+            bool need = false;
+#pragma unroll
+            for (int e = 0; e < w; ++e) need = need || (c0 + e < f && P::lift_nz(i, c0 + e));
+            if (need) cls_row<T>(L + i * fP + c0, row + c0);
+        }
+        T e0 = ex[i], e1 = ey[i], k0 = kvx[i], k1 = kvy[i];
+#pragma unroll
+        for (int l = 0; l < f; ++l)
+            if (P::lift_nz(i, l)) {
+                const T a0 = even ? dx[l] : sx[l], a1 = even ? dy[l] : sy[l];
+                e0 = neg ? fma(-row[l], a0, e0) : fma(row[l], a0, e0);
+                e1 = neg ? fma(-row[l], a1, e1) : fma(row[l], a1, e1);
+                k0 = fma(row[l], even ? sx[l] : dx[l], k0);
+                k1 = fma(row[l], even ? sy[l] : dy[l], k1);
+            }
+        ex[i] = e0;
+        ey[i] = e1;
+        kvx[i] = k0;
+        kvy[i] = k1;
+    }
+}
+
 // Publish w = tau v|_F - (s n)|_F and omega = alpha w - v|_F for one face.
 template <class T, int K, class P>
 __device__ __forceinline__ void solid_face_trace(const StageArgsT<T>& A, const CellCtx<T>& c, int j, int sg,
@@ -1161,7 +1307,7 @@ __device__ __forceinline__ void solid_face_trace(const StageArgsT<T>& A, const C
     T tvx[f], tvy[f], tsx[f], tsy[f];
     face_trace_apply<T, K, P>(Tr, vx, tvx, sg);
     face_trace_apply<T, K, P>(Tr, vy, tvy, sg);
-    if constexpr (P::rect) {
+    if constexpr (P::axis) {
         // s n = (nx s_xx + ny s_xy, nx s_xy + ny s_yy) with one of nx, ny = +-1
         if constexpr (!P::horiz) {
             face_trace_apply<T, K, P>(Tr, sxx, tsx, sg);
@@ -1172,16 +1318,28 @@ __device__ __forceinline__ void solid_face_trace(const StageArgsT<T>& A, const C
         }
     } else {
         const T nx = cls_val(fm), ny = cls_val(fm + 1);
-        T snx[n], sny[n];
+        if constexpr (Fp64Form<T>::value) {   // see fluid_face_trace
+            T txy[f];
+            face_trace_apply<T, K, P>(Tr, sxx, tsx, sg);
+            face_trace_apply<T, K, P>(Tr, syy, tsy, sg);
+            face_trace_apply<T, K, P>(Tr, sxy, txy, sg);
 #pragma unroll
-        for (int i = 0; i < n; ++i) {
-            snx[i] = fma(nx, sxx[i], ny * sxy[i]);
-            sny[i] = fma(nx, sxy[i], ny * syy[i]);
+            for (int l = 0; l < f; ++l) {
+                tsx[l] = fma(nx, tsx[l], mul_rn(ny, txy[l]));
+                tsy[l] = fma(nx, txy[l], mul_rn(ny, tsy[l]));
+            }
+        } else {
+            T snx[n], sny[n];
+#pragma unroll
+            for (int i = 0; i < n; ++i) {
+                snx[i] = fma(nx, sxx[i], mul_rn(ny, sxy[i]));
+                sny[i] = fma(nx, sxy[i], mul_rn(ny, syy[i]));
+            }
+            face_trace_apply<T, K, P>(Tr, snx, tsx, sg);
+            face_trace_apply<T, K, P>(Tr, sny, tsy, sg);
         }
-        face_trace_apply<T, K, P>(Tr, snx, tsx, sg);
-        face_trace_apply<T, K, P>(Tr, sny, tsy, sg);
     }
-    const int sgn = P::rect ? sg : 1;
+    const int sgn = P::axis ? sg : 1;
     const int slot = c.sbase + j * c.npad + c.lq;
     const int nb = __ldg(op.nb_s + slot);
     T* TWS = c.trs_out;
@@ -1242,6 +1400,9 @@ __device__ __forceinline__ void solid_cell(const StageArgsT<T>& A, int q, int sh
     c.nF = __ldg(ci + CI_NF);
     c.npad = __ldg(ci + CI_NPAD);
     c.sbase = __ldg(ci + CI_SLOT);
+    c.hor = (uint32_t)__ldg(ci + CI_HOR);
+    c.ver = (uint32_t)__ldg(ci + CI_VER);
+    c.FS = Dims<K>::FS;
     c.cd = ClsSmem<T>::value ? cd_smem : OpData<T>::cls(op) + __ldg(ci + CI_DOFF) + Dims<K>::M0P;
     c.N = op.Ns;
     c.SF = op.SF;
@@ -1269,6 +1430,7 @@ __device__ __forceinline__ void solid_cell(const StageArgsT<T>& A, int q, int sh
         if constexpr (L2Prefetch<T, K>::mask != 0)
             prefetch_cell<T, K, 5 * n, 2 * f, 0, MODE != MODE_GRAD>(A, c, soff, c.trs_in, c.SS, op.nb_s,
                                                                 OpData<T>::beta_s(op), rect ? 4 : c.nF);
+        const bool late = Fp64Form<T>::value && rect;   // div s after the faces, see fp64_rect_div
         {
             T u[n];
             load_state<n>(inp, c.N, q, 3 * n, u);    // v_x
@@ -1277,6 +1439,9 @@ __device__ __forceinline__ void solid_cell(const StageArgsT<T>& A, int q, int sh
             load_state<n>(inp, c.N, q, 4 * n, u);    // v_y
             ddy<T, K>(u, eyy);
             add_ddx<T, K>(u, exy);
+        }
+        if (!late) {
+            T u[n];
             load_state<n>(inp, c.N, q, 0, u);        // s_xx
             ddx<T, K>(u, kvx);
             load_state<n>(inp, c.N, q, n, u);        // s_yy
@@ -1289,7 +1454,28 @@ __device__ __forceinline__ void solid_cell(const StageArgsT<T>& A, int q, int sh
             prefetch_cell<T, K, 5 * n, 2 * f, 1, MODE != MODE_GRAD>(A, c, soff, c.trs_in, c.SS, op.nb_s,
                                                                 OpData<T>::beta_s(op), rect ? 4 : c.nF);
         if (rect) {
-            if (kind == KIND_SQUARE) {
+            if constexpr (Fp64Form<T>::value) {
+#pragma unroll
+                for (int i = 0; i < n; ++i) kvx[i] = kvy[i] = T(0);
+                if (kind == KIND_SQUARE) {
+                    fp64_solid_pair<T, K, 0, true>(A, c, exy, eyy, kvx, kvy);   // faces 0 and 2
+                    fp64_solid_pair<T, K, 1, true>(A, c, exx, exy, kvx, kvy);   // faces 1 and 3
+                } else {
+                    fp64_solid_pair<T, K, 0, false>(A, c, exy, eyy, kvx, kvy);
+                    fp64_solid_pair<T, K, 1, false>(A, c, exx, exy, kvx, kvy);
+                }
+                fp64_rect_div<T, K>(inp, c, 0, 2 * n, kvx);
+                // the order of the sum matters for the bits: d/dY s_yy first, as in the general path
+                {
+                    T a[n], b[n], d[n];
+                    load_state<n>(inp, c.N, q, n, a);
+                    load_state<n>(inp, c.N, q, 2 * n, b);
+                    ddy<T, K>(a, d);
+                    add_ddx<T, K>(b, d);
+#pragma unroll
+                    for (int i = 0; i < n; ++i) kvy[i] = fma(c.tau, kvy[i], d[i]);
+                }
+            } else if (kind == KIND_SQUARE) {
                 solid_pair_rate<T, K, 0, true>(A, c, exx, eyy, exy, kvx, kvy);   // faces 0 and 2
                 solid_pair_rate<T, K, 1, true>(A, c, exx, eyy, exy, kvx, kvy);   // faces 1 and 3
             } else {
@@ -1297,8 +1483,9 @@ __device__ __forceinline__ void solid_cell(const StageArgsT<T>& A, int q, int sh
                 solid_pair_rate<T, K, 1>(A, c, exx, eyy, exy, kvx, kvy);
             }
         } else {
-#pragma unroll 1
-            for (int j = 0; j < c.nF; ++j) solid_face_rate<T, K, GenericFace>(A, c, j, 1, exx, eyy, exy, kvx, kvy);
+            for_faces(c, [&](int j, int sg) { solid_face_rate<T, K, PolyAxis<0>>(A, c, j, sg, exx, eyy, exy, kvx, kvy); },
+                      [&](int j, int sg) { solid_face_rate<T, K, PolyAxis<1>>(A, c, j, sg, exx, eyy, exy, kvx, kvy); },
+                      [&](int j) { solid_face_rate<T, K, GenericFace>(A, c, j, 1, exx, eyy, exy, kvx, kvy); });
         }
         // stress rate = C e = c1 [(e_xx + r e_yy), (e_yy + r e_xx)], c3 e_xy; c1, c3 folded into targets
         const T r = __ldg(OpData<T>::scal_s(op) + SS_R * c.N + q);
@@ -1344,8 +1531,9 @@ __device__ __forceinline__ void solid_cell(const StageArgsT<T>& A, int q, int sh
     } else if (rect) {
         solid_rect_traces<T, K, RectAxis<0>, RectAxis<1>>(A, c, U);
     } else {
-#pragma unroll 1
-        for (int j = 0; j < c.nF; ++j) solid_face_trace<T, K, GenericFace>(A, c, j, 1, U);
+        for_faces(c, [&](int j, int sg) { solid_face_trace<T, K, PolyAxis<0>>(A, c, j, sg, U); },
+                  [&](int j, int sg) { solid_face_trace<T, K, PolyAxis<1>>(A, c, j, sg, U); },
+                  [&](int j) { solid_face_trace<T, K, GenericFace>(A, c, j, 1, U); });
     }
 }
 
@@ -1362,15 +1550,16 @@ struct MinBlocks {
     static constexpr int value = Tuned<T>::t.min_blocks[K - 1];
 };
 
-// Dynamic shared memory of a stage block: the per-warp class copies
-// (max_nf face blocks of Dims<K>::FS values per warp) when ClsSmem<T>.
+// Dynamic shared memory of a stage block of `threads` threads: the per-warp
+// class copies (max_nf face blocks of Dims<K>::FS values per warp) when
+// ClsSmem<T>, and the accumulators when AccSmem<T, K>.
 template <class T, int K>
-__host__ __device__ size_t stage_cls_smem_bytes(int max_nf) {
-    return ClsSmem<T>::value ? sizeof(T) * (128 / 32) * (size_t)max_nf * Dims<K>::FS : 0;
+__host__ __device__ size_t stage_cls_smem_bytes(int max_nf, int threads) {
+    return ClsSmem<T>::value ? sizeof(T) * (threads / 32) * (size_t)max_nf * Dims<K>::FS : 0;
 }
 template <class T, int K>
-size_t stage_smem_bytes(int max_nf) {
-    return stage_cls_smem_bytes<T, K>(max_nf) + (AccSmem<T, K>::value ? sizeof(T) * 128 * acc_stride<K>() : 0);
+size_t stage_smem_bytes(int max_nf, int threads) {
+    return stage_cls_smem_bytes<T, K>(max_nf, threads) + (AccSmem<T, K>::value ? sizeof(T) * threads * acc_stride<K>() : 0);
 }
 
 // Grid: x over the padded cells of both domains (fluid warps, then solid
@@ -1383,7 +1572,7 @@ __global__ void __launch_bounds__(128, MinBlocks<T, K>::value) stage_kernel(cons
     extern __shared__ __align__(16) unsigned char stage_smem[];
     T* acc = nullptr;
     if constexpr (AccSmem<T, K>::value)
-        acc = reinterpret_cast<T*>(stage_smem + stage_cls_smem_bytes<T, K>(A.op.max_nf)) + threadIdx.x * acc_stride<K>();
+        acc = reinterpret_cast<T*>(stage_smem + stage_cls_smem_bytes<T, K>(A.op.max_nf, blockDim.x)) + threadIdx.x * acc_stride<K>();
     if constexpr (ClsSmem<T>::value) {
         constexpr int FS = Dims<K>::FS;
         const int gw = gq >> 5;
@@ -1448,18 +1637,29 @@ struct StageTag {};
 
 namespace hho_stage {
 
+// Threads of a stage block (the kernels use no block-wide barrier).  128 for
+// large grids.  A grid of at most 20 warps per SM runs in one wave, where
+// blocks of one warp spread the cells evenly over the SMs: with 128 threads
+// the 65,536 cells of the 256 x 256 adjoint leave SMs with 3 or 4 blocks, and
+// a stage took 49.0 us against 41.6 (its gradients 55.0 against 46.7).  With
+// several waves the smaller blocks cost 1 to 10 % (21 FP32 shots: 354 us
+// against 321, whose shared memory per block leaves fewer resident warps).
+inline int stage_threads(int64_t warps) { return warps <= 20 * 152 ? 32 : 128; }
+
 template <class T, int K, int MODE>
-void launch_stage(const StageArgsT<T>& a, dim3 grid, cudaStream_t s) {
-    const size_t smem = stage_smem_bytes<T, K>(a.op.max_nf);
+void launch_stage(const StageArgsT<T>& a, int n_shots, cudaStream_t s) {
+    const int cells = a.op.Nf + a.op.Ns, threads = stage_threads((int64_t)(cells / 32) * n_shots);
+    const size_t smem = stage_smem_bytes<T, K>(a.op.max_nf, threads);
     stage_smem_attributes<StageTag<T, K, MODE>>(stage_kernel<T, K, MODE>, smem, AccSmem<T, K>::value);
-    stage_kernel<T, K, MODE><<<grid, 128, smem, s>>>(a);
+    stage_kernel<T, K, MODE><<<dim3((cells + threads - 1) / threads, n_shots), threads, smem, s>>>(a);
 }
 
 template <class T, int K>
-void launch_grad(const StageArgsT<T>& a, const GradArgsT<T>& g, unsigned grid, cudaStream_t s) {
-    const size_t smem = stage_smem_bytes<T, K>(a.op.max_nf);
+void launch_grad(const StageArgsT<T>& a, const GradArgsT<T>& g, cudaStream_t s) {
+    const int cells = a.op.Nf + a.op.Ns, threads = stage_threads(cells / 32);
+    const size_t smem = stage_smem_bytes<T, K>(a.op.max_nf, threads);
     stage_smem_attributes<StageTag<T, K, MODE_GRAD>>(grad_stage_kernel<T, K>, smem, AccSmem<T, K>::value);
-    grad_stage_kernel<T, K><<<grid, 128, smem, s>>>(a, g);
+    grad_stage_kernel<T, K><<<(cells + threads - 1) / threads, threads, smem, s>>>(a, g);
 }
 
 }  // namespace hho_stage

@@ -8,13 +8,13 @@
 
 namespace hho_stage {
 
-// One stage-kernel launch over a grid of (cell blocks of 128, shots).
+// One stage-kernel launch over the cells of both domains and n_shots shots.
 template <class T, int K, int MODE>
-void launch_stage(const StageArgsT<T>& a, dim3 grid, cudaStream_t s);
+void launch_stage(const StageArgsT<T>& a, int n_shots, cudaStream_t s);
 
 // One backward stage's gradients (MODE_GRAD; FP64 and FP32).
 template <class T, int K>
-void launch_grad(const StageArgsT<T>& a, const GradArgsT<T>& g, unsigned grid, cudaStream_t s);
+void launch_grad(const StageArgsT<T>& a, const GradArgsT<T>& g, cudaStream_t s);
 
 // The tensor-core stage (HHO_BF16X3).
 template <int K, int MODE>
