@@ -463,7 +463,8 @@ struct CellCtx {
 };
 
 // The faces of a polygon.  FP64: horizontal ones, then vertical ones (each with
-// the sign of its normal), then the others; the order is part of the arithmetic.  Other types: in local order
+// the sign of its normal), then the others; the order is part of the arithmetic,
+// and the team form adds the faces in the same one.  Other types: in local order
 // through the general body.
 template <class T, class H, class V, class O>
 __device__ __forceinline__ void for_faces(const CellCtx<T>& c, H hor, V ver, O other) {
@@ -1609,6 +1610,8 @@ __global__ void __launch_bounds__(128, MinBlocks<T, K>::value)
         solid_cell<T, K, MODE_GRAD>(A, gq - A.op.Nf, 0, nullptr, acc, &G);
 }
 
+#include "stage_team.cuh"
+
 // Per function and device: the opt-in above 48 KB of dynamic shared memory
 // (the largest size set is remembered), and the largest carveout where the
 // accumulators live in shared memory, for the resident blocks that the
@@ -1646,8 +1649,66 @@ namespace hho_stage {
 // against 321, whose shared memory per block leaves fewer resident warps).
 inline int stage_threads(int64_t warps) { return warps <= 20 * 152 ? 32 : 128; }
 
+template <class T, int K, int MODE, int W>
+struct TeamTag {};
+
+// Where the team form (stage_team.cuh) is the faster one: up to so many groups
+// of 32 cells (times shots), by arithmetic, degree, mode (stage, application,
+// traces alone) and mesh (at least a quarter of the groups not rectangles: gen).
+// Small grids take W warps a block, larger ones four (fewer idle warps, more
+// blocks an SM) but for the 8-byte types at k = 3, whose ten rows fit ten warps.
+// Both forms give the same bits, so the choice is free.  Measured on GB300, us
+// a stage, thread form / team form:
+//                             128 groups    1024 groups    4096 groups
+//   FP64 k = 2 squares        26.4 / 8.6    30.4 / 25.8    82.6 / 93.2
+//   FP64 k = 3 hanging        81.9 / 18.2   97 / 61        214 / 196
+//   double-float k = 2 squares 23.1 / 6.4   26.9 / 13.6    65.2 / 54.2
+//   double-float k = 3 tri.   49.6 / 8.4    57.7 / 25.7    162 / 96
+//   FP32 k = 2 squares        13.8 / 4.8    19.0 / 8.3     22.6 / 25.6
+// Large FP64 grids are bound by the FP64 pipe, and the thread form issues the
+// fewer FP64 instructions; large FP32 ones by memory, where its coalesced rows
+// of one warp do as well with less code.
+template <class T, int K>
+struct TeamRule;
+constexpr int TEAM_ALL = 1 << 30;
+#define HHO_TEAM_RULE(T_, K_, W_, rect_, gen_, app_, tr_rect_, tr_gen_)                                        \
+    template <>                                                                                               \
+    struct TeamRule<T_, K_> {                                                                                 \
+        static constexpr int W = W_, rect = rect_, gen = gen_, app = app_, tr_rect = tr_rect_, tr_gen = tr_gen_; \
+    }
+HHO_TEAM_RULE(double, 1, 8, 1000, 1300, 900, 128, 400);
+HHO_TEAM_RULE(double, 2, 8, 1500, 2000, 1150, 200, 600);
+HHO_TEAM_RULE(double, 3, 10, 2000, 3500, 1500, 300, 900);
+HHO_TEAM_RULE(f2x, 1, 8, 2000, 2600, 1500, 700, 900);
+HHO_TEAM_RULE(f2x, 2, 8, TEAM_ALL, TEAM_ALL, 3000, 512, 1100);
+HHO_TEAM_RULE(f2x, 3, 10, TEAM_ALL, TEAM_ALL, 3000, 1100, TEAM_ALL);
+HHO_TEAM_RULE(float, 1, 8, 1800, 2100, 0, 200, 300);
+HHO_TEAM_RULE(float, 2, 8, 3000, 3000, 0, 200, 300);
+HHO_TEAM_RULE(float, 3, 10, 3500, 4100, 0, 200, 400);
+#undef HHO_TEAM_RULE
+
+// Warps of a team block for this launch, 0 for the thread form.
+template <class T, int K, int MODE>
+int team_warps(const DevOps& op, int n_shots) {
+    using R = TeamRule<T, K>;
+    const int64_t cells = op.n_warps_f + op.n_warps_s, groups = cells * n_shots;
+    const bool gen = 4 * (cells - op.n_warps_rect) >= cells;
+    const int limit = MODE == MODE_TRACES ? (gen ? R::tr_gen : R::tr_rect) : MODE == MODE_APPLY ? R::app : gen ? R::gen : R::rect;
+    if (groups > limit || op.max_nf > 32 || sizeof(T) * team_smem_elems<T, K>(op.max_nf) > 200 * 1024) return 0;
+    return groups <= 600 || (K == 3 && sizeof(T) == 8) ? R::W : 4;
+}
+
 template <class T, int K, int MODE>
 void launch_stage(const StageArgsT<T>& a, int n_shots, cudaStream_t s) {
+    const int W = team_warps<T, K, MODE>(a.op, n_shots);
+    auto team = [&](auto wc) {
+        constexpr int TW = decltype(wc)::value;
+        const size_t smem = sizeof(T) * team_smem_elems<T, K>(a.op.max_nf);
+        stage_smem_attributes<TeamTag<T, K, MODE, TW>>(team_kernel<T, K, MODE, TW>, smem, true);
+        team_kernel<T, K, MODE, TW><<<dim3(a.op.n_warps_f + a.op.n_warps_s, n_shots), 32 * TW, smem, s>>>(a);
+    };
+    if (W == 4) return team(std::integral_constant<int, 4>());
+    if (W) return team(std::integral_constant<int, TeamRule<T, K>::W>());
     const int cells = a.op.Nf + a.op.Ns, threads = stage_threads((int64_t)(cells / 32) * n_shots);
     const size_t smem = stage_smem_bytes<T, K>(a.op.max_nf, threads);
     stage_smem_attributes<StageTag<T, K, MODE>>(stage_kernel<T, K, MODE>, smem, AccSmem<T, K>::value);
