@@ -16,7 +16,7 @@ OBJ = os.path.join(ROOT, "_build")
 LIB = os.path.join(HERE, "libhho.so")
 PROBE_LIB = os.path.join(HERE, "libhho_probe.so")
 # the translation units that stage_tuning.h reaches
-STAGE_SOURCES = ["stage_f64.cu", "stage_f32.cu", "stage_f2x.cu", "stage_tc.cu"]
+STAGE_SOURCES = ["stage_f64.cu", "stage_f32.cu", "stage_f2x.cu", "stage_tc.cu", "sdirk_bj.cu"]
 SOURCES = STAGE_SOURCES + ["mesh.cpp", "operators.cpp", "stage.cu", "adjoint.cu", "sdirk.cu", "tc.cu", "f2x_check.cu",
                            "probe.cu"]
 

@@ -219,6 +219,12 @@ void launch_record_f64(const hho_ops* ops, const double* state, double* out, voi
 int erk_steps_f32(hho_ops* ops, const hho_tableau* tab, double t0, double dt, int64_t nsteps, float* d_state,
                   float* d_work, void* stream);
 int check_cuda(const char* what);
+// y = *scale P^-1 x (scale null: 1; bj null: P = I; accumulate: y += ..., not with
+// traces), P^-1 the inverse cell blocks of hho_ops::d_bj; with tr, the FP64
+// face traces of y too, where bj_traces_fit (sdirk_bj.cu).
+bool bj_traces_fit(const hho_ops* ops);
+void launch_bj(const hho_ops* ops, const double* bj, const double* x, const double* scale, double* y, bool accumulate,
+               double* tr, void* stream);
 
 struct hho_ops {
     int32_t k = 0, n = 0, f = 0;
@@ -334,6 +340,8 @@ struct hho_ops {
     double bj_adt = 0.0;
     int32_t* d_bj_colour = nullptr;   // cell colouring, fluid then solid slots
     int32_t bj_colours = 0;
+    double* h_krylov = nullptr;       // pinned: a Krylov vector's sums and the combination's coefficients
+    void* krylov_event = nullptr;     // cudaEvent_t: those sums have arrived
     // stage-kernel timing (hho_profile_*)
     bool prof_on = false;
     int32_t prof_n = 0;

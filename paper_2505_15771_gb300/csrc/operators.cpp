@@ -968,6 +968,8 @@ extern "C" void hho_ops_destroy(hho_ops* ops) {
     if (ops->d_host_work) cudaFree(ops->d_host_work);
     if (ops->d_bj) cudaFree(ops->d_bj);
     if (ops->d_bj_colour) cudaFree(ops->d_bj_colour);
+    if (ops->h_krylov) cudaFreeHost(ops->h_krylov);
+    if (ops->krylov_event) cudaEventDestroy((cudaEvent_t)ops->krylov_event);
     for (void* e : ops->prof_events) cudaEventDestroy((cudaEvent_t)e);
     for (auto& g : ops->graphs)
         if (g.exec) cudaGraphExecDestroy((cudaGraphExec_t)g.exec);

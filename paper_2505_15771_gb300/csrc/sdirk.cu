@@ -17,9 +17,9 @@
 // inverse mass) with the target v - a* dt J v, so no global matrix is
 // assembled or stored and the implicit path reuses the explicit one's
 // kernels.  Orthogonalisation is classical Gram-Schmidt applied twice, with
-// its coefficients kept on the device; one copy to the host and one stream
-// synchronisation per Krylov vector.  All reductions are block-partial sums
-// added in a fixed order, so results are deterministic.
+// its coefficients kept on the device; the host reads each vector's sums while
+// the operator runs on the next.  All reductions are block-partial sums added in
+// a fixed order, so results are deterministic.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -31,72 +31,157 @@
 
 namespace {
 
-constexpr int RED_BLOCKS = 608;   // 4 x 152 SMs
-constexpr int RED_THREADS = 256;
+constexpr int RED_BLOCKS = 608;   // the partials' share of the work layout
 constexpr int MAX_RESTART = 64;
 
-// partial[b * nv + l] = block b's share of sum_i V_l[i] w[i], l < nv
-// (V_l = V + l * stride).  Four vectors per pass over i (independent FP64
-// chains), then one fixed tree over the block for the four sums.
-constexpr int MD_W = 4;
-__global__ void multidot_kernel(const double* __restrict__ V, int64_t stride, int nv, const double* __restrict__ w,
-                                int64_t n, double* __restrict__ partial) {
-    __shared__ double sh[MD_W][RED_THREADS];
-    for (int l0 = 0; l0 < nv; l0 += MD_W) {
-        const int nl = min(MD_W, nv - l0);
-        double acc[MD_W] = {0.0, 0.0, 0.0, 0.0};
-        for (int64_t i = blockIdx.x * (int64_t)RED_THREADS + threadIdx.x; i < n; i += (int64_t)gridDim.x * RED_THREADS) {
-            const double wi = w[i];
-#pragma unroll
-            for (int l = 0; l < MD_W; ++l)
-                if (l < nl) acc[l] = fma(V[(size_t)(l0 + l) * stride + i], wi, acc[l]);
-        }
-#pragma unroll
-        for (int l = 0; l < MD_W; ++l) sh[l][threadIdx.x] = acc[l];
-        __syncthreads();
-        for (int o = RED_THREADS / 2; o > 0; o >>= 1) {
-            if ((int)threadIdx.x < o)
-                for (int l = 0; l < nl; ++l) sh[l][threadIdx.x] += sh[l][threadIdx.x + o];
-            __syncthreads();
-        }
-        if ((int)threadIdx.x < nl) partial[(size_t)blockIdx.x * nv + l0 + threadIdx.x] = sh[threadIdx.x][0];
-        __syncthreads();
-    }
-}
+// ---- Krylov vector passes -------------------------------------------------------------
+// The Gram-Schmidt passes over n values and NV basis vectors V_l, which are kept
+// as computed, with factors inv_l = 1/||V_l|| beside them.  Each pass reads the
+// vectors once:
+//   DOT          out_l = inv_l V_l . w
+//   UPDATE       w -= sum_l c_l V_l,  c_l = in_l inv_l  (in: the DOT's out)
+//   UPDATE_DOT   the update, then the DOT with the new w in the same pass
+//   UPDATE_NORM  the update, then out_0 = w . w and *inv_out = 1/||w||
+//   NORM         out_0 = w . w, *inv_out as above
+//   RESIDUAL     w = V_0 - V_1 (operands b and A x), then as NORM
+// Block sums go through shared memory (a warp adds one vector's 256 values, so
+// the tree costs 13 FP64 instructions a vector and block), and the last block to
+// finish adds the blocks' partials: fixed orders, no second launch.  The main loop
+// shares w between the NV multiply-adds.  Before, one pass
+// each for the two dots and updates, the norm and the scaling with trees of
+// eight levels and a launch for every set of partials took 104 us of the 190 us
+// per vector on 786,432 values.
+enum { KR_DOT, KR_UPDATE, KR_UPDATE_DOT, KR_UPDATE_NORM, KR_NORM, KR_RESIDUAL };
+constexpr int KR_THREADS = 256, KR_MAX_BLOCKS = 3 * 152, KR_CHUNK = 12;
 
-// out[l] = sum over blocks of partial[b * nv + l]: block l; thread t adds
-// b = t, t + 256, ... in increasing order, then a fixed tree over the
-// threads.  (A single dependent chain over the 608 partials took about
-// 50 us a call on GB300, whose FP64 add latency is long.)
-__global__ void sum_partials_kernel(const double* __restrict__ partial, int nb, int nv, double* __restrict__ out) {
-    __shared__ double sh[RED_THREADS];
-    const int l = blockIdx.x;
-    double s = 0.0;
-    for (int b = threadIdx.x; b < nb; b += RED_THREADS) s += partial[(size_t)b * nv + l];
-    sh[threadIdx.x] = s;
+struct KrylovArgs {
+    const double* V;
+    int64_t stride, n;
+    double* w;
+    const double* in;        // previous dots (updates)
+    const double* inv;
+    double* partial;
+    unsigned* ticket;        // 0 before and after every launch
+    double* out;
+    double* inv_out;
+    const double* b;         // RESIDUAL: w = b - V
+};
+
+template <int NV, int MODE>
+__global__ void __launch_bounds__(KR_THREADS, 3) krylov_kernel(const KrylovArgs A) {
+    constexpr bool UPD = MODE == KR_UPDATE || MODE == KR_UPDATE_DOT || MODE == KR_UPDATE_NORM;
+    constexpr bool DOTS = MODE == KR_DOT || MODE == KR_UPDATE_DOT;
+    constexpr int NR = MODE == KR_UPDATE ? 0 : DOTS ? NV : 1;   // sums
+    constexpr int M = NV > 0 ? NV : 1, R = NR > 0 ? NR : 1;
+    double c[M], acc[R];
+    if constexpr (UPD) {
+#pragma unroll
+        for (int l = 0; l < NV; ++l) c[l] = A.in[l] * A.inv[l];
+    }
+#pragma unroll
+    for (int l = 0; l < R; ++l) acc[l] = 0.0;
+    const int64_t step = (int64_t)gridDim.x * KR_THREADS;
+    auto update = [&](double w, const double* v) {
+#pragma unroll
+        for (int l = 0; l < NV; ++l) w = fma(-c[l], v[l], w);
+        return w;
+    };
+    auto sums = [&](double w, const double* v) {
+        if constexpr (DOTS) {
+#pragma unroll
+            for (int l = 0; l < NV; ++l) acc[l] = fma(w, v[l], acc[l]);
+        } else if constexpr (NR > 0) {
+            acc[0] = fma(w, w, acc[0]);
+        }
+    };
+    int64_t i = blockIdx.x * (int64_t)KR_THREADS + threadIdx.x;
+    for (; i + step < A.n; i += 2 * step) {   // two elements' loads in flight
+        double v0[M], v1[M];
+#pragma unroll
+        for (int l = 0; l < NV; ++l) {
+            v0[l] = A.V[(size_t)l * A.stride + i];
+            v1[l] = A.V[(size_t)l * A.stride + i + step];
+        }
+        double w0 = MODE == KR_RESIDUAL ? A.b[i] - v0[0] : A.w[i];
+        double w1 = MODE == KR_RESIDUAL ? A.b[i + step] - v1[0] : A.w[i + step];
+        if constexpr (UPD) {
+            w0 = update(w0, v0);
+            w1 = update(w1, v1);
+        }
+        if constexpr (UPD || MODE == KR_RESIDUAL) {
+            A.w[i] = w0;
+            A.w[i + step] = w1;
+        }
+        sums(w0, v0);
+        sums(w1, v1);
+    }
+    if (i < A.n) {
+        double v[M];
+#pragma unroll
+        for (int l = 0; l < NV; ++l) v[l] = A.V[(size_t)l * A.stride + i];
+        double w = MODE == KR_RESIDUAL ? A.b[i] - v[0] : A.w[i];
+        if constexpr (UPD) w = update(w, v);
+        if constexpr (UPD || MODE == KR_RESIDUAL) A.w[i] = w;
+        sums(w, v);
+    }
+    if constexpr (NR == 0) return;
+    __shared__ double sh[R][KR_THREADS];
+    __shared__ bool last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int l = 0; l < R; ++l) sh[l][threadIdx.x] = acc[l];
     __syncthreads();
-    for (int o = RED_THREADS / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
+    auto warp_sum = [&](double x) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        return x;
+    };
+    for (int l = warp; l < R; l += KR_THREADS / 32) {
+        double x = sh[l][lane];
+#pragma unroll
+        for (int t = 1; t < KR_THREADS / 32; ++t) x += sh[l][lane + 32 * t];
+        x = warp_sum(x);
+        if (lane == 0) A.partial[(size_t)l * gridDim.x + blockIdx.x] = x;
     }
-    if (threadIdx.x == 0) out[l] = sh[0];
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(A.ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int l = warp; l < R; l += KR_THREADS / 32) {
+        double x = 0.0;
+        for (int b = lane; b < (int)gridDim.x; b += 32) x += __ldcg(A.partial + (size_t)l * gridDim.x + b);
+        x = warp_sum(x);
+        if (lane == 0) {
+            A.out[l] = DOTS ? x * A.inv[l] : x;
+            if (!DOTS && A.inv_out) *A.inv_out = x > 0.0 ? 1.0 / sqrt(x) : 0.0;
+        }
+    }
+    if (threadIdx.x == 0) *A.ticket = 0;
 }
 
-// y = alpha y + beta sum_l coef[l] V_l  (coef in device memory; y may be
-// one of the V_l: each element is read before the same thread writes it)
-__global__ void lincomb_kernel(double* y, double alpha, double beta, const double* V, int64_t stride, int nv,
+template <int MODE>
+void krylov(int nv, const KrylovArgs& A, cudaStream_t st) {
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((A.n + KR_THREADS - 1) / KR_THREADS, KR_MAX_BLOCKS));
+    switch (nv) {
+#define KR_CASE(N) case N: krylov_kernel<N, MODE><<<blocks, KR_THREADS, 0, st>>>(A); break;
+        KR_CASE(1) KR_CASE(2) KR_CASE(3) KR_CASE(4) KR_CASE(5) KR_CASE(6)
+        KR_CASE(7) KR_CASE(8) KR_CASE(9) KR_CASE(10) KR_CASE(11) KR_CASE(12)
+#undef KR_CASE
+    }
+}
+
+// y = alpha y + sum_l coef[l] V_l  (coef in device memory; alpha = 0: y is not
+// read; y may be one of the V_l: each element is read before the same thread
+// writes it)
+__global__ void lincomb_kernel(double* y, double alpha, const double* V, int64_t stride, int nv,
                                const double* __restrict__ coef, int64_t n) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         double v = 0.0;
         for (int l = 0; l < nv; ++l) v = fma(coef[l], V[(size_t)l * stride + i], v);
-        y[i] = fma(beta, v, alpha * y[i]);
+        y[i] = alpha == 0.0 ? v : fma(alpha, y[i], v);
     }
-}
-
-// y *= c
-__global__ void scale_kernel(double* y, double c, int64_t n) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        y[i] *= c;
 }
 
 // Up to 8 terms with coefficients passed by value: y = sum_l c_l x_l.
@@ -189,6 +274,9 @@ bool sdirk_tableau_ok(const hho_tableau* tab) {
 // preconditioned vector
 struct SdirkWork {
     double *Z, *Y, *T, *W, *K, *V, *zero, *tr, *partial, *sums, *coef, *PZ;
+    double* inv;        // 1/||V_l||
+    double* norms;      // ||b||^2, ||r||^2
+    unsigned* ticket;
     int64_t n;
 };
 
@@ -214,19 +302,25 @@ int64_t sdirk_layout(const hho_ops* ops, int s, int m, SdirkWork* w, double* bas
     W.sums = take(2 * (m + 1) + 2);
     W.coef = take(m + 1);
     W.PZ = take(n);
+    // behind the partials in use (at most KR_MAX_BLOCKS per vector)
+    double* spare = W.partial ? W.partial + (int64_t)KR_MAX_BLOCKS * (m + 1) : nullptr;
+    W.inv = spare;
+    W.norms = spare ? spare + (m + 1) : nullptr;
+    W.ticket = spare ? (unsigned*)(spare + (m + 3)) : nullptr;
     if (w) *w = W;
     return off;
 }
 
-// out = v - a_dt J v (sources off), or out = J v + s(t) when rate is true
+// out = v - a_dt J v (sources off), or out = J v + s(t) when rate is true;
+// traced: the traces of v are in tr already
 void apply_op(hho_ops* ops, const double* v, double* out, double* tr, double a_dt, bool rate, double t,
-              cudaStream_t st) {
+              cudaStream_t st, bool traced = false) {
     StageArgsT<double> a;
     memset(&a, 0, sizeof(a));
     a.op = ops->dev;
     a.inp = v;
     a.tr_out = tr;
-    launch_stage_f64(ops, MODE_TRACES, a, 1, 0.0, -1, 0.0, false, st);
+    if (!traced) launch_stage_f64(ops, MODE_TRACES, a, 1, 0.0, -1, 0.0, false, st);
     a.tr_in = tr;
     a.tr_out = nullptr;
     a.n_tgt = 1;
@@ -378,24 +472,6 @@ __global__ void bj_invert_kernel(double* __restrict__ bj, const int32_t* __restr
     }
 }
 
-// y = P^-1 x (accumulate: y += P^-1 x); one thread per state entry (row r of
-// cell q at r N + q)
-__global__ void bj_apply_kernel(const double* __restrict__ bj, const double* __restrict__ x, double* __restrict__ y,
-                                int accumulate, int Nf, int Ns, int n) {
-    const int64_t nf = (int64_t)3 * n * Nf, tot = nf + (int64_t)5 * n * Ns;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
-        const bool fl = e < nf;
-        const int64_t e2 = fl ? e : e - nf;
-        const int N = fl ? Nf : Ns, nv = (fl ? 3 : 5) * n;
-        const int r = (int)(e2 / N), q = (int)(e2 % N);
-        const double* b = (fl ? bj : bj + (size_t)9 * n * n * Nf) + (size_t)r * nv * N + q;
-        const double* xb = (fl ? x : x + nf) + q;
-        double s = 0.0;
-        for (int c = 0; c < nv; ++c) s = fma(b[(size_t)c * N], xb[(size_t)c * N], s);
-        y[e] = accumulate ? y[e] + s : s;
-    }
-}
-
 // Builds (or reuses, for the same a* dt) the inverse blocks; scratch: x, y, tr.
 int build_block_jacobi(hho_ops* ops, double a_dt, double* x, double* y, double* tr, cudaStream_t st) {
     const int Nf = ops->dev.Nf, Ns = ops->dev.Ns, n = ops->n;
@@ -453,32 +529,86 @@ int build_block_jacobi(hho_ops* ops, double a_dt, double* x, double* y, double* 
     return HHO_OK;
 }
 
-// dst[l] = V_l . w for l < nv, on the device (no synchronisation)
-void dots_dev(const SdirkWork& W, const double* V, int nv, const double* w, double* dst, cudaStream_t st) {
-    multidot_kernel<<<RED_BLOCKS, RED_THREADS, 0, st>>>(V, W.n, nv, w, W.n, W.partial);
-    sum_partials_kernel<<<nv, RED_THREADS, 0, st>>>(W.partial, RED_BLOCKS, nv, dst);
+// Pinned host memory for a solve's sums and coefficients, and the event that
+// tells when the sums are there; kept with ops.
+int krylov_host(hho_ops* ops) {
+    if (!ops->h_krylov &&
+        cudaHostAlloc((void**)&ops->h_krylov, sizeof(double) * 4 * (MAX_RESTART + 2), cudaHostAllocDefault) !=
+            cudaSuccess) {
+        ops->h_krylov = nullptr;
+        hho_set_error("hho_sdirk_step: pinned host allocation failed");
+        return HHO_ENOMEM;
+    }
+    if (!ops->krylov_event) {
+        cudaEvent_t e;
+        if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
+            hho_set_error("hho_sdirk_step: event creation failed");
+            return HHO_ECUDA;
+        }
+        ops->krylov_event = (void*)e;
+    }
+    return HHO_OK;
 }
 
-// the same, copied to the host (synchronises)
-int dots(const SdirkWork& W, const double* V, int nv, const double* w, double* h, cudaStream_t st) {
-    dots_dev(W, V, nv, w, W.sums, st);
-    if (cudaMemcpyAsync(h, W.sums, sizeof(double) * nv, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess) {
+int fetch(hho_ops* ops, const double* d, double* h, int count, cudaStream_t st) {
+    if (cudaMemcpyAsync(h, d, sizeof(double) * count, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaEventRecord((cudaEvent_t)ops->krylov_event, st) != cudaSuccess) {
+        hho_set_error("hho_sdirk_step: reduction failed");
+        return HHO_ECUDA;
+    }
+    return HHO_OK;
+}
+int wait_sums(hho_ops* ops) {
+    if (cudaEventSynchronize((cudaEvent_t)ops->krylov_event) != cudaSuccess) {
         hho_set_error("hho_sdirk_step: reduction failed");
         return HHO_ECUDA;
     }
     return HHO_OK;
 }
 
-// y = alpha y + sum_l c[l] V_l with host coefficients (a copy from pageable
-// memory returns once the source is staged, so c may be reused at once)
-int combine(const SdirkWork& W, double* y, double alpha, const double* V, int nv, const double* c, cudaStream_t st) {
-    if (cudaMemcpyAsync(W.coef, c, sizeof(double) * nv, cudaMemcpyHostToDevice, st) != cudaSuccess) {
-        hho_set_error("hho_sdirk_step: coefficient upload failed");
-        return HHO_ECUDA;
+// Orthogonalises w against V_0..V_j (classical Gram-Schmidt twice): S1, S2 the
+// two sets of coefficients, *S3 = w . w afterwards and inv[j + 1] its factor.
+void orthogonalise(const SdirkWork& W, int j, double* w, double* S1, double* S2, double* S3, cudaStream_t st) {
+    KrylovArgs A;
+    A.stride = A.n = W.n;
+    A.w = w;
+    A.partial = W.partial;
+    A.ticket = W.ticket;
+    A.b = nullptr;
+    auto at = [&](int l0, const double* in, double* out) {
+        A.V = W.V + (size_t)l0 * W.n;
+        A.inv = W.inv + l0;
+        A.in = in ? in + l0 : nullptr;
+        A.out = out;
+        A.inv_out = nullptr;
+    };
+    const int nv = j + 1;
+    auto chunks = [&](auto f) {
+        for (int l0 = 0; l0 < nv; l0 += KR_CHUNK) f(l0, std::min(KR_CHUNK, nv - l0));
+    };
+    chunks([&](int l0, int c) {
+        at(l0, nullptr, S1 + l0);
+        krylov<KR_DOT>(c, A, st);
+    });
+    if (nv <= KR_CHUNK) {
+        at(0, S1, S2);
+        krylov<KR_UPDATE_DOT>(nv, A, st);
+    } else {
+        chunks([&](int l0, int c) {
+            at(l0, S1, nullptr);
+            krylov<KR_UPDATE>(c, A, st);
+        });
+        chunks([&](int l0, int c) {
+            at(l0, nullptr, S2 + l0);
+            krylov<KR_DOT>(c, A, st);
+        });
     }
-    lincomb_kernel<<<grid_for(W.n), 256, 0, st>>>(y, alpha, 1.0, V, W.n, nv, W.coef, W.n);
-    return HHO_OK;
+    chunks([&](int l0, int c) {
+        at(l0, S2, S3);
+        A.inv_out = W.inv + nv;
+        if (l0 + c < nv) krylov<KR_UPDATE>(c, A, st);
+        else krylov<KR_UPDATE_NORM>(c, A, st);
+    });
 }
 
 // Restarted GMRES for (I - a_dt J) x = b, x holding the initial guess; with
@@ -488,35 +618,60 @@ int combine(const SdirkWork& W, double* y, double alpha, const double* V, int nv
 // does not halve the true residual the remaining cycles run without the
 // preconditioner, which reaches the FP64 floor.  Adds its operator
 // applications to *its; HHO_ENOCONV if tol is missed.
+// The host needs a vector's sums only to decide whether to stop, so it queues
+// the operator on the next vector before it waits for them (the work of one
+// application is dropped when a solve ends inside a cycle).
 int gmres(hho_ops* ops, const SdirkWork& W, const double* b, double* x, double a_dt, double tol, int m,
           int max_iter, const double* bj, int64_t* its, cudaStream_t st) {
-    const int Nf = ops->dev.Nf, Ns = ops->dev.Ns, nn = ops->n;
-    double bn = 0.0;
-    int rc = dots(W, b, 1, b, &bn, st);
+    int rc = krylov_host(ops);
     if (rc) return rc;
-    bn = std::sqrt(bn);
-    if (bn == 0.0) {
-        cudaMemsetAsync(x, 0, sizeof(double) * W.n, st);
-        return HHO_OK;
-    }
-    std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m), hs(2 * (m + 1) + 1);
+    double* hs = ops->h_krylov;                              // S1, S2 (m + 1 each), S3
+    double* hn2 = hs + 2 * (MAX_RESTART + 1) + 1;            // ||b||^2, ||r||^2
+    double* hc = hn2 + 2;                                    // coefficients of the combination
+    double* S1 = W.sums;
+    double* S2 = W.sums + (m + 1);
+    double* S3 = W.sums + 2 * (m + 1);
+    const bool fused = bj_traces_fit(ops);
+    // V_{l + 1} = A P^-1 V_l / ||V_l||
+    auto apply_vector = [&](int l) {
+        launch_bj(ops, bj, W.V + (size_t)l * W.n, W.inv + l, W.PZ, false, fused ? W.tr : nullptr, (void*)st);
+        apply_op(ops, W.PZ, W.V + (size_t)(l + 1) * W.n, W.tr, a_dt, false, 0.0, st, fused);
+    };
+    KrylovArgs N;
+    N.V = W.W;
+    N.stride = N.n = W.n;
+    N.in = nullptr;
+    N.inv = W.inv;
+    N.partial = W.partial;
+    N.ticket = W.ticket;
+    N.b = b;
+    N.w = const_cast<double*>(b);
+    N.out = W.norms;
+    N.inv_out = nullptr;
+    krylov<KR_NORM>(1, N, st);
+    std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m), nrm(m + 1);
     int used = 0;
-    double rn = 0.0, rn_prev = 0.0;
-    while (true) {
+    double bn = 0.0, rn = 0.0, rn_prev = 0.0;
+    for (bool first = true;; first = false) {
         // r = b - A x into V_0; the true residual decides convergence
         apply_op(ops, x, W.W, W.tr, a_dt, false, 0.0, st);
         ++used;
-        Terms T;
-        T.n = 2;
-        T.x[0] = b;
-        T.c[0] = 1.0;
-        T.x[1] = W.W;
-        T.c[1] = -1.0;
-        terms_kernel<<<grid_for(W.n), 256, 0, st>>>(W.V, T, W.n);
-        double r2 = 0.0;
-        rc = dots(W, W.V, 1, W.V, &r2, st);
+        N.w = W.V;
+        N.out = W.norms + 1;
+        N.inv_out = W.inv;
+        krylov<KR_RESIDUAL>(1, N, st);
+        rc = fetch(ops, W.norms, hn2, 2, st);
         if (rc) return rc;
-        rn = std::sqrt(r2);
+        rc = wait_sums(ops);
+        if (rc) return rc;
+        if (first) {
+            bn = std::sqrt(hn2[0]);
+            if (bn == 0.0) {
+                cudaMemsetAsync(x, 0, sizeof(double) * W.n, st);
+                return HHO_OK;
+            }
+        }
+        rn = std::sqrt(hn2[1]);
         if (!std::isfinite(rn)) {
             hho_set_error("hho_sdirk_step: non-finite residual");
             return HHO_EUNSTABLE;
@@ -524,35 +679,20 @@ int gmres(hho_ops* ops, const SdirkWork& W, const double* b, double* x, double a
         if (rn <= tol * bn || used >= max_iter) break;
         if (bj && rn_prev > 0.0 && rn > 0.5 * rn_prev) bj = nullptr;   // stagnation: finish unpreconditioned
         rn_prev = rn;
-        scale_kernel<<<grid_for(W.n), 256, 0, st>>>(W.V, 1.0 / rn, W.n);
         std::fill(g.begin(), g.end(), 0.0);
-        g[0] = rn;
+        g[0] = nrm[0] = rn;
         int j = 0;
+        apply_vector(0);
         for (; j < m && used < max_iter; ++j) {
-            double* vj1 = W.V + (size_t)(j + 1) * W.n;
-            if (bj) {
-                bj_apply_kernel<<<grid_for(W.n), 256, 0, st>>>(bj, W.V + (size_t)j * W.n, W.PZ, 0, Nf, Ns, nn);
-                apply_op(ops, W.PZ, vj1, W.tr, a_dt, false, 0.0, st);
-            } else {
-                apply_op(ops, W.V + (size_t)j * W.n, vj1, W.tr, a_dt, false, 0.0, st);
-            }
             ++used;
-            // classical Gram-Schmidt twice, coefficients kept on the device
-            double* S1 = W.sums;
-            double* S2 = W.sums + (m + 1);
-            double* S3 = W.sums + 2 * (m + 1);
-            dots_dev(W, W.V, j + 1, vj1, S1, st);
-            lincomb_kernel<<<grid_for(W.n), 256, 0, st>>>(vj1, 1.0, -1.0, W.V, W.n, j + 1, S1, W.n);
-            dots_dev(W, W.V, j + 1, vj1, S2, st);
-            lincomb_kernel<<<grid_for(W.n), 256, 0, st>>>(vj1, 1.0, -1.0, W.V, W.n, j + 1, S2, W.n);
-            dots_dev(W, vj1, 1, vj1, S3, st);
-            if (cudaMemcpyAsync(hs.data(), W.sums, sizeof(double) * hs.size(), cudaMemcpyDeviceToHost, st) !=
-                    cudaSuccess ||
-                cudaStreamSynchronize(st) != cudaSuccess) {
-                hho_set_error("hho_sdirk_step: reduction failed");
-                return HHO_ECUDA;
-            }
+            orthogonalise(W, j, W.V + (size_t)(j + 1) * W.n, S1, S2, S3, st);
+            rc = fetch(ops, W.sums, hs, 2 * (m + 1) + 1, st);
+            if (rc) return rc;
+            if (j + 1 < m && used < max_iter) apply_vector(j + 1);
+            rc = wait_sums(ops);
+            if (rc) return rc;
             const double hn = std::sqrt(hs[2 * (m + 1)]);
+            nrm[j + 1] = hn;
             double* col = &H[(size_t)j * (m + 1)];
             for (int l = 0; l <= j; ++l) col[l] = hs[l] + hs[m + 1 + l];
             col[j + 1] = hn;
@@ -572,7 +712,6 @@ int gmres(hho_ops* ops, const SdirkWork& W, const double* b, double* x, double a
                 ++j;
                 break;
             }
-            scale_kernel<<<grid_for(W.n), 256, 0, st>>>(vj1, 1.0 / hn, W.n);
         }
         // x += V y with H y = g (upper triangular, j x j)
         for (int r = j - 1; r >= 0; --r) {
@@ -580,15 +719,18 @@ int gmres(hho_ops* ops, const SdirkWork& W, const double* b, double* x, double a
             for (int c2 = r + 1; c2 < j; ++c2) v -= H[(size_t)c2 * (m + 1) + r] * y[c2];
             y[r] = v / H[(size_t)r * (m + 1) + r];
         }
-        if (j > 0 && bj) {   // x += P^-1 (V y)
-            cudaMemsetAsync(W.W, 0, sizeof(double) * W.n, st);
-            rc = combine(W, W.W, 0.0, W.V, j, y.data(), st);
-            if (rc) return rc;
-            bj_apply_kernel<<<grid_for(W.n), 256, 0, st>>>(bj, W.W, x, 1, Nf, Ns, nn);
-        } else if (j > 0) {
-            rc = combine(W, x, 1.0, W.V, j, y.data(), st);
-            if (rc) return rc;
+        if (j > 0) {
+            // the previous copy from hc has run: a wait for sums came after it
+            for (int l = 0; l < j; ++l) hc[l] = y[l] / nrm[l];
+            if (cudaMemcpyAsync(W.coef, hc, sizeof(double) * j, cudaMemcpyHostToDevice, st) != cudaSuccess) {
+                hho_set_error("hho_sdirk_step: coefficient upload failed");
+                return HHO_ECUDA;
+            }
+            lincomb_kernel<<<grid_for(W.n), 256, 0, st>>>(bj ? W.W : x, bj ? 0.0 : 1.0, W.V, W.n, j, W.coef, W.n);
+            if (bj) launch_bj(ops, bj, W.W, nullptr, x, true, nullptr, (void*)st);   // x += P^-1 (V y)
         }
+        rc = check_cuda("hho_sdirk_step");
+        if (rc) return rc;
     }
     *its += used;
     if (rn > tol * bn) {

@@ -1567,7 +1567,8 @@ size_t stage_smem_bytes(int max_nf, int threads) {
 // warps; a warp lies in one class), y over shots; 128 threads.
 template <class T, int K, int MODE>
 __global__ void __launch_bounds__(128, MinBlocks<T, K>::value) stage_kernel(const StageArgsT<T> A) {
-    const int gq = blockIdx.x * blockDim.x + threadIdx.x;
+    // the last cells first: solid cells are the longer ones and should not make the tail
+    const int gq = (gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x;
     const int shot = blockIdx.y;
     const T* cd = nullptr;
     extern __shared__ __align__(16) unsigned char stage_smem[];
@@ -1601,7 +1602,7 @@ template <class T, int K>
 __global__ void __launch_bounds__(128, MinBlocks<T, K>::value)
     grad_stage_kernel(const StageArgsT<T> A, const GradArgsT<T> G) {
     extern __shared__ __align__(16) unsigned char stage_smem[];
-    const int gq = blockIdx.x * blockDim.x + threadIdx.x;
+    const int gq = (gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x;   // solid cells first, as stage_kernel
     T* acc = nullptr;
     if constexpr (AccSmem<T, K>::value) acc = reinterpret_cast<T*>(stage_smem) + threadIdx.x * acc_stride<K>();
     if (gq < A.op.Nf)

@@ -81,10 +81,143 @@ __device__ __forceinline__ void team_jump(const StageArgsT<T>& A, const T* trf, 
     }
 }
 
+// What publishing the traces of 32 cells needs (uniform but for lq and tau).
+template <class T>
+struct TeamFaces {
+    int nF, npad, sbase, kind, lq;
+    uint32_t hor, other;   // horizontal faces; faces that are neither horizontal nor vertical
+    const T* cd;           // the class's face blocks in shared memory
+    T tau;
+    bool real;
+};
+
+// Publishes w and omega of the cells' state V (rows of 32, this lane's column)
+// into the trace buffer `tr`: warp w takes (face, coefficient) pairs w, w + W, ...
+template <class T, int K, int W, bool SOLID>
+__device__ __forceinline__ void team_traces(const DevOps& op, const TeamFaces<T>& F, const T* V, T* tr, int w) {
+    constexpr int n = Dims<K>::n, f = Dims<K>::f, FS = Dims<K>::FS, TR = Dims<K>::TR, nP = Dims<K>::nP;
+    constexpr int NC = SOLID ? 2 : 1;
+    T* out = tr + (SOLID ? (size_t)2 * f * op.SF : 0);
+    const size_t S = SOLID ? op.SS : op.SF;
+    for (int it = w; it < F.nF * f; it += W) {
+        const int j = it / f, l = it - j * f;
+        const T* fm = F.cd + j * FS;
+        const T* row = fm + TR + l * nP;
+        const int slot = F.sbase + j * F.npad + F.lq;
+        const int nb = __ldg((SOLID ? op.nb_s : op.nb_f) + slot);
+        const T be = __ldg((SOLID ? OpData<T>::beta_s(op) : OpData<T>::beta_f(op)) + slot);
+        T u[NC], g[NC];   // traces of the primal field and of the normal flux
+#pragma unroll
+        for (int c = 0; c < NC; ++c) u[c] = g[c] = T(0);
+        if ((F.other >> j) & 1) {
+            const T nx = fm[0], ny = fm[1];
+            T m0(0), m1(0), m2(0);   // m_x, m_y or s_xx, s_yy, s_xy
+#pragma unroll 1
+            for (int i = 0; i < n; ++i) {
+                const T v = row[i];
+                const T* P = V + 32 * i;
+#pragma unroll
+                for (int c = 0; c < NC; ++c) u[c] = fma(v, P[32 * (SOLID ? 3 + c : 2) * n], u[c]);
+                if constexpr (Fp64Form<T>::value) {
+                    m0 = fma(v, P[0], m0);
+                    m1 = fma(v, P[32 * n], m1);
+                    if constexpr (SOLID) m2 = fma(v, P[32 * 2 * n], m2);
+                } else if constexpr (SOLID) {   // the flux's coefficients first, as the thread form
+                    const T xy = P[32 * 2 * n];
+                    g[0] = fma(v, fma(nx, P[0], mul_rn(ny, xy)), g[0]);
+                    g[1] = fma(v, fma(nx, xy, mul_rn(ny, P[32 * n])), g[1]);
+                } else {
+                    g[0] = fma(v, fma(nx, P[0], mul_rn(ny, P[32 * n])), g[0]);
+                }
+            }
+            if constexpr (Fp64Form<T>::value && SOLID) {
+                g[0] = fma(nx, m0, mul_rn(ny, m2));
+                g[1] = fma(nx, m2, mul_rn(ny, m1));
+            } else if constexpr (Fp64Form<T>::value) {
+                g[0] = fma(nx, m0, mul_rn(ny, m1));
+            }
+        } else {
+            // on a horizontal face (fixed Y) the monomial (a, b) has coefficients l <= a; l = a only on a rectangle,
+            // whose centroid the face is centred on; likewise b on a vertical face
+            const bool hor = (F.hor >> j) & 1;
+            const bool neg = is_negative(fm[hor ? 1 : 0]);
+            const T* F0 = V + 32 * (SOLID ? (hor ? 2 : 0) * n : (hor ? n : 0));   // s_xy / s_xx, m_y / m_x
+            const T* F1 = V + 32 * (hor ? n : 2 * n);                             // s_yy / s_xy
+            // values of the monomial with exponents l along and e across the face
+            auto idx = [&](int e) { return (l + e) * (l + e + 1) / 2 + (hor ? e : l); };
+            if (F.kind == KIND_SQUARE) {                    // Horner in +-rho0, see trace_square
+                const T rho = signed_face_rho<T>(j == 1 || j == 2 ? 1 : -1);
+                int i = idx(K - l);
+#pragma unroll
+                for (int c = 0; c < NC; ++c) u[c] = V[32 * ((SOLID ? 3 + c : 2) * n + i)];
+                g[0] = F0[32 * i];
+                if constexpr (SOLID) g[1] = F1[32 * i];
+#pragma unroll 1
+                for (int e = K - l - 1; e >= 0; --e) {
+                    i = idx(e);
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) u[c] = fma(rho, u[c], V[32 * ((SOLID ? 3 + c : 2) * n + i)]);
+                    g[0] = fma(rho, g[0], F0[32 * i]);
+                    if constexpr (SOLID) g[1] = fma(rho, g[1], F1[32 * i]);
+                }
+                if ((l & 1) && j >= 2) {                  // s_t = -1 on faces 2 and 3
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        u[c] = -u[c];
+                        g[c] = -g[c];
+                    }
+                }
+            } else {
+                auto add = [&](int i) {
+                    const T v = row[i];
+                    const T* P = V + 32 * i;
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) u[c] = fma(v, P[32 * (SOLID ? 3 + c : 2) * n], u[c]);
+                    g[0] = fma(v, F0[32 * i], g[0]);
+                    if constexpr (SOLID) g[1] = fma(v, F1[32 * i], g[1]);
+                };
+                if (F.kind != KIND_GENERIC) {
+#pragma unroll 1
+                    for (int e = 0; e <= K - l; ++e) add(idx(e));
+                } else {
+#pragma unroll 1
+                    for (int dgr = l; dgr <= K; ++dgr)    // by degree, the order of the basis
+#pragma unroll 1
+                        for (int b = hor ? 0 : l; b <= (hor ? dgr - l : dgr); ++b) add(dgr * (dgr + 1) / 2 + b);
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < NC; ++c) g[c] = neg ? -g[c] : g[c];
+        }
+        T wv[NC], om[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) wv[c] = fma(F.tau, u[c], -g[c]);
+        if (nb >= NB_BOUNDARY) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) om[c] = fma(be, wv[c], -u[c]);
+        } else {
+            const T* co = OpData<T>::if_coef(op) + 6 * (-2 - nb);
+            if constexpr (SOLID) {
+                om[0] = fma(__ldg(co), wv[0], fma(__ldg(co + 1), wv[1], -u[0]));
+                om[1] = fma(__ldg(co + 2), wv[0], fma(__ldg(co + 3), wv[1], -u[1]));
+            } else {
+                om[0] = fma(__ldg(co), wv[0], -u[0]);
+            }
+        }
+        if (F.real) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                out[(size_t)(c * f + l) * S + slot] = norm(wv[c]);
+                out[(size_t)((NC + c) * f + l) * S + slot] = norm(om[c]);
+            }
+        }
+    }
+}
+
 template <class T, int K, int MODE, int W, bool SOLID>
 __device__ __forceinline__ void team_cells(const StageArgsT<T>& A, int gw, int shot, T* smem) {
-    constexpr int n = Dims<K>::n, f = Dims<K>::f, FS = Dims<K>::FS, TR = Dims<K>::TR, LI = Dims<K>::LI;
-    constexpr int nP = Dims<K>::nP, fP = Dims<K>::fP;
+    constexpr int n = Dims<K>::n, f = Dims<K>::f, FS = Dims<K>::FS, LI = Dims<K>::LI;
+    constexpr int fP = Dims<K>::fP;
     constexpr int NV = SOLID ? 5 * n : 3 * n, NC = SOLID ? 2 : 1;
     const DevOps& op = A.op;
     const int lane = threadIdx.x & 31;
@@ -311,121 +444,18 @@ __device__ __forceinline__ void team_cells(const StageArgsT<T>& A, int gw, int s
         __syncthreads();
     }
     // ---- 3. traces: coefficient l on face j ---------------------------------------------
-    T* out = A.tr_out + toff + (SOLID ? (size_t)2 * f * op.SF : 0);
-    const size_t S = SOLID ? op.SS : op.SF;
-    for (int it = w; it < nF * f; it += W) {
-        const int j = it / f, l = it - j * f;
-        const T* fm = cd + j * FS;
-        const T* row = fm + TR + l * nP;
-        const int slot = sbase + j * npad + lq;
-        const int nb = __ldg((SOLID ? op.nb_s : op.nb_f) + slot);
-        const T be = __ldg((SOLID ? OpData<T>::beta_s(op) : OpData<T>::beta_f(op)) + slot);
-        T u[NC], g[NC];   // traces of the primal field and of the normal flux
-#pragma unroll
-        for (int c = 0; c < NC; ++c) u[c] = g[c] = T(0);
-        if ((faces_g >> j) & 1) {
-            const T nx = fm[0], ny = fm[1];
-            T m0(0), m1(0), m2(0);   // m_x, m_y or s_xx, s_yy, s_xy
-#pragma unroll 1
-            for (int i = 0; i < n; ++i) {
-                const T v = row[i];
-                const T* P = V + 32 * i;
-#pragma unroll
-                for (int c = 0; c < NC; ++c) u[c] = fma(v, P[32 * (SOLID ? 3 + c : 2) * n], u[c]);
-                if constexpr (Fp64Form<T>::value) {
-                    m0 = fma(v, P[0], m0);
-                    m1 = fma(v, P[32 * n], m1);
-                    if constexpr (SOLID) m2 = fma(v, P[32 * 2 * n], m2);
-                } else if constexpr (SOLID) {   // the flux's coefficients first, as the thread form
-                    const T xy = P[32 * 2 * n];
-                    g[0] = fma(v, fma(nx, P[0], mul_rn(ny, xy)), g[0]);
-                    g[1] = fma(v, fma(nx, xy, mul_rn(ny, P[32 * n])), g[1]);
-                } else {
-                    g[0] = fma(v, fma(nx, P[0], mul_rn(ny, P[32 * n])), g[0]);
-                }
-            }
-            if constexpr (Fp64Form<T>::value && SOLID) {
-                g[0] = fma(nx, m0, mul_rn(ny, m2));
-                g[1] = fma(nx, m2, mul_rn(ny, m1));
-            } else if constexpr (Fp64Form<T>::value) {
-                g[0] = fma(nx, m0, mul_rn(ny, m1));
-            }
-        } else {
-            // on a horizontal face (fixed Y) the monomial (a, b) has coefficients l <= a; l = a only on a rectangle,
-            // whose centroid the face is centred on; likewise b on a vertical face
-            const bool hor = (faces_h >> j) & 1;
-            const bool neg = is_negative(fm[hor ? 1 : 0]);
-            const T* F0 = V + 32 * (SOLID ? (hor ? 2 : 0) * n : (hor ? n : 0));   // s_xy / s_xx, m_y / m_x
-            const T* F1 = V + 32 * (hor ? n : 2 * n);                             // s_yy / s_xy
-            // values of the monomial with exponents l along and e across the face
-            auto idx = [&](int e) { return (l + e) * (l + e + 1) / 2 + (hor ? e : l); };
-            if (kind == KIND_SQUARE) {                    // Horner in +-rho0, see trace_square
-                const T rho = signed_face_rho<T>(j == 1 || j == 2 ? 1 : -1);
-                int i = idx(K - l);
-#pragma unroll
-                for (int c = 0; c < NC; ++c) u[c] = V[32 * ((SOLID ? 3 + c : 2) * n + i)];
-                g[0] = F0[32 * i];
-                if constexpr (SOLID) g[1] = F1[32 * i];
-#pragma unroll 1
-                for (int e = K - l - 1; e >= 0; --e) {
-                    i = idx(e);
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) u[c] = fma(rho, u[c], V[32 * ((SOLID ? 3 + c : 2) * n + i)]);
-                    g[0] = fma(rho, g[0], F0[32 * i]);
-                    if constexpr (SOLID) g[1] = fma(rho, g[1], F1[32 * i]);
-                }
-                if ((l & 1) && j >= 2) {                  // s_t = -1 on faces 2 and 3
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        u[c] = -u[c];
-                        g[c] = -g[c];
-                    }
-                }
-            } else {
-                auto add = [&](int i) {
-                    const T v = row[i];
-                    const T* P = V + 32 * i;
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) u[c] = fma(v, P[32 * (SOLID ? 3 + c : 2) * n], u[c]);
-                    g[0] = fma(v, F0[32 * i], g[0]);
-                    if constexpr (SOLID) g[1] = fma(v, F1[32 * i], g[1]);
-                };
-                if (rect) {
-#pragma unroll 1
-                    for (int e = 0; e <= K - l; ++e) add(idx(e));
-                } else {
-#pragma unroll 1
-                    for (int dgr = l; dgr <= K; ++dgr)    // by degree, the order of the basis
-#pragma unroll 1
-                        for (int b = hor ? 0 : l; b <= (hor ? dgr - l : dgr); ++b) add(dgr * (dgr + 1) / 2 + b);
-                }
-            }
-#pragma unroll
-            for (int c = 0; c < NC; ++c) g[c] = neg ? -g[c] : g[c];
-        }
-        T wv[NC], om[NC];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) wv[c] = fma(tau, u[c], -g[c]);
-        if (nb >= NB_BOUNDARY) {
-#pragma unroll
-            for (int c = 0; c < NC; ++c) om[c] = fma(be, wv[c], -u[c]);
-        } else {
-            const T* co = OpData<T>::if_coef(op) + 6 * (-2 - nb);
-            if constexpr (SOLID) {
-                om[0] = fma(__ldg(co), wv[0], fma(__ldg(co + 1), wv[1], -u[0]));
-                om[1] = fma(__ldg(co + 2), wv[0], fma(__ldg(co + 3), wv[1], -u[1]));
-            } else {
-                om[0] = fma(__ldg(co), wv[0], -u[0]);
-            }
-        }
-        if (real) {
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                out[(size_t)(c * f + l) * S + slot] = norm(wv[c]);
-                out[(size_t)((NC + c) * f + l) * S + slot] = norm(om[c]);
-            }
-        }
-    }
+    TeamFaces<T> F;
+    F.nF = nF;
+    F.npad = npad;
+    F.sbase = sbase;
+    F.kind = kind;
+    F.lq = lq;
+    F.hor = faces_h;
+    F.other = faces_g;
+    F.cd = cd;
+    F.tau = tau;
+    F.real = real;
+    team_traces<T, K, W, SOLID>(op, F, V, A.tr_out + toff, w);
 }
 
 // Grid: x over the warps of cells of both domains (fluid, then solid), y over shots.
@@ -433,6 +463,7 @@ template <class T, int K, int MODE, int W>
 __global__ void __launch_bounds__(32 * W, 32 / W) team_kernel(const StageArgsT<T> A) {
     extern __shared__ __align__(16) unsigned char stage_smem[];
     T* smem = reinterpret_cast<T*>(stage_smem);
-    if ((int)blockIdx.x < A.op.n_warps_f) team_cells<T, K, MODE, W, false>(A, blockIdx.x, blockIdx.y, smem);
-    else team_cells<T, K, MODE, W, true>(A, blockIdx.x, blockIdx.y, smem);
+    const int gw = gridDim.x - 1 - blockIdx.x;   // solid cells, the longer ones, first
+    if (gw < A.op.n_warps_f) team_cells<T, K, MODE, W, false>(A, gw, blockIdx.y, smem);
+    else team_cells<T, K, MODE, W, true>(A, gw, blockIdx.y, smem);
 }
