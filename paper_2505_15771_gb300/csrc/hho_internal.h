@@ -123,6 +123,8 @@ constexpr int MAX_SOURCES = 8;
 struct StageClock {
     double t0;
     int64_t step;
+    uint32_t ticket;   // blocks of the receiver kernel that have read the step
+    uint32_t pad;
 };
 
 template <class T>

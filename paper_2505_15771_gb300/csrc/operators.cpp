@@ -875,7 +875,7 @@ extern "C" int hho_operators_build_tau(const hho_mesh* m, int32_t k, const doubl
     D.n_warps_f = Nf / 32;
     D.n_warps_s = Ns / 32;
     {
-        std::vector<StageClock> clk(1, StageClock{0.0, 0});
+        std::vector<StageClock> clk(1, StageClock{0.0, 0, 0, 0});
         ops->d_clock = dev_upload(ops, clk, &err);
     }
     D.n_warps_rect = 0;

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "basis.h"
+#include "dependent_launch.cuh"
 #include "f2x.cuh"
 #include "hho_internal.h"
 #include "stage_launch.h"
@@ -235,55 +236,77 @@ __global__ void sum_kernel(const double* __restrict__ partial, int np, double* o
 
 // Receivers: fluid [p, m_x, m_y, 0, 0]; solid [v_x, v_y, s_xx, s_yy, s_xy];
 // interface [p_F, v_Fx, v_Fy, 0, 0] from the pointwise face solve.
-// y = shot: state shot stride n_state, output shot stride 5 n_rec.
+// One block a receiver (y = shot): thread (field, i) fetches a coefficient, one
+// thread a field adds them up, then one thread an output.  The chain of loads is
+// two long, and FP64 instructions, 64 cycles each to a warp, are issued for all
+// fields at once (one thread a receiver took 7.3 us for the eight interface
+// receivers of the academic run, a sixth of its step).  State shot stride
+// n_state, output shot stride 5 n_rec; with a device clock (graph replay) out is
+// the trace base, offset by the step, and the last block to have read the step
+// advances it.
+constexpr int REC_FIELDS = 8;   // three of the fluid cell, five of the solid cell
+constexpr int REC_MAX_N = 10;
+inline int record_threads(int n) { return (REC_FIELDS * n + 31) / 32 * 32; }
 template <class T, class TO = T>
 __global__ void record_kernel(DevOps op, int n_rec, const int32_t* __restrict__ ri, const double* __restrict__ rd,
-                              const T* __restrict__ state, int64_t n_state, TO* out,
-                              const StageClock* clock = nullptr) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n_rec) return;
-    const int n = op.n;
-    const int stride = 2 * n + 15;
-    const double* d = rd + (size_t)r * stride;
+                              const T* __restrict__ state, int64_t n_state, TO* out, StageClock* clock = nullptr) {
+    __shared__ double val[REC_FIELDS][REC_MAX_N], field[REC_FIELDS], flux[3];
+    const int r = blockIdx.x, n = op.n, t = threadIdx.x;
+    const double* d = rd + (size_t)r * (2 * n + 15);
     const int kind = ri[4 * r], qf = ri[4 * r + 1], qs = ri[4 * r + 2];
+    const int fld = t / n, i = t - fld * n;   // 0..2 fluid m_x, m_y, p; 3..7 solid s_xx, s_yy, s_xy, v_x, v_y
+    release_successor();
+    wait_for_predecessor();
     const T* sf = state + (size_t)blockIdx.y * n_state;
     const T* ss = sf + (size_t)3 * n * op.Nf;
-    auto ev = [&](const T* base, int N, int q, int field, const double* phi) {
+    if (fld < 3 && kind != 1) val[fld][i] = double(sf[(size_t)(fld * n + i) * op.Nf + qf]);
+    if (fld >= 3 && fld < REC_FIELDS && kind != 0) val[fld][i] = double(ss[(size_t)((fld - 3) * n + i) * op.Ns + qs]);
+    int64_t step = 0;
+    if (clock && t == 0) {
+        step = *(volatile int64_t*)&clock->step;
+        if (atomicAdd(&clock->ticket, 1u) == gridDim.x * gridDim.y - 1) {   // every block has read it
+            clock->ticket = 0;
+            clock->step = step + 1;
+        }
+    }
+    __shared__ int64_t step_sh;
+    if (t == 0) step_sh = step;
+    __syncthreads();
+    if (t < REC_FIELDS) {
+        const double* phi = kind == 2 && t >= 3 ? d + n : d;
         double s = 0.0;
-        for (int i = 0; i < n; ++i) s = fma(phi[i], double(base[(size_t)(field * n + i) * N + q]), s);
-        return s;
-    };
-    double o[5] = {0, 0, 0, 0, 0};
-    if (kind == 0) {
-        o[0] = ev(sf, op.Nf, qf, 2, d);
-        o[1] = ev(sf, op.Nf, qf, 0, d);
-        o[2] = ev(sf, op.Nf, qf, 1, d);
-    } else if (kind == 1) {
-        o[0] = ev(ss, op.Ns, qs, 3, d);
-        o[1] = ev(ss, op.Ns, qs, 4, d);
-        o[2] = ev(ss, op.Ns, qs, 0, d);
-        o[3] = ev(ss, op.Ns, qs, 1, d);
-        o[4] = ev(ss, op.Ns, qs, 2, d);
-    } else {
-        const double* pf = d;
-        const double* ps = d + n;
+        if (kind == 2 || (t >= 3) == (kind == 1))
+            for (int j = 0; j < n; ++j) s = fma(phi[j], val[t][j], s);
+        field[t] = s;
+    }
+    __syncthreads();
+    const double* g = field;
+    if (kind == 2 && t < 3) {   // tau_f p - m.n_f, tau_s v - s n_s
         const double tf = d[2 * n], ts = d[2 * n + 1];
         const double nfx = d[2 * n + 2], nfy = d[2 * n + 3], nsx = d[2 * n + 4], nsy = d[2 * n + 5];
-        const double* Ai = d + 2 * n + 6;
-        const double p = ev(sf, op.Nf, qf, 2, pf), mx = ev(sf, op.Nf, qf, 0, pf), my = ev(sf, op.Nf, qf, 1, pf);
-        const double sxx = ev(ss, op.Ns, qs, 0, ps), syy = ev(ss, op.Ns, qs, 1, ps), sxy = ev(ss, op.Ns, qs, 2, ps);
-        const double vx = ev(ss, op.Ns, qs, 3, ps), vy = ev(ss, op.Ns, qs, 4, ps);
-        const double wf = tf * p - (mx * nfx + my * nfy);
-        const double wsx = ts * vx - (sxx * nsx + sxy * nsy);
-        const double wsy = ts * vy - (sxy * nsx + syy * nsy);
-        o[0] = Ai[0] * wf + Ai[1] * wsx + Ai[2] * wsy;
-        o[1] = Ai[3] * wf + Ai[4] * wsx + Ai[5] * wsy;
-        o[2] = Ai[6] * wf + Ai[7] * wsx + Ai[8] * wsy;
+        flux[t] = t == 0   ? tf * g[2] - (g[0] * nfx + g[1] * nfy)
+                  : t == 1 ? ts * g[6] - (g[3] * nsx + g[5] * nsy)
+                           : ts * g[7] - (g[5] * nsx + g[4] * nsy);
     }
-    // with a device clock (graph replay) out is the trace base, offset by the step
-    if (clock) out += (size_t)clock->step * 5 * n_rec * gridDim.y;
-    TO* ob = out + (size_t)blockIdx.y * 5 * n_rec + 5 * r;
-    for (int j = 0; j < 5; ++j) ob[j] = TO(o[j]);
+    __syncthreads();
+    if (t >= 5) return;
+    double o = 0.0;
+    if (kind == 0) {
+        if (t < 3) o = g[t == 0 ? 2 : t - 1];
+    } else if (kind == 1) {
+        o = g[t < 2 ? 6 + t : 1 + t];
+    } else if (t < 3) {
+        const double* Ai = d + 2 * n + 6 + 3 * t;
+        o = Ai[0] * flux[0] + Ai[1] * flux[1] + Ai[2] * flux[2];
+    }
+    if (clock) out += (size_t)step_sh * 5 * n_rec * gridDim.y;
+    out[(size_t)blockIdx.y * 5 * n_rec + 5 * r + t] = TO(o);
+}
+
+template <class T, class TO>
+void launch_record(const hho_ops* ops, int n_shots, const T* state, TO* out, StageClock* clock, cudaStream_t st) {
+    launch_dependent(record_kernel<T, TO>, dim3(ops->n_rec, n_shots), record_threads(ops->n), 0, st, ops->dev, ops->n_rec,
+                     ops->d_rec_int, ops->d_rec_dbl, state, ops->n_state, out, clock);
 }
 
 template <class T, int MODE>
@@ -450,6 +473,7 @@ namespace {
 __global__ void clock_set_kernel(StageClock* c, double t0) {
     c->t0 = t0;
     c->step = 0;
+    c->ticket = 0;
 }
 __global__ void clock_advance_kernel(StageClock* c) { c->step += 1; }
 
@@ -547,7 +571,6 @@ static int erk_run(hho_ops* ops, const hho_tableau* tab, double t0, double dt, i
         rc = check_launch(who);
         if (rc) return rc;
         const bool rec = d_seis && ops->n_rec > 0;
-        const dim3 rgrid((ops->n_rec + 63) / 64, n_shots);
         cudaGraphExec_t execs[2] = {nullptr, nullptr};
         for (int par = 0; par < ((tab->s & 1) ? 2 : 1); ++par) {
             std::vector<StageArgsT<T>> args(tab->s);
@@ -596,10 +619,10 @@ static int erk_run(hho_ops* ops, const hho_tableau* tab, double t0, double dt, i
                     return HHO_ECUDA;
                 }
                 for (int j = 0; j < tab->s; ++j) launch_stage<T, MODE_STAGE>(ops, args[j], n_shots, cs);
-                if (rec)
-                    record_kernel<T, TS><<<rgrid, 64, 0, cs>>>(ops->dev, ops->n_rec, ops->d_rec_int, ops->d_rec_dbl,
-                                                             d_state, ops->n_state, d_seis, ops->d_clock);
-                clock_advance_kernel<<<1, 1, 0, cs>>>(ops->d_clock);
+                if (rec)   // advances the clock too
+                    launch_record<T, TS>(ops, n_shots, d_state, d_seis, ops->d_clock, cs);
+                else
+                    clock_advance_kernel<<<1, 1, 0, cs>>>(ops->d_clock);
                 const cudaError_t ce = cudaStreamEndCapture(cs, &graph);
                 if (ce != cudaSuccess || !graph || cudaGraphInstantiate(&found, graph, 0) != cudaSuccess) {
                     if (graph) cudaGraphDestroy(graph);
@@ -647,9 +670,7 @@ static int erk_run(hho_ops* ops, const hho_tableau* tab, double t0, double dt, i
             cur ^= 1;
         }
         if (d_seis && ops->n_rec > 0) {
-            record_kernel<T, TS><<<dim3((ops->n_rec + 63) / 64, n_shots), 64, 0, st>>>(
-                ops->dev, ops->n_rec, ops->d_rec_int, ops->d_rec_dbl, d_state, ops->n_state,
-                d_seis + (size_t)step * 5 * ops->n_rec * n_shots);
+            launch_record<T, TS>(ops, n_shots, d_state, d_seis + (size_t)step * 5 * ops->n_rec * n_shots, nullptr, st);
             rc = check_launch(who);
             if (rc) return rc;
         }
@@ -1262,8 +1283,7 @@ extern "C" int hho_record(hho_ops* ops, const double* d_state, double* d_out, vo
         return HHO_EINVAL;
     }
     if (ops->n_rec == 0) return HHO_OK;
-    record_kernel<double><<<dim3((ops->n_rec + 63) / 64, 1), 64, 0, (cudaStream_t)stream>>>(
-        ops->dev, ops->n_rec, ops->d_rec_int, ops->d_rec_dbl, d_state, ops->n_state, d_out);
+    launch_record<double, double>(ops, 1, d_state, d_out, nullptr, (cudaStream_t)stream);
     return check_launch("hho_record");
 }
 
@@ -1526,8 +1546,7 @@ int erk_steps_f32(hho_ops* ops, const hho_tableau* tab, double t0, double dt, in
 
 void launch_record_f64(const hho_ops* ops, const double* state, double* out, void* stream) {
     if (ops->n_rec == 0) return;
-    record_kernel<double><<<dim3((ops->n_rec + 63) / 64, 1), 64, 0, (cudaStream_t)stream>>>(
-        ops->dev, ops->n_rec, ops->d_rec_int, ops->d_rec_dbl, state, ops->n_state, out);
+    launch_record<double, double>(ops, 1, state, out, nullptr, (cudaStream_t)stream);
 }
 
 int check_cuda(const char* what) { return check_launch(what); }

@@ -40,6 +40,7 @@
 #include <type_traits>
 
 #include "basis.h"
+#include "dependent_launch.cuh"
 #include "f2x.cuh"
 #include "hho_internal.h"
 #include "stage_launch.h"
@@ -1570,6 +1571,7 @@ __global__ void __launch_bounds__(128, MinBlocks<T, K>::value) stage_kernel(cons
     // the last cells first: solid cells are the longer ones and should not make the tail
     const int gq = (gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x;
     const int shot = blockIdx.y;
+    wait_for_predecessor();
     const T* cd = nullptr;
     extern __shared__ __align__(16) unsigned char stage_smem[];
     T* acc = nullptr;
@@ -1706,14 +1708,14 @@ void launch_stage(const StageArgsT<T>& a, int n_shots, cudaStream_t s) {
         constexpr int TW = decltype(wc)::value;
         const size_t smem = sizeof(T) * team_smem_elems<T, K>(a.op.max_nf);
         stage_smem_attributes<TeamTag<T, K, MODE, TW>>(team_kernel<T, K, MODE, TW>, smem, true);
-        team_kernel<T, K, MODE, TW><<<dim3(a.op.n_warps_f + a.op.n_warps_s, n_shots), 32 * TW, smem, s>>>(a);
+        launch_dependent(team_kernel<T, K, MODE, TW>, dim3(a.op.n_warps_f + a.op.n_warps_s, n_shots), 32 * TW, smem, s, a);
     };
     if (W == 4) return team(std::integral_constant<int, 4>());
     if (W) return team(std::integral_constant<int, TeamRule<T, K>::W>());
     const int cells = a.op.Nf + a.op.Ns, threads = stage_threads((int64_t)(cells / 32) * n_shots);
     const size_t smem = stage_smem_bytes<T, K>(a.op.max_nf, threads);
     stage_smem_attributes<StageTag<T, K, MODE>>(stage_kernel<T, K, MODE>, smem, AccSmem<T, K>::value);
-    stage_kernel<T, K, MODE><<<dim3((cells + threads - 1) / threads, n_shots), threads, smem, s>>>(a);
+    launch_dependent(stage_kernel<T, K, MODE>, dim3((cells + threads - 1) / threads, n_shots), threads, smem, s, a);
 }
 
 template <class T, int K>

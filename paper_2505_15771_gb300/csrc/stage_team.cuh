@@ -251,6 +251,7 @@ __device__ __forceinline__ void team_cells(const StageArgsT<T>& A, int gw, int s
     const uint32_t faces_h = (uint32_t)__ldg(ci + CI_HOR), faces_v = (uint32_t)__ldg(ci + CI_VER);
     const uint32_t faces_g = (nF >= 32 ? 0xffffffffu : (1u << nF) - 1u) & ~(faces_h | faces_v);
     const T* inp = A.inp + soff + q;
+    wait_for_predecessor();   // so far: operator data only
     if constexpr (MODE == MODE_TRACES) {
         for (int i = w; i < NV; i += W) V[32 * i] = inp[(size_t)i * N];
         __syncthreads();
@@ -444,6 +445,10 @@ __device__ __forceinline__ void team_cells(const StageArgsT<T>& A, int gw, int s
         __syncthreads();
     }
     // ---- 3. traces: coefficient l on face j ---------------------------------------------
+    // The next stage's blocks may come in where they find idle SMs.  On a fuller
+    // GPU they would be placed while this stage still holds its share, unevenly
+    // (20 % of a stage at 400 groups), so there they come as blocks leave.
+    if (gridDim.x * gridDim.y <= 76) release_successor();
     TeamFaces<T> F;
     F.nF = nF;
     F.npad = npad;
