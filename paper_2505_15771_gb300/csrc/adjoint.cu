@@ -74,59 +74,63 @@ __global__ void axpby_kernel(int64_t n, double a, const T* x, double b, const T*
     }
 }
 
-// d(G^T d)/dtau of the interface receivers at one time node.  Such a
+// d(G^T d)/dtau of an interface receiver at one time node.  Such a
 // receiver records [p_F, v_F] = Ai w at its point, w = (tau_f p - m.n_f,
 // tau_s v - s n_s) from the two cells' values there and A = [tau_f, n^T;
 // -n, tau_s I]; so dd/dtau_f = Ai e_0 (p - p_F) and dd/dtau_s = Ai [0; v - v_F].
 // grec[2r] (the fluid cell's tau) and grec[2r + 1] (the solid cell's) sum
-// these over the time nodes; other receivers do not depend on tau.
+// these over the time nodes; other receivers do not depend on tau.  One block a
+// receiver, the eight field values by eight threads (as record_kernel).
 template <class T>
-__device__ __forceinline__ void rec_tau(const DevOps& op, int r, int n_rec, const int32_t* __restrict__ ri,
+__device__ __forceinline__ void rec_tau(const DevOps& op, int r, const int32_t* __restrict__ ri,
                                         const double* __restrict__ rd, const T* __restrict__ state,
                                         const T* __restrict__ G, double* __restrict__ grec) {
-    if (r >= n_rec || ri[4 * r] != 2) return;
-    const int n = op.n;
+    __shared__ double val[8][10], g[8], w[3], o[3], hg[3];
+    if (ri[4 * r] != 2) return;
+    const int n = op.n, t = threadIdx.x;
     const double* d = rd + (size_t)r * (2 * n + 15);
     const int qf = ri[4 * r + 1], qs = ri[4 * r + 2];
-    const T* sf = state;
     const T* ss = state + (size_t)3 * n * op.Nf;
-    auto ev = [&](const T* base, int N, int q, int field, const double* phi) {
-        double v = 0.0;
-        for (int i = 0; i < n; ++i) v = fma(phi[i], (double)base[(size_t)(field * n + i) * N + q], v);
-        return v;
-    };
-    const double* pf = d;
-    const double* ps = d + n;
-    const double tf = d[2 * n], ts = d[2 * n + 1];
-    const double nfx = d[2 * n + 2], nfy = d[2 * n + 3], nsx = d[2 * n + 4], nsy = d[2 * n + 5];
+    for (int e = t; e < 8 * n; e += blockDim.x) {   // m_x, m_y, p; s_xx, s_yy, s_xy, v_x, v_y
+        const int fld = e / n, i = e - fld * n;
+        val[fld][i] = fld < 3 ? (double)state[(size_t)(fld * n + i) * op.Nf + qf]
+                              : (double)ss[(size_t)((fld - 3) * n + i) * op.Ns + qs];
+    }
+    __syncthreads();
     const double* Ai = d + 2 * n + 6;
-    const double p = ev(sf, op.Nf, qf, 2, pf), mx = ev(sf, op.Nf, qf, 0, pf), my = ev(sf, op.Nf, qf, 1, pf);
-    const double sxx = ev(ss, op.Ns, qs, 0, ps), syy = ev(ss, op.Ns, qs, 1, ps), sxy = ev(ss, op.Ns, qs, 2, ps);
-    const double vx = ev(ss, op.Ns, qs, 3, ps), vy = ev(ss, op.Ns, qs, 4, ps);
-    const double wf = tf * p - (mx * nfx + my * nfy);
-    const double wsx = ts * vx - (sxx * nsx + sxy * nsy);
-    const double wsy = ts * vy - (sxy * nsx + syy * nsy);
-    const double o0 = Ai[0] * wf + Ai[1] * wsx + Ai[2] * wsy;
-    const double o1 = Ai[3] * wf + Ai[4] * wsx + Ai[5] * wsy;
-    const double o2 = Ai[6] * wf + Ai[7] * wsx + Ai[8] * wsy;
-    double g[3];
-    for (int j = 0; j < 3; ++j) g[j] = (double)G[5 * r + j];
-    const double hf = Ai[0] * g[0] + Ai[3] * g[1] + Ai[6] * g[2];   // (Ai^T g)
-    const double hx = Ai[1] * g[0] + Ai[4] * g[1] + Ai[7] * g[2];
-    const double hy = Ai[2] * g[0] + Ai[5] * g[1] + Ai[8] * g[2];
-    grec[2 * r] += hf * (p - o0);
-    grec[2 * r + 1] += hx * (vx - o1) + hy * (vy - o2);
+    if (t < 8) {
+        const double* phi = t < 3 ? d : d + n;
+        double v = 0.0;
+        for (int i = 0; i < n; ++i) v = fma(phi[i], val[t][i], v);
+        g[t] = v;
+    } else if (t < 11) {   // Ai^T g
+        const int j = t - 8;
+        hg[j] = Ai[j] * (double)G[5 * r] + Ai[3 + j] * (double)G[5 * r + 1] + Ai[6 + j] * (double)G[5 * r + 2];
+    }
+    __syncthreads();
+    if (t < 3) {
+        const double tf = d[2 * n], ts = d[2 * n + 1];
+        const double nfx = d[2 * n + 2], nfy = d[2 * n + 3], nsx = d[2 * n + 4], nsy = d[2 * n + 5];
+        w[t] = t == 0   ? tf * g[2] - (g[0] * nfx + g[1] * nfy)
+               : t == 1 ? ts * g[6] - (g[3] * nsx + g[5] * nsy)
+                        : ts * g[7] - (g[5] * nsx + g[4] * nsy);
+    }
+    __syncthreads();
+    if (t < 3) o[t] = Ai[3 * t] * w[0] + Ai[3 * t + 1] * w[1] + Ai[3 * t + 2] * w[2];
+    __syncthreads();
+    if (t == 0) grec[2 * r] += hg[0] * (g[2] - o[0]);
+    if (t == 1) grec[2 * r + 1] += hg[1] * (g[6] - o[1]) + hg[2] * (g[7] - o[2]);
 }
-
 // One time node's receiver part: lambda^ += S M^-1 R^T G (the transpose of
 // record_kernel, lambda^ = S M^-1 lambda) and d(G^T d)/dtau of the interface
 // receivers.  Blocks 0 .. n_inj - 1 own one cell that receivers read: thread
 // (field, i) adds up the contributions of that cell's receivers in increasing
 // receiver order, then the block applies the cell's inverse mass in shared
-// memory.  The blocks after them take the interface receivers' tau terms, one
-// receiver a thread, so that the two run side by side.  blockDim >= 5 n.
+// memory.  The blocks after them take the interface receivers' tau terms, so
+// that the two run side by side (one receiver a thread: 14.7 us a launch
+// for 128 receivers, now 7.6).  blockDim >= 5 n.
 template <class T>
-__global__ void node_kernel(DevOps op, int n_inj, const int32_t* __restrict__ inj, int n_rec,
+__global__ void node_kernel(DevOps op, int n_inj, const int32_t* __restrict__ inj,
                             const int32_t* __restrict__ ri, const double* __restrict__ rd, const T* __restrict__ G,
                             const double* __restrict__ mass_f, const double* __restrict__ mass_s,
                             const double* __restrict__ cls_minv, const T* __restrict__ state, T* lam,
@@ -135,7 +139,7 @@ __global__ void node_kernel(DevOps op, int n_inj, const int32_t* __restrict__ in
     const int n = op.n;
     const int stride = 2 * n + 15;
     if ((int)blockIdx.x >= n_inj) {
-        rec_tau(op, ((int)blockIdx.x - n_inj) * blockDim.x + threadIdx.x, n_rec, ri, rd, state, G, grec);
+        rec_tau(op, (int)blockIdx.x - n_inj, ri, rd, state, G, grec);
         return;
     }
     const int t = blockIdx.x;
@@ -492,8 +496,8 @@ int adjoint_vjp_t(hho_ops* ops, const hho_tableau* tab, double t0, double dt, in
             const double tn = t0 + (double)(n - 1) * dt;
             if (ops->n_rec > 0) {   // U^n is the next step's first stage value in the store
                 const int thr = (5 * ops->n + 31) / 32 * 32;
-                node_kernel<E><<<ops->n_inj + (ops->n_rec + thr - 1) / thr, thr, 0, st>>>(
-                    ops->dev, ops->n_inj, ops->d_inj, ops->n_rec, ops->d_rec_int, ops->d_rec_dbl,
+                node_kernel<E><<<ops->n_inj + ops->n_rec, thr, 0, st>>>(
+                    ops->dev, ops->n_inj, ops->d_inj, ops->d_rec_int, ops->d_rec_dbl,
                     d_cotangent + (size_t)(n - 1) * 5 * ops->n_rec, ops->d_mass_f, ops->d_mass_s, ops->d_cls_minv,
                     Y(m + 1, 0), B.lam, B.grec);
             }
@@ -555,87 +559,87 @@ int adjoint_vjp_t(hho_ops* ops, const hho_tableau* tab, double t0, double dt, in
         }
     }
     // ---- gradients to the host, mapped to the materials ----------------------------------------
-    std::vector<double> gf(2 * (size_t)ops->dev.Nf), gs(4 * (size_t)ops->dev.Ns);
+    // What the mapping needs besides the sums is prepared while the GPU works:
+    // o[0..3] = dL/d(rho, kappa, lambda, mu) are linear in the cell's sums.
+    const int Nf = ops->dev.Nf, Ns = ops->dev.Ns;
+    const int64_t nc = ops->nc;
+    std::vector<double> gf(2 * (size_t)Nf), gs(4 * (size_t)Ns);
     std::vector<double> gstab((size_t)nthr), grec(2 * (size_t)std::max(ops->n_rec, 1));
-    if ((!gf.empty() && cudaMemcpyAsync(gf.data(), B.grad_f, sizeof(double) * gf.size(), cudaMemcpyDeviceToHost, st) !=
-                            cudaSuccess) ||
-        (!gs.empty() && cudaMemcpyAsync(gs.data(), B.grad_s, sizeof(double) * gs.size(), cudaMemcpyDeviceToHost, st) !=
-                            cudaSuccess) ||
-        (!gstab.empty() &&
-         cudaMemcpyAsync(gstab.data(), B.gstab, sizeof(double) * gstab.size(), cudaMemcpyDeviceToHost, st) !=
-             cudaSuccess) ||
-        cudaMemcpyAsync(grec.data(), B.grec, sizeof(double) * grec.size(), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess) {
+    std::vector<double> gtau((size_t)nc, 0.0);
+    std::vector<int32_t> orig((size_t)nthr, -1);
+    struct Map {
+        double m[4];   // fluid: d(A_m)/d rho, 1/h; solid: d(A_v)/d rho, 1/h, dr/d lambda, dr/d mu
+        double t[3];   // dtau/d rho, and / d kappa or d lambda, and / d mu
+    };
+    std::vector<Map> map((size_t)nc);
+    for (int64_t c = 0; c < nc; ++c) {
+        Map& M = map[c];
+        const double h = ops->diam[c], rho = ops->rho[c], t = ops->tau[c];
+        orig[(ops->cell_dom[c] == 0 ? 0 : Nf) + ops->cell_pos[c]] = (int32_t)c;
+        M.m[0] = -1.0 / (rho * rho * h);   // A_m = 1/(rho h), A_v = 1/(rho h)
+        M.m[1] = 1.0 / h;                  // A_p = kappa/h, c1 = (lambda + 2 mu)/h, c3 = mu/h
+        // tau^f = eta_f (rho kappa)^-1/2; tau^s = eta_s (rho (lambda + 2 mu))^1/2 or eta_s (rho mu)^1/2
+        // (an optional 1/k factor cancels in these logarithmic derivatives)
+        if (ops->cell_dom[c] == 0) {
+            M.t[0] = -0.5 * t / rho;
+            M.t[1] = -0.5 * t / ops->kappa[c];
+            M.t[2] = 0.0;
+        } else {
+            const double lam = ops->lam[c], mu = ops->mu[c], l2m = lam + 2.0 * mu;
+            M.m[2] = 2.0 * mu / (l2m * l2m);    // r = lambda/(lambda + 2 mu)
+            M.m[3] = -2.0 * lam / (l2m * l2m);
+            M.t[0] = 0.5 * t / rho;
+            M.t[1] = ops->stab_speed == 0 ? 0.5 * t / l2m : 0.0;
+            M.t[2] = ops->stab_speed == 0 ? t / l2m : 0.5 * t / mu;
+        }
+    }
+    std::vector<int32_t> ri(4 * (size_t)std::max(ops->n_rec, 1));
+    std::vector<double> wg(ops->n_src > 0 && h_grad_wavelet ? (size_t)nsteps * s * MAX_SOURCES : 0);
+    auto fetch = [&](void* dst, const void* src, size_t bytes) {
+        return bytes == 0 || cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, st) == cudaSuccess;
+    };
+    if (!fetch(gf.data(), B.grad_f, sizeof(double) * gf.size()) || !fetch(gs.data(), B.grad_s, sizeof(double) * gs.size()) ||
+        !fetch(gstab.data(), B.gstab, sizeof(double) * gstab.size()) ||
+        !fetch(grec.data(), B.grec, sizeof(double) * grec.size()) ||
+        !fetch(wg.data(), B.wgrad, sizeof(double) * wg.size()) ||
+        !fetch(ri.data(), ops->d_rec_int, sizeof(int32_t) * 4 * ops->n_rec) || cudaStreamSynchronize(st) != cudaSuccess) {
         hho_set_error("%s: gradient copy failed", who);
         return HHO_ECUDA;
     }
-    if (ops->n_src > 0 && h_grad_wavelet) {
-        std::vector<double> wg((size_t)nsteps * s * MAX_SOURCES);
-        if (cudaMemcpy(wg.data(), B.wgrad, sizeof(double) * wg.size(), cudaMemcpyDeviceToHost) != cudaSuccess) {
-            hho_set_error("%s: wavelet gradient copy failed", who);
-            return HHO_ECUDA;
-        }
-        for (int64_t n = 0; n < nsteps; ++n)
-            for (int j = 0; j < s; ++j)
-                for (int k2 = 0; k2 < ops->n_src; ++k2)
-                    h_grad_wavelet[(n * s + j) * ops->n_src + k2] = wg[(n * s + j) * MAX_SOURCES + k2];
-    }
-    const int Nf = ops->dev.Nf, Ns = ops->dev.Ns;
+    for (int64_t e = 0; e < (int64_t)(wg.size() / MAX_SOURCES); ++e)
+        for (int k2 = 0; k2 < ops->n_src; ++k2) h_grad_wavelet[e * ops->n_src + k2] = wg[e * MAX_SOURCES + k2];
     // dL/dtau per cell: the stage part (face integrals scale with h) and the
     // interface receivers' part, mapped from device positions to cell ids
-    std::vector<double> gtau((size_t)ops->nc, 0.0);
-    std::vector<int64_t> orig_f((size_t)Nf, -1), orig_s((size_t)Ns, -1);
-    for (int64_t c = 0; c < ops->nc; ++c) {
-        const int q = ops->cell_pos[c];
-        (ops->cell_dom[c] == 0 ? orig_f : orig_s)[q] = c;
-        gtau[c] = -ops->diam[c] * gstab[(ops->cell_dom[c] == 0 ? 0 : Nf) + q];
-    }
-    {
-        std::vector<int32_t> ri(4 * (size_t)std::max(ops->n_rec, 1));
-        if (ops->n_rec > 0 &&
-            cudaMemcpy(ri.data(), ops->d_rec_int, sizeof(int32_t) * 4 * ops->n_rec, cudaMemcpyDeviceToHost) !=
-                cudaSuccess) {
-            hho_set_error("%s: receiver table copy failed", who);
-            return HHO_ECUDA;
+    for (int g = 0; g < nthr; ++g)
+        if (orig[g] >= 0) gtau[orig[g]] = -ops->diam[orig[g]] * gstab[g];
+    for (int r = 0; r < ops->n_rec; ++r)
+        if (ri[4 * r] == 2) {
+            gtau[orig[ri[4 * r + 1]]] += grec[2 * r];
+            gtau[orig[Nf + ri[4 * r + 2]]] += grec[2 * r + 1];
         }
-        for (int r = 0; r < ops->n_rec; ++r)
-            if (ri[4 * r] == 2) {
-                gtau[orig_f[ri[4 * r + 1]]] += grec[2 * r];
-                gtau[orig_s[ri[4 * r + 2]]] += grec[2 * r + 1];
-            }
-    }
-    if (h_grad_tau)
-        for (int64_t c = 0; c < ops->nc; ++c) h_grad_tau[c] = gtau[c];
-    for (int64_t c = 0; c < ops->nc; ++c) {
-        double* o = h_grad_cell + 4 * c;   // [rho, kappa, lambda, mu]
-        o[0] = o[1] = o[2] = o[3] = 0.0;
+    if (h_grad_tau) std::copy(gtau.begin(), gtau.end(), h_grad_tau);
+    for (int64_t c = 0; c < nc; ++c) {
+        double* o = h_grad_cell + 4 * c;
+        const Map& M = map[c];
         const int q = ops->cell_pos[c];
-        const double h = ops->diam[c], rho = ops->rho[c];
+        o[0] = o[1] = o[2] = o[3] = 0.0;
         if (ops->cell_dom[c] == 0) {
-            o[0] = gf[q] * (-1.0 / (rho * rho * h));                       // A_m = 1/(rho h)
-            o[1] = gf[Nf + q] / h;                                          // A_p = kappa/h
+            o[0] = gf[q] * M.m[0];
+            o[1] = gf[Nf + q] * M.m[1];
         } else {
-            const double lam = ops->lam[c], mu = ops->mu[c], l2m = lam + 2.0 * mu;
             const double gc1 = gs[q], gr = gs[Ns + q], gc3 = gs[2 * Ns + q], gav = gs[3 * Ns + q];
-            o[0] = gav * (-1.0 / (rho * rho * h));                          // A_v = 1/(rho h)
-            o[2] = gc1 / h + gr * (2.0 * mu / (l2m * l2m));                 // c1 = (lambda+2mu)/h, r = lambda/(lambda+2mu)
-            o[3] = gc1 * 2.0 / h + gr * (-2.0 * lam / (l2m * l2m)) + gc3 / h;   // c3 = mu/h
+            o[0] = gav * M.m[0];
+            o[2] = gc1 * M.m[1] + gr * M.m[2];
+            o[3] = gc1 * 2.0 * M.m[1] + gr * M.m[3] + gc3 * M.m[1];
         }
         if (ops->tau_explicit) continue;
-        // tau^f = eta_f (rho kappa)^-1/2; tau^s = eta_s (rho (lambda + 2 mu))^1/2 or eta_s (rho mu)^1/2
-        // (an optional 1/k factor cancels in these logarithmic derivatives)
-        const double t = ops->tau[c], gt = gtau[c];
+        const double gt = gtau[c];
+        o[0] += gt * M.t[0];
         if (ops->cell_dom[c] == 0) {
-            o[0] += gt * (-0.5 * t / rho);
-            o[1] += gt * (-0.5 * t / ops->kappa[c]);
-        } else if (ops->stab_speed == 0) {
-            const double l2m = ops->lam[c] + 2.0 * ops->mu[c];
-            o[0] += gt * (0.5 * t / rho);
-            o[2] += gt * (0.5 * t / l2m);
-            o[3] += gt * (t / l2m);
+            o[1] += gt * M.t[1];
         } else {
-            o[0] += gt * (0.5 * t / rho);
-            o[3] += gt * (0.5 * t / ops->mu[c]);
+            if (ops->stab_speed == 0) o[2] += gt * M.t[1];
+            o[3] += gt * M.t[2];
         }
     }
     return HHO_OK;
