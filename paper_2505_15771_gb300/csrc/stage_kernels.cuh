@@ -408,36 +408,42 @@ __device__ __forceinline__ void load_state(const T* __restrict__ src, int N, int
 // per-cell material factor of value i (the inverse mass, folded into the
 // target coefficient).  Target 0 is kept in `k` (overwritten).  `off` is the
 // offset of this shot's domain block.
+//
+// The sources are read TARGET_BATCH at a time before any of the batch is
+// stored: a target may be its own source (the ERK accumulator), so the compiler
+// keeps every later load behind every earlier store, and value by value the
+// targets were 100 memory round trips in a row for a k = 3 solid cell.  Stage
+// kernel, us, by batch 1 | 5 | 10 | 16 | 25: FP32, 16 shots of the 680 x 340
+// k = 3 hybrid mesh 1174 | 892 | 866 | 869 | 908; FP32, 21 shots of the 331 x 167
+// k = 2 hanging mesh 318 | 288 | 283 | 279 | 292; double-float, 1024 x 512,
+// k = 2: 210 | - | 172 | 174 (15); FP64 the same: 247 | 237 (3) | 238.
+constexpr int TARGET_BATCH = 10;
 template <int NV, class GRP, class T>
 __device__ __forceinline__ void write_targets(const StageArgsT<T>& A, int N, size_t off, int q, T* k, const T* sc) {
-    for (int t = A.n_tgt - 1; t >= 1; --t) {
+    constexpr int B = TARGET_BATCH;
+#pragma unroll 1
+    for (int t = A.n_tgt - 1; t >= 0; --t) {
         const TargetT<T> G = A.tgt[t];
         const T c[3] = {G.coef * sc[0], G.coef * sc[1], G.coef * sc[2]};
         T* dst = G.dst + off;
-        if (G.src) {
-            const T* src = G.src + off;
-#pragma unroll
-            for (int i = 0; i < NV; ++i) dst[(size_t)i * N + q] = norm(fma(c[GRP::g(i)], k[i], src[(size_t)i * N + q]));
-        } else {
-#pragma unroll
-            for (int i = 0; i < NV; ++i) dst[(size_t)i * N + q] = norm(c[GRP::g(i)] * k[i]);
-        }
-    }
-    const TargetT<T> G = A.tgt[0];
-    const T c[3] = {G.coef * sc[0], G.coef * sc[1], G.coef * sc[2]};
-    T* dst = G.dst + off;
-    if (G.src) {
         const T* src = G.src + off;
+        const bool add = G.src != nullptr;
 #pragma unroll
-        for (int i = 0; i < NV; ++i) {
-            k[i] = norm(fma(c[GRP::g(i)], k[i], src[(size_t)i * N + q]));
-            dst[(size_t)i * N + q] = k[i];
-        }
-    } else {
+        for (int i0 = 0; i0 < NV; i0 += B) {
+            T s[B];
+            if (add) {
 #pragma unroll
-        for (int i = 0; i < NV; ++i) {
-            k[i] = norm(c[GRP::g(i)] * k[i]);
-            dst[(size_t)i * N + q] = k[i];
+                for (int b = 0; b < B; ++b)
+                    if (i0 + b < NV) s[b] = src[(size_t)(i0 + b) * N + q];
+            }
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                const int i = i0 + b;
+                if (i >= NV) continue;
+                const T v = norm(add ? fma(c[GRP::g(i)], k[i], s[b]) : c[GRP::g(i)] * k[i]);
+                dst[(size_t)i * N + q] = v;
+                if (t == 0) k[i] = v;
+            }
         }
     }
 }
@@ -497,11 +503,11 @@ __device__ __forceinline__ void for_faces(const CellCtx<T>& c, H hor, V ver, O o
 // Prefetch hints take no register and bring the lines of later rounds into
 // L2 early.  Mask bits: 1 state, 2 own traces and face tables, 4 neighbour
 // traces, 8 target sources, all at the start of the cell; 16 target sources
-// and 32 neighbour traces just before the face loop.  The FP32 kernel gains
-// about 20 % from them (mask 50, the best of a sweep on GB300).  The 8-byte
-// kernels with register accumulators (spilled) lost with every mask; the
-// 8-byte k = 2 kernels with shared-memory accumulators gain from mask 50 too
-// (double-float about 10 % over no hints, FP64 a few per cent).
+// and 32 neighbour traces just before the face loop.  Stage kernel, us, by mask:
+// FP32, 16 shots of the 680 x 340 k = 3 hybrid mesh 0: 944, 34: 902, 51: 843;
+// double-float, 1024 x 512, k = 2, 0: 169.9, 34: 169.4, 50: 172, 51: 174;
+// FP64 the same 0: 225, 34: 230, 50: 236 (its pipe binds, and the hints are
+// instructions).  Register accumulators (spilled) lost with every mask.
 template <class T, int K>
 struct L2Prefetch {
     static constexpr int mask = Tuned<T>::t.prefetch[K - 1];
@@ -1539,12 +1545,13 @@ __device__ __forceinline__ void solid_cell(const StageArgsT<T>& A, int q, int sh
 
 // Resident blocks per SM asked of the register allocator (128 threads a
 // block): 2 blocks allow 255 registers, 3 allow 168, 4 allow 128, 5 allow 96,
-// 6 allow 80, 8 allow 64.  The stage kernels are bound by load latency, so
-// occupancy pays even at the price of spills to local memory; where the
-// accumulators sit in shared memory (AccSmem) the shared memory may cap the
-// resident blocks below this count.  The values are the fastest of sweeps
-// on the 1024 x 512 bilayer (and, for FP32, the 1.2 M-cell hybrid mesh) on
-// GB300.
+// 6 allow 80, 8 allow 64.  The kernels wait for loads, so occupancy pays until
+// the registers no longer hold a batch of them (write_targets): us a stage by
+// blocks, FP32 k = 3 (16 hybrid shots) 8: 866, 6: 849, 5: 862, 4: 903; FP32 k = 2
+// (21 hanging shots) 12: 309, 10: 283, 8: 260, 6: 260, 5: 277; double-float k = 2
+// (1024 x 512) 6: 177, 5: 172, 4: 182; FP64 k = 2 8: 225, 6: 224, 5: 225; FP64
+// k = 3 (680 x 340 hybrid) 8: 291, 6: 286, 5: 284.  Where the accumulators sit in
+// shared memory (AccSmem) it may cap the resident blocks below this count.
 template <class T, int K>
 struct MinBlocks {
     static constexpr int value = Tuned<T>::t.min_blocks[K - 1];
@@ -1616,7 +1623,8 @@ __device__ __forceinline__ void tau_cell(const StageArgsT<T>& A, const GradArgsT
 // forward stage value, taken straight into the gradient sums instead of being
 // stored.  y = 0: the mass part, y = 1: the tau part, which share nothing but the
 // traces they read; side by side they halve the chain of a thread and fill a
-// grid of one wave (65,536 cells, k = 2: FP64 44.4 -> 42.8 us, FP32 30.1 -> 20.8).
+// grid of one wave (65,536 cells, k = 2: FP64 44.4 -> 42.8 us, FP32 30.1 -> 20.8; 40.8 and 19.2
+// with the block counts of stage_tuning.h).
 template <class T, int K>
 __global__ void __launch_bounds__(128, MinBlocks<T, K>::value)
     grad_stage_kernel(const StageArgsT<T> A, const GradArgsT<T> G) {
@@ -1668,7 +1676,8 @@ namespace hho_stage {
 // large grids.  A grid of at most 20 warps per SM runs in one wave, where
 // blocks of one warp spread the cells evenly over the SMs: with 128 threads
 // the 65,536 cells of the 256 x 256 adjoint leave SMs with 3 or 4 blocks, and
-// a stage took 49.0 us against 41.6 (its gradients 55.0 against 46.7).  With
+// a stage took 49.0 us against 41.6 when that was measured (its gradients 55.0
+// against 46.7).  With
 // several waves the smaller blocks cost 1 to 10 % (21 FP32 shots: 354 us
 // against 321, whose shared memory per block leaves fewer resident warps).
 inline int stage_threads(int64_t warps) { return warps <= 20 * 152 ? 32 : 128; }
@@ -1683,12 +1692,12 @@ struct TeamTag {};
 // blocks an SM) but for the 8-byte types at k = 3, whose ten rows fit ten warps.
 // Both forms give the same bits, so the choice is free.  Measured on GB300, us
 // a stage, thread form / team form:
-//                             128 groups    1024 groups    4096 groups
-//   FP64 k = 2 squares        26.4 / 8.6    30.4 / 25.8    82.6 / 93.2
-//   FP64 k = 3 hanging        81.9 / 18.2   97 / 61        214 / 196
-//   double-float k = 2 squares 23.1 / 6.4   26.9 / 13.6    65.2 / 54.2
-//   double-float k = 3 tri.   49.6 / 8.4    57.7 / 25.7    162 / 96
-//   FP32 k = 2 squares        13.8 / 4.8    19.0 / 8.3     22.6 / 25.6
+//                               512 groups    1024          2048          4096
+//   FP64 k = 2 squares          18.9 / 17.1   21.4 / 26.7   31.7 / 44.3   68.7 / 87.8
+//   FP64 k = 3 hanging          68.2 / 28.2   74.6 / 46.0   107 / 91.2    165 / 174
+//   double-float k = 2 squares  19.5 / 8.3    20.6 / 12.6   22.5 / 23.0   52.3 / 54.9
+//   double-float k = 3 squares  31.2 / 12.9   36.5 / 20.4   68.3 / 46.7   113 / 88.3
+//   FP32 k = 2 squares          8.9 / 5.5     9.7 / 7.7     10.5 / 13.8   14.8 / 25.2
 // Large FP64 grids are bound by the FP64 pipe, and the thread form issues the
 // fewer FP64 instructions; large FP32 ones by memory, where its coalesced rows
 // of one warp do as well with less code.
@@ -1700,15 +1709,15 @@ constexpr int TEAM_ALL = 1 << 30;
     struct TeamRule<T_, K_> {                                                                                 \
         static constexpr int W = W_, rect = rect_, gen = gen_, app = app_, tr_rect = tr_rect_, tr_gen = tr_gen_; \
     }
-HHO_TEAM_RULE(double, 1, 8, 1000, 1300, 900, 128, 400);
-HHO_TEAM_RULE(double, 2, 8, 1500, 2000, 1150, 200, 600);
-HHO_TEAM_RULE(double, 3, 10, 2000, 3500, 1500, 300, 900);
-HHO_TEAM_RULE(f2x, 1, 8, 2000, 2600, 1500, 700, 900);
-HHO_TEAM_RULE(f2x, 2, 8, TEAM_ALL, TEAM_ALL, 3000, 512, 1100);
-HHO_TEAM_RULE(f2x, 3, 10, TEAM_ALL, TEAM_ALL, 3000, 1100, TEAM_ALL);
-HHO_TEAM_RULE(float, 1, 8, 1800, 2100, 0, 200, 300);
-HHO_TEAM_RULE(float, 2, 8, 3000, 3000, 0, 200, 300);
-HHO_TEAM_RULE(float, 3, 10, 3500, 4100, 0, 200, 400);
+HHO_TEAM_RULE(double, 1, 8, 800, 2500, 1300, 128, 900);
+HHO_TEAM_RULE(double, 2, 8, 650, 2100, 1100, 200, 900);
+HHO_TEAM_RULE(double, 3, 10, 1050, 3200, 1500, 300, 1500);
+HHO_TEAM_RULE(f2x, 1, 8, 1800, 3200, 2500, 1300, 3000);
+HHO_TEAM_RULE(f2x, 2, 8, 2000, TEAM_ALL, 4000, 700, 4000);
+HHO_TEAM_RULE(f2x, 3, 10, TEAM_ALL, TEAM_ALL, 3000, 1500, 5500);
+HHO_TEAM_RULE(float, 1, 8, 1300, 1900, 0, 200, 900);
+HHO_TEAM_RULE(float, 2, 8, 1400, 1900, 0, 200, 850);
+HHO_TEAM_RULE(float, 3, 10, 1250, 1700, 0, 200, 1200);
 #undef HHO_TEAM_RULE
 
 // Warps of a team block for this launch, 0 for the thread form.
