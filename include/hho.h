@@ -309,10 +309,12 @@ int hho_erk_step_record(hho_ops* ops, const hho_tableau* tab, double t0, double 
  * stepped, unpacked back into h_canonical, and the stream is synchronised.
  * Pinned host memory (cudaHostAlloc, or a pinned torch tensor) mapped into
  * the device's address space is read and written by the pack kernels
- * directly; other host memory is staged through a device copy.  Both give
- * the same bits as hho_state_pack, hho_erk_step and hho_state_unpack.  The
- * device buffers it needs are allocated on the first call and kept with
- * ops. */
+ * directly or, on large meshes (4096 warps of 32 cells and more), copied in
+ * pieces that overlap the first and the last stage; other host memory is
+ * staged through one device copy.  All give the same bits as
+ * hho_state_pack, hho_erk_step and hho_state_unpack.  The device buffers,
+ * the copy stream and the events it needs are made on the first call and
+ * kept with ops. */
 int hho_erk_run_host(hho_ops* ops, const hho_tableau* tab, double t0, double dt, int64_t nsteps,
                      double* h_canonical, void* stream);
 

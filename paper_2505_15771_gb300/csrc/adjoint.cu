@@ -37,7 +37,7 @@
 // eta_F = -K_F^-T K_TF^T eta the adjoint face values of eta = M^-1 mu.  By the
 // same block structure eta_F are the face values of the coupling-reversed
 // operator A' applied to x = S eta, which the backward stage computes anyway:
-// tau_grad (stage.cu) takes the products of both jumps from the two trace
+// tau_grad (stage_kernels.cuh) takes the products of both jumps from the two trace
 // buffers.  The interface receivers read face values, which depend on tau
 // too (rec_tau).  The host maps dL/dtheta and dL/dtau to
 // dL/d(rho, kappa, lambda, mu); with tau given explicitly

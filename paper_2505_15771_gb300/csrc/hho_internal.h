@@ -145,6 +145,7 @@ struct StageArgsT {
     T* tr_out;               // traces of the target-0 result (same layout)
     TargetT<T> tgt[MAX_TARGETS];
     int32_t n_tgt;
+    int32_t warp0, n_warps;  // the launch's warps of cells (of both domains' concatenation); n_warps 0: all
     int32_t pad0;
     int64_t state_stride, trace_stride;
     // point sources applied to every shot
@@ -200,6 +201,7 @@ struct StagePlan {
     int n_tgt;
     TargetPlan t[MAX_TARGETS];
 };
+void free_host_pipe(struct HostPipe* p);
 int build_plan(const hho_tableau* tab, std::vector<StagePlan>& plan, int* n_buf);
 
 // Launches one stage-kernel pass (FP64) over n_shots shots; and the receiver
@@ -228,6 +230,30 @@ bool bj_traces_fit(const hho_ops* ops);
 void launch_bj(const hho_ops* ops, const double* bj, const double* x, const double* scale, double* y, bool accumulate,
                double* tr, void* stream);
 
+// The pieces of a host-buffer call on a large mesh: host pieces are runs of
+// canonical cells, compute pieces runs of warps in the device order.  The copy
+// engine brings host piece c while earlier pieces are packed, traced and taken
+// through the first stage; after the last stage each piece returns as soon as its
+// cells are done.  A compute piece's traces need its own cells, its first stage
+// the traces of its face neighbours too.  The order only decides what overlaps:
+// a mesh whose device order is unrelated to its cell order runs one after the other.
+//
+// From 4096 warps of cells (131 K cells, 15 to 25 MB each way at k = 2), a piece
+// for every 2048 of them: smaller pieces leave the SMs idle between them for
+// longer than the copies they hide.  One FP64 step of the k = 2 bilayer, us, by
+// pieces 1 | 2 | 4 | 8 | 16: 1024 x 512 2038 | 1889 | 1823 | 1719 | 1815; 724 x 362
+// 1083 | 1035 | 999 | 1023 | 1312; 512 x 272 590 | 575 | 591 | 690 | 946.
+constexpr int STAGED_CELLS = 64;   // cells of a block of the host pack kernels
+struct HostPieces {
+    static constexpr int MAX = 8, WARPS = 2048;
+    int n = 1;
+    int blocks[MAX + 1], warps[MAX + 1];   // host pieces in blocks of STAGED_CELLS cells, compute pieces in warps
+    int64_t off[MAX + 1];                  // host pieces in values
+    int own[MAX], need[MAX];               // the last host piece that compute piece d's traces / first stage wait for
+    int order[MAX];                        // compute pieces by need
+    int last[MAX];                         // host piece c is complete after order[last[c]]
+};
+struct HostPipe;
 struct hho_ops {
     int32_t k = 0, n = 0, f = 0;
     int64_t nc = 0;
@@ -313,6 +339,8 @@ struct hho_ops {
     double* d_host_canon = nullptr;
     double* d_host_work = nullptr;
     int64_t host_work_size = 0;
+    HostPieces host_pieces;
+    HostPipe* host_pipe = nullptr;   // the copy stream and events of a call in pieces (stage.cu)
     int64_t n_state = 0;
     int64_t trace_doubles = 0;    // one trace buffer (fluid + solid parts)
     // tensor-core batched stage (HHO_BF16X3): per class the split-BF16

@@ -7,6 +7,8 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <functional>
+#include <memory>
 #include <type_traits>
 #include <vector>
 
@@ -111,16 +113,15 @@ void launch_unpack(const hho_ops* ops, int n_shots, const void* state, double* c
 // crosses the host link in coalesced 8-byte accesses (eight in flight per
 // thread) and is reordered through shared memory, one thread per cell on the
 // device side.  Padding slots of the state are not touched.
-constexpr int STAGED_CELLS = 64;
 template <class T>
 __global__ void __launch_bounds__(STAGED_CELLS) pack_host_kernel(const int32_t* __restrict__ cell_dom,
                                                                  const int32_t* __restrict__ cell_pos,
                                                                  const int64_t* __restrict__ canon_off, int nc,
                                                                  int64_t n_canon, int Nf, int Ns, int n,
                                                                  const double* __restrict__ canon,
-                                                                 T* __restrict__ state) {
+                                                                 T* __restrict__ state, int block0) {
     extern __shared__ double run[];
-    const int c0 = blockIdx.x * STAGED_CELLS;
+    const int c0 = (block0 + blockIdx.x) * STAGED_CELLS;
     const int c1 = min(c0 + STAGED_CELLS, nc);
     const int64_t e0 = canon_off[c0];
     const int len = (int)((c1 < nc ? canon_off[c1] : n_canon) - e0);
@@ -155,9 +156,9 @@ __global__ void __launch_bounds__(STAGED_CELLS) unpack_host_kernel(const int32_t
                                                                    const int64_t* __restrict__ canon_off, int nc,
                                                                    int64_t n_canon, int Nf, int Ns, int n,
                                                                    const T* __restrict__ state,
-                                                                   double* __restrict__ canon) {
+                                                                   double* __restrict__ canon, int block0) {
     extern __shared__ double run[];
-    const int c0 = blockIdx.x * STAGED_CELLS;
+    const int c0 = (block0 + blockIdx.x) * STAGED_CELLS;
     const int c1 = min(c0 + STAGED_CELLS, nc);
     const int64_t e0 = canon_off[c0];
     const int len = (int)((c1 < nc ? canon_off[c1] : n_canon) - e0);
@@ -516,9 +517,57 @@ struct SeisOf<f2x> {
     using type = double;
 };
 
+// What a host-buffer call in pieces (HostPieces) keeps with the operator: its copy
+// stream and the events of the pieces.
+struct HostPipe {
+    cudaStream_t copy = nullptr;
+    cudaEvent_t start = nullptr, in[HostPieces::MAX] = {}, out[HostPieces::MAX] = {};
+};
+
+// Whether erk_run replays the step as a graph (blocks: of 128 cells, all shots).
+static bool uses_graph(const hho_ops* ops, int64_t blocks, int64_t nsteps) {
+    return !ops->prof_on && ops->d_clock && !ops->src_sampled &&
+           (ops->launch_mode == HHO_LAUNCH_GRAPH || (ops->launch_mode == HHO_LAUNCH_AUTO && blocks <= 2048 && nsteps >= 8));
+}
+
+// A call that takes its state and hands it back in pieces (HostPieces): arrive(c)
+// enqueues host piece c into the state, leave(c) out of it.
+struct PieceHooks {
+    std::function<int(int)> arrive, leave;
+};
+
+// The first stage (its pieces follow their arrivals and the traces they need),
+// the last one (its pieces are followed by the host pieces they complete), or a
+// stage that is both.
+template <class T>
+static int stage_pieces(const hho_ops* ops, const StageArgsT<T>& traces, const StageArgsT<T>& stage,
+                        const PieceHooks& hooks, bool first, bool last, cudaStream_t st) {
+    const HostPieces& p = ops->host_pieces;
+    auto part = [&](StageArgsT<T> a, int d) {
+        a.warp0 = p.warps[d];
+        a.n_warps = p.warps[d + 1] - p.warps[d];
+        return a;
+    };
+    int rc = HHO_OK;
+    for (int c = 0, i = 0; c < p.n && !rc; ++c) {
+        if (first) {
+            rc = hooks.arrive(c);
+            for (int d = 0; d < p.n && !rc; ++d)
+                if (p.own[d] == c) launch_stage<T, MODE_TRACES>(ops, part(traces, d), 1, st);
+        }
+        for (; i < p.n && !rc && (!first || p.need[p.order[i]] <= c); ++i) {
+            launch_stage<T, MODE_STAGE>(ops, part(stage, p.order[i]), 1, st);
+            for (int h = 0; h < p.n && last && !rc; ++h)
+                if (p.last[h] == i) rc = hooks.leave(h);
+        }
+    }
+    return rc;
+}
+
 template <class T>
 static int erk_run(hho_ops* ops, const hho_tableau* tab, double t0, double dt, int64_t nsteps, int n_shots,
-                   T* d_state, T* d_work, void* d_seis_v, void* stream, const char* who) {
+                   T* d_state, T* d_work, void* d_seis_v, void* stream, const char* who,
+                   const PieceHooks* pieces = nullptr) {
     using TS = typename SeisOf<T>::type;
     TS* d_seis = (TS*)d_seis_v;
     if (!ops || !tab || !d_state || !d_work || nsteps < 0 || n_shots < 1 || n_shots > 65535 || !std::isfinite(dt) ||
@@ -555,13 +604,14 @@ static int erk_run(hho_ops* ops, const hho_tableau* tab, double t0, double dt, i
     a.inp = d_state;
     a.tr_out = tr[0];
     a.n_tgt = 0;
-    const bool use_graph =
-        !ops->prof_on && ops->d_clock && !ops->src_sampled &&
-        (ops->launch_mode == HHO_LAUNCH_GRAPH ||
-         (ops->launch_mode == HHO_LAUNCH_AUTO && (int64_t)grid.x * n_shots <= 2048 && nsteps >= 8));
-    launch_stage<T, MODE_TRACES>(ops, a, n_shots, st);
-    int rc = check_launch(who);
-    if (rc) return rc;
+    const bool use_graph = uses_graph(ops, (int64_t)grid.x * n_shots, nsteps);
+    const StageArgsT<T> traces = a;
+    int rc = HHO_OK;
+    if (!pieces) {
+        launch_stage<T, MODE_TRACES>(ops, traces, n_shots, st);
+        rc = check_launch(who);
+        if (rc) return rc;
+    }
     int cur = 0;
     if (use_graph) {
         // One step = its stage kernels, the receiver record and the clock
@@ -663,9 +713,11 @@ static int erk_run(hho_ops* ops, const hho_tableau* tab, double t0, double dt, i
             fill_sources<T>(ops, a, tn, j, tab->c[j] * dt, n_shots);
             const bool prof = ops->prof_on && 2 * ops->prof_n + 1 < (int)ops->prof_events.size();
             if (prof) cudaEventRecord((cudaEvent_t)ops->prof_events[2 * ops->prof_n], st);
-            launch_stage<T, MODE_STAGE>(ops, a, n_shots, st);
+            const bool first = pieces && step == 0 && j == 0, last = pieces && step == nsteps - 1 && j == tab->s - 1;
+            if (first || last) rc = stage_pieces<T>(ops, traces, a, *pieces, first, last, st);
+            else launch_stage<T, MODE_STAGE>(ops, a, n_shots, st);
             if (prof) cudaEventRecord((cudaEvent_t)ops->prof_events[2 * ops->prof_n++ + 1], st);
-            rc = check_launch(who);
+            if (!rc) rc = check_launch(who);
             if (rc) return rc;
             cur ^= 1;
         }
@@ -721,48 +773,118 @@ static int erk_single(hho_ops* ops, const hho_tableau* tab, double t0, double dt
     return check_launch(who);
 }
 
-// hho_erk_run_host on a pinned, mapped host buffer: the state is packed
-// from the host buffer straight into the arithmetic's device state (the
-// double-float pair copy, or the FP64 state), stepped, and unpacked
-// straight back, with no device copy of the canonical vector.
-static int erk_run_mapped(hho_ops* ops, const hho_tableau* tab, double t0, double dt, int64_t nsteps,
-                          double* m_canonical, cudaStream_t st) {
+template <class T>
+static int launch_host_pack(const hho_ops* ops, const double* canon, T* state, int block0, int blocks, cudaStream_t st) {
+    const size_t smem = sizeof(double) * STAGED_CELLS * 5 * ops->n;
+    pack_host_kernel<T><<<blocks, STAGED_CELLS, smem, st>>>(ops->d_cell_dom, ops->d_cell_pos, ops->d_canon_off,
+                                                            (int)ops->nc, ops->n_canonical, ops->dev.Nf, ops->dev.Ns,
+                                                            ops->n, canon, state, block0);
+    return check_launch("hho_erk_run_host");
+}
+template <class T>
+static int launch_host_unpack(const hho_ops* ops, const T* state, double* canon, int block0, int blocks, cudaStream_t st) {
+    const size_t smem = sizeof(double) * STAGED_CELLS * 5 * ops->n;
+    unpack_host_kernel<T><<<blocks, STAGED_CELLS, smem, st>>>(ops->d_cell_dom, ops->d_cell_pos, ops->d_canon_off,
+                                                              (int)ops->nc, ops->n_canonical, ops->dev.Nf, ops->dev.Ns,
+                                                              ops->n, state, canon, block0);
+    return check_launch("hho_erk_run_host");
+}
+
+void free_host_pipe(HostPipe* p) {
+    if (!p) return;
+    for (int c = 0; c < HostPieces::MAX; ++c) {
+        if (p->in[c]) cudaEventDestroy(p->in[c]);
+        if (p->out[c]) cudaEventDestroy(p->out[c]);
+    }
+    if (p->start) cudaEventDestroy(p->start);
+    if (p->copy) cudaStreamDestroy(p->copy);
+    delete p;
+}
+
+static int host_pieces(const hho_ops* ops, int64_t nsteps) {
+    if (nsteps < 1 || ops->prof_on || uses_graph(ops, (ops->dev.Nf + ops->dev.Ns + 127) / 128, nsteps)) return 1;
+    return ops->host_pieces.n;
+}
+
+static HostPipe* host_pipe(hho_ops* ops) {
+    if (ops->host_pipe) return ops->host_pipe;
+    std::unique_ptr<HostPipe, void (*)(HostPipe*)> p(new HostPipe, free_host_pipe);
+    bool ok = cudaStreamCreateWithFlags(&p->copy, cudaStreamNonBlocking) == cudaSuccess &&
+              cudaEventCreateWithFlags(&p->start, cudaEventDisableTiming) == cudaSuccess;
+    for (int c = 0; c < ops->host_pieces.n; ++c)
+        ok = ok && cudaEventCreateWithFlags(&p->in[c], cudaEventDisableTiming) == cudaSuccess &&
+             cudaEventCreateWithFlags(&p->out[c], cudaEventDisableTiming) == cudaSuccess;
+    return ok ? ops->host_pipe = p.release() : nullptr;
+}
+
+// hho_erk_run_host on a pinned host buffer: the state is packed into the
+// arithmetic's device state (the double-float pair copy, or the FP64 state),
+// stepped and unpacked.  Small meshes: the pack kernels read and write the
+// mapped buffer themselves.  Large ones: in pieces (HostPieces) through the
+// device's canonical buffer by the copy engine, which moves the same bytes a
+// second (209 GB/s in, 191 out) without holding SM resources.
+template <class T>
+static int erk_run_pinned(hho_ops* ops, const hho_tableau* tab, double t0, double dt, int64_t nsteps,
+                          double* h_canonical, double* m_canonical, T* dst, cudaStream_t st) {
     const char* who = "hho_erk_run_host";
+    const int nc = (int)ops->nc;
+    if (nc == 0) return HHO_OK;
+    const int blocks = (nc + STAGED_CELLS - 1) / STAGED_CELLS, np = host_pieces(ops, nsteps);
+    if (np == 1) {
+        int rc = launch_host_pack<T>(ops, m_canonical, dst, 0, blocks, st);
+        if (!rc) rc = erk_run<T>(ops, tab, t0, dt, nsteps, 1, dst, (T*)ops->d_host_work, nullptr, st, who);
+        return rc ? rc : launch_host_unpack<T>(ops, dst, m_canonical, 0, blocks, st);
+    }
+    const HostPieces& cut = ops->host_pieces;
+    HostPipe* p = host_pipe(ops);
+    if (!p) {
+        cudaGetLastError();
+        hho_set_error("%s: stream or event creation failed", who);
+        return HHO_ECUDA;
+    }
+    auto ok = [&](cudaError_t e) {
+        if (e != cudaSuccess) hho_set_error("%s: %s", who, cudaGetErrorString(e));
+        return e == cudaSuccess;
+    };
+    double* canon = ops->d_host_canon;
+    auto bytes = [&](int c) { return sizeof(double) * (size_t)(cut.off[c + 1] - cut.off[c]); };
+    PieceHooks hooks{[&](int c) -> int {   // host piece c arrives
+                         if (!ok(cudaStreamWaitEvent(st, p->in[c], 0))) return HHO_ECUDA;
+                         return launch_host_pack<T>(ops, canon, dst, cut.blocks[c], cut.blocks[c + 1] - cut.blocks[c], st);
+                     },
+                     [&](int c) -> int {   // and leaves
+                         const int rc = launch_host_unpack<T>(ops, dst, canon, cut.blocks[c],
+                                                              cut.blocks[c + 1] - cut.blocks[c], st);
+                         if (rc) return rc;
+                         if (!ok(cudaEventRecord(p->out[c], st)) || !ok(cudaStreamWaitEvent(p->copy, p->out[c], 0)) ||
+                             !ok(cudaMemcpyAsync(h_canonical + cut.off[c], canon + cut.off[c], bytes(c),
+                                                 cudaMemcpyDeviceToHost, p->copy)))
+                             return HHO_ECUDA;
+                         return HHO_OK;
+                     }};
+    int rc = HHO_OK;
+    if (!ok(cudaEventRecord(p->start, st)) || !ok(cudaStreamWaitEvent(p->copy, p->start, 0))) rc = HHO_ECUDA;
+    for (int c = 0; c < np && !rc; ++c)
+        if (!ok(cudaMemcpyAsync(canon + cut.off[c], h_canonical + cut.off[c], bytes(c), cudaMemcpyHostToDevice, p->copy)) ||
+            !ok(cudaEventRecord(p->in[c], p->copy)))
+            rc = HHO_ECUDA;
+    if (!rc) rc = erk_run<T>(ops, tab, t0, dt, nsteps, 1, dst, (T*)ops->d_host_work, nullptr, st, who, &hooks);
+    if (!ok(cudaStreamSynchronize(p->copy)) && !rc) rc = HHO_ECUDA;   // the buffer is the caller's again
+    return rc;
+}
+
+static int erk_run_mapped(hho_ops* ops, const hho_tableau* tab, double t0, double dt, int64_t nsteps,
+                          double* h_canonical, double* m_canonical, cudaStream_t st) {
     std::vector<StagePlan> plan;
     int nb = 0;
     if (build_plan(tab, plan, &nb) != HHO_OK) {
-        hho_set_error("%s: unsupported tableau", who);
+        hho_set_error("hho_erk_run_host: unsupported tableau");
         return HHO_EINVAL;
     }
-    const int nc = (int)ops->nc;
-    if (nc == 0) return HHO_OK;
-    const int blocks = (nc + STAGED_CELLS - 1) / STAGED_CELLS;
-    const size_t smem = sizeof(double) * STAGED_CELLS * 5 * ops->n;
-    const bool pairs = ops->arith == HHO_F32X2;
-    void* dst = pairs ? (void*)(ops->d_host_work + work_f64_part(ops, nb)) : (void*)ops->d_host_state;
-    if (pairs)
-        pack_host_kernel<f2x><<<blocks, STAGED_CELLS, smem, st>>>(ops->d_cell_dom, ops->d_cell_pos, ops->d_canon_off, nc,
-                                                                   ops->n_canonical, ops->dev.Nf, ops->dev.Ns, ops->n,
-                                                                   m_canonical, (f2x*)dst);
-    else
-        pack_host_kernel<double><<<blocks, STAGED_CELLS, smem, st>>>(ops->d_cell_dom, ops->d_cell_pos, ops->d_canon_off,
-                                                                      nc, ops->n_canonical, ops->dev.Nf, ops->dev.Ns,
-                                                                      ops->n, m_canonical, (double*)dst);
-    int rc = check_launch(who);
-    if (rc) return rc;
-    rc = pairs ? erk_run<f2x>(ops, tab, t0, dt, nsteps, 1, (f2x*)dst, (f2x*)ops->d_host_work, nullptr, st, who)
-               : erk_run<double>(ops, tab, t0, dt, nsteps, 1, (double*)dst, ops->d_host_work, nullptr, st, who);
-    if (rc) return rc;
-    if (pairs)
-        unpack_host_kernel<f2x><<<blocks, STAGED_CELLS, smem, st>>>(ops->d_cell_dom, ops->d_cell_pos, ops->d_canon_off,
-                                                                     nc, ops->n_canonical, ops->dev.Nf, ops->dev.Ns,
-                                                                     ops->n, (const f2x*)dst, m_canonical);
-    else
-        unpack_host_kernel<double><<<blocks, STAGED_CELLS, smem, st>>>(ops->d_cell_dom, ops->d_cell_pos,
-                                                                        ops->d_canon_off, nc, ops->n_canonical,
-                                                                        ops->dev.Nf, ops->dev.Ns, ops->n,
-                                                                        (const double*)dst, m_canonical);
-    return check_launch(who);
+    if (ops->arith == HHO_F32X2)
+        return erk_run_pinned<f2x>(ops, tab, t0, dt, nsteps, h_canonical, m_canonical,
+                                   (f2x*)(ops->d_host_work + work_f64_part(ops, nb)), st);
+    return erk_run_pinned<double>(ops, tab, t0, dt, nsteps, h_canonical, m_canonical, ops->d_host_state, st);
 }
 
 extern "C" int hho_set_launch_mode(hho_ops* ops, int32_t mode) {
@@ -1320,12 +1442,13 @@ extern "C" int hho_erk_run_host(hho_ops* ops, const hho_tableau* tab, double t0,
         }
     }
     // A pinned host buffer mapped into the device's address space is read
-    // and written by the pack kernels directly (over NVLink-C2C on GB300);
-    // any other host memory goes through a staging copy.
+    // and written by the pack kernels directly (over NVLink-C2C on GB300) or,
+    // on large meshes, copied in overlapping pieces; any other host memory goes
+    // through one staging copy.
     cudaPointerAttributes pa;
     if (cudaPointerGetAttributes(&pa, h_canonical) == cudaSuccess && pa.type == cudaMemoryTypeHost &&
         pa.devicePointer) {
-        rc = erk_run_mapped(ops, tab, t0, dt, nsteps, (double*)pa.devicePointer, st);
+        rc = erk_run_mapped(ops, tab, t0, dt, nsteps, h_canonical, (double*)pa.devicePointer, st);
         if (rc) return rc;
         if (cudaStreamSynchronize(st) != cudaSuccess) {
             hho_set_error("hho_erk_run_host: %s", cudaGetErrorString(cudaGetLastError()));

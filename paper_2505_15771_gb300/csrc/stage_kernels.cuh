@@ -1574,7 +1574,7 @@ size_t stage_smem_bytes(int max_nf, int threads) {
 template <class T, int K, int MODE>
 __global__ void __launch_bounds__(128, MinBlocks<T, K>::value) stage_kernel(const StageArgsT<T> A) {
     // the last cells first: solid cells are the longer ones and should not make the tail
-    const int gq = (gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x;
+    const int gq = 32 * A.warp0 + (gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x;
     const int shot = blockIdx.y;
     wait_for_predecessor();
     const T* cd = nullptr;
@@ -1722,9 +1722,9 @@ HHO_TEAM_RULE(float, 3, 10, 1250, 1700, 0, 200, 1200);
 
 // Warps of a team block for this launch, 0 for the thread form.
 template <class T, int K, int MODE>
-int team_warps(const DevOps& op, int n_shots) {
+int team_warps(const DevOps& op, int warps, int n_shots) {
     using R = TeamRule<T, K>;
-    const int64_t cells = op.n_warps_f + op.n_warps_s, groups = cells * n_shots;
+    const int64_t cells = op.n_warps_f + op.n_warps_s, groups = (int64_t)warps * n_shots;
     const bool gen = 4 * (cells - op.n_warps_rect) >= cells;
     const int limit = MODE == MODE_TRACES ? (gen ? R::tr_gen : R::tr_rect) : MODE == MODE_APPLY ? R::app : gen ? R::gen : R::rect;
     if (groups > limit || op.max_nf > 32 || sizeof(T) * team_smem_elems<T, K>(op.max_nf) > 200 * 1024) return 0;
@@ -1733,16 +1733,17 @@ int team_warps(const DevOps& op, int n_shots) {
 
 template <class T, int K, int MODE>
 void launch_stage(const StageArgsT<T>& a, int n_shots, cudaStream_t s) {
-    const int W = team_warps<T, K, MODE>(a.op, n_shots);
+    const int warps = a.n_warps ? a.n_warps : a.op.n_warps_f + a.op.n_warps_s;
+    const int W = team_warps<T, K, MODE>(a.op, warps, n_shots);
     auto team = [&](auto wc) {
         constexpr int TW = decltype(wc)::value;
         const size_t smem = sizeof(T) * team_smem_elems<T, K>(a.op.max_nf);
         stage_smem_attributes<TeamTag<T, K, MODE, TW>>(team_kernel<T, K, MODE, TW>, smem, true);
-        launch_dependent(team_kernel<T, K, MODE, TW>, dim3(a.op.n_warps_f + a.op.n_warps_s, n_shots), 32 * TW, smem, s, a);
+        launch_dependent(team_kernel<T, K, MODE, TW>, dim3(warps, n_shots), 32 * TW, smem, s, a);
     };
     if (W == 4) return team(std::integral_constant<int, 4>());
     if (W) return team(std::integral_constant<int, TeamRule<T, K>::W>());
-    const int cells = a.op.Nf + a.op.Ns, threads = stage_threads((int64_t)(cells / 32) * n_shots);
+    const int cells = 32 * warps, threads = stage_threads((int64_t)warps * n_shots);
     const size_t smem = stage_smem_bytes<T, K>(a.op.max_nf, threads);
     stage_smem_attributes<StageTag<T, K, MODE>>(stage_kernel<T, K, MODE>, smem, AccSmem<T, K>::value);
     launch_dependent(stage_kernel<T, K, MODE>, dim3((cells + threads - 1) / threads, n_shots), threads, smem, s, a);

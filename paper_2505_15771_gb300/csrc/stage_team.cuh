@@ -468,7 +468,7 @@ template <class T, int K, int MODE, int W>
 __global__ void __launch_bounds__(32 * W, 32 / W) team_kernel(const StageArgsT<T> A) {
     extern __shared__ __align__(16) unsigned char stage_smem[];
     T* smem = reinterpret_cast<T*>(stage_smem);
-    const int gw = gridDim.x - 1 - blockIdx.x;   // solid cells, the longer ones, first
+    const int gw = A.warp0 + gridDim.x - 1 - blockIdx.x;   // solid cells, the longer ones, first
     if (gw < A.op.n_warps_f) team_cells<T, K, MODE, W, false>(A, gw, blockIdx.y, smem);
     else team_cells<T, K, MODE, W, true>(A, gw, blockIdx.y, smem);
 }
