@@ -1550,7 +1550,7 @@ __device__ __forceinline__ void solid_cell(const StageArgsT<T>& A, int q, int sh
 // blocks, FP32 k = 3 (16 hybrid shots) 8: 866, 6: 849, 5: 862, 4: 903; FP32 k = 2
 // (21 hanging shots) 12: 309, 10: 283, 8: 260, 6: 260, 5: 277; double-float k = 2
 // (1024 x 512) 6: 177, 5: 172, 4: 182; FP64 k = 2 8: 225, 6: 224, 5: 225; FP64
-// k = 3 (680 x 340 hybrid) 8: 291, 6: 286, 5: 284.  Where the accumulators sit in
+// k = 3 (680 x 340 hybrid) 8: 291, 6: 286, 5: 284, 4: 276, 3: 276.  Where the accumulators sit in
 // shared memory (AccSmem) it may cap the resident blocks below this count.
 template <class T, int K>
 struct MinBlocks {

@@ -24,7 +24,7 @@ struct StageTuning {
 };
 
 // tune.py: begin tables
-constexpr StageTuning TUNED_F64 = {{8, 6, 5}, {0, 1, 0}, {0, 0, 0}, {0, 0, 0}};
+constexpr StageTuning TUNED_F64 = {{8, 6, 4}, {0, 1, 0}, {0, 0, 0}, {0, 0, 0}};
 constexpr StageTuning TUNED_F32 = {{8, 8, 6}, {0, 1, 1}, {50, 51, 51}, {0, 0, 0}};
 constexpr StageTuning TUNED_F2X = {{8, 5, 5}, {0, 1, 0}, {0, 34, 0}, {1, 1, 1}};
 // tune.py: end tables
