@@ -238,9 +238,10 @@ int hho_set_arithmetic(hho_ops* ops, int32_t arith);
  *     Ricker wavelets come from a clock in device memory, so the replayed
  *     kernels have identical arguments.  The graph is captured again when the
  *     arguments of a step change (buffers, tableau, dt, sources, receivers);
- *   HHO_LAUNCH_AUTO (default): graphs when a stage grid has at most 2048
- *     blocks (about 260,000 cells x shots) and a call has at least 8 steps,
- *     where launch overhead matters, else stream launches.
+ *   HHO_LAUNCH_AUTO (default): the faster of the two, which is stream
+ *     launches at every size measured (consecutive stages overlap across
+ *     steps there); graphs leave the host free, so they are there to be asked
+ *     for.
  * Stage profiling (hho_profile_enable) always uses stream launches.  Device
  * and host evaluate the wavelet's exponential separately, so the two modes
  * agree to rounding (about 1e-16 relative), not bit for bit.  HHO_EINVAL for
@@ -349,7 +350,7 @@ int hho_sdirk_work_size(const hho_ops* ops, const hho_tableau* tab, int32_t rest
  * operator applications per stage) to ||r|| <= tol ||rhs||; the operator is
  * the stage kernel of hho_erk_step in FP64 (hho_set_arithmetic does not
  * apply).  h_iterations (host, may be NULL) receives the total number of
- * operator applications inside GMRES.  Synchronises the stream once per
+ * operator applications inside GMRES.  Waits for the device once per
  * Krylov vector (the Hessenberg matrix and the Givens rotations live on the
  * host).  HHO_ENOCONV if a stage misses tol within max_iter (d_state then
  * holds the steps completed so far); HHO_EINVAL for a tableau that is not

@@ -524,10 +524,13 @@ struct HostPipe {
     cudaEvent_t start = nullptr, in[HostPieces::MAX] = {}, out[HostPieces::MAX] = {};
 };
 
-// Whether erk_run replays the step as a graph (blocks: of 128 cells, all shots).
-static bool uses_graph(const hho_ops* ops, int64_t blocks, int64_t nsteps) {
-    return !ops->prof_on && ops->d_clock && !ops->src_sampled &&
-           (ops->launch_mode == HHO_LAUNCH_GRAPH || (ops->launch_mode == HHO_LAUNCH_AUTO && blocks <= 2048 && nsteps >= 8));
+// Whether erk_run replays the step as a graph.  AUTO does not: consecutive stages
+// of a stream are dependent launches that overlap across steps too, while a graph
+// ends with its step, and the host launches a stage in less time than the
+// smallest one runs (512 triangles, k = 1, four stages and a record: 28.2 us a
+// step launched, 34.9 replayed).
+static bool uses_graph(const hho_ops* ops) {
+    return !ops->prof_on && ops->d_clock && !ops->src_sampled && ops->launch_mode == HHO_LAUNCH_GRAPH;
 }
 
 // A call that takes its state and hands it back in pieces (HostPieces): arrive(c)
@@ -604,7 +607,7 @@ static int erk_run(hho_ops* ops, const hho_tableau* tab, double t0, double dt, i
     a.inp = d_state;
     a.tr_out = tr[0];
     a.n_tgt = 0;
-    const bool use_graph = uses_graph(ops, (int64_t)grid.x * n_shots, nsteps);
+    const bool use_graph = uses_graph(ops);
     const StageArgsT<T> traces = a;
     int rc = HHO_OK;
     if (!pieces) {
@@ -802,7 +805,7 @@ void free_host_pipe(HostPipe* p) {
 }
 
 static int host_pieces(const hho_ops* ops, int64_t nsteps) {
-    if (nsteps < 1 || ops->prof_on || uses_graph(ops, (ops->dev.Nf + ops->dev.Ns + 127) / 128, nsteps)) return 1;
+    if (nsteps < 1 || ops->prof_on || uses_graph(ops)) return 1;
     return ops->host_pieces.n;
 }
 

@@ -358,12 +358,11 @@ __device__ __forceinline__ void lift_apply(const T* __restrict__ L, const T* j, 
 // registers they do not fit the 64-register budget of 8 resident blocks and
 // spill to local memory, whose footprint (over 400 bytes a thread) exceeds
 // L1.  With AccSmem the block's dynamic shared memory holds them instead,
-// thread-major with an odd stride in elements (no bank conflicts).  That
-// makes the FP32 kernel about 20 % faster at k = 3 (still 8 blocks).  For
-// 8-byte values the shared memory allows at most 6 blocks: the double-float
-// k = 2 kernel at 5 blocks (96 registers, no spills) with prefetched target
-// sources is 7 % faster than with 8 blocks and spills; the FP64 kernel, bound
-// by its FP64 pipe, and double-float k = 3 (4 blocks) gain nothing.
+// thread-major with an odd stride in elements (no bank conflicts).  That made
+// the FP32 kernel about 20 % faster at k = 3 and the double-float one 7 % at
+// k = 2.  FP64 is indifferent (k = 2, 1024 x 512: 224.0 us either way; k = 3 at
+// 4 blocks, 680 x 340 hybrid: 275.6 us against 275.7 in registers), and
+// double-float k = 3 gains nothing (4 blocks).
 template <class T>
 struct Tuned;
 template <>
