@@ -725,9 +725,9 @@ def measure_e2e(a, torch, hho, P, dt, stream, arith, world):
     el = time.perf_counter() - t0
     return {"value": world * ndof * a.stages * ne / el, "unit": UNIT, "h2d_bytes_per_step": 8 * ndof,
             "d2h_bytes_per_step": 8 * ndof, "steps": ne, "arith": "f64" if arith == hho.HHO_F64 else "f32x2",
-            "path": "hho_erk_run_host on a pinned host buffer: the pack kernel reads the canonical state from "
-                    "host memory (NVLink-C2C), 1 ERK step, the unpack kernel writes it back to host memory, "
-                    "stream sync"}
+            "path": "hho_erk_run_host on a pinned host buffer: the canonical state is copied or packed from host "
+                    "memory (NVLink-C2C), 1 ERK step, and back to host memory (large meshes in pieces that overlap "
+                    "the first and the last stage), stream sync"}
 
 
 RANDOM_STATE_SEED = 11
