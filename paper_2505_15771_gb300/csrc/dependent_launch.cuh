@@ -4,6 +4,13 @@
 // anything that it reads or writes.  A step of a small mesh is a chain of short
 // kernels, and the launch latency between two of them is a good part of it.
 // Without the attribute both instructions do nothing.
+//
+// Such a kernel is resident while the kernel before it still writes, so what any
+// kernel writes (states, traces, partial sums, clocks) is read with ordinary
+// coherent loads after the wait.  The read-only path (__ldg, or a const
+// __restrict__ kernel parameter, which the compiler may take as one) is for the
+// operator's tables, uploaded by blocking copies before any launch: its loads need
+// data that stay the same for the kernel's whole life, and no wait orders them.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -250,7 +250,7 @@ constexpr int REC_MAX_N = 10;
 inline int record_threads(int n) { return (REC_FIELDS * n + 31) / 32 * 32; }
 template <class T, class TO = T>
 __global__ void record_kernel(DevOps op, int n_rec, const int32_t* __restrict__ ri, const double* __restrict__ rd,
-                              const T* __restrict__ state, int64_t n_state, TO* out, StageClock* clock = nullptr) {
+                              const T* state, int64_t n_state, TO* out, StageClock* clock = nullptr) {
     __shared__ double val[REC_FIELDS][REC_MAX_N], field[REC_FIELDS], flux[3];
     const int r = blockIdx.x, n = op.n, t = threadIdx.x;
     const double* d = rd + (size_t)r * (2 * n + 15);

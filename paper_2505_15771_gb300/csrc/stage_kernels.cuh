@@ -398,7 +398,7 @@ __device__ __forceinline__ void add_signed(const T* x, T* y, int s) {
 }
 
 template <int NV, class T>
-__device__ __forceinline__ void load_state(const T* __restrict__ src, int N, int q, int first, T* u) {
+__device__ __forceinline__ void load_state(const T* src, int N, int q, int first, T* u) {
 #pragma unroll
     for (int i = 0; i < NV; ++i) u[i] = src[(size_t)(first + i) * N + q];
 }
@@ -691,7 +691,7 @@ __device__ __forceinline__ W face_inner(const W* a, const W* b, W acc) {
 // published traces tr (fluid part then solid part) and interface
 // coefficients `co6`; NC = 1 component in a fluid cell, 2 in a solid cell.
 template <class T, int K, int NC, class W>
-__device__ __forceinline__ void wide_jump(const DevOps& op, const T* __restrict__ tr, const double* __restrict__ co6,
+__device__ __forceinline__ void wide_jump(const DevOps& op, const T* tr, const double* co6,
                                           int slot, int nb, W* jmp) {
     constexpr int f = Dims<K>::f;
     const size_t S = NC == 1 ? op.SF : op.SS;
@@ -699,12 +699,12 @@ __device__ __forceinline__ void wide_jump(const DevOps& op, const T* __restrict_
     const T* trs = tr + (size_t)2 * f * op.SF;
     const T* own = NC == 1 ? trf : trs;
 #pragma unroll
-    for (int i = 0; i < NC * f; ++i) jmp[i] = widen(__ldg(own + (NC * f + i) * S + slot));
+    for (int i = 0; i < NC * f; ++i) jmp[i] = widen(own[(NC * f + i) * S + slot]);
     if (nb >= 0) {
         const W be = __ldg((NC == 1 ? WideData<T>::beta_f(op) : WideData<T>::beta_s(op)) + slot);
 #pragma unroll
         for (int i = 0; i < NC * f; ++i) {
-            const W w = widen(__ldg(own + i * S + nb));
+            const W w = widen(own[i * S + nb]);
             jmp[i] = ((i % f) & 1) ? fma(-be, w, jmp[i]) : fma(be, w, jmp[i]);
         }
     } else if (nb < NB_BOUNDARY) {
@@ -715,14 +715,14 @@ __device__ __forceinline__ void wide_jump(const DevOps& op, const T* __restrict_
             const W bx(__ldg(co + 1)), by(__ldg(co + 2));
 #pragma unroll
             for (int l = 0; l < f; ++l) {
-                const W ws = fma(bx, widen(__ldg(trs + (size_t)l * op.SS + no)), by * widen(__ldg(trs + (size_t)(f + l) * op.SS + no)));
+                const W ws = fma(bx, widen(trs[(size_t)l * op.SS + no]), by * widen(trs[(size_t)(f + l) * op.SS + no]));
                 jmp[l] = (l & 1) ? jmp[l] - ws : jmp[l] + ws;
             }
         } else {
             const W b0(__ldg(co + 4)), b1(__ldg(co + 5));
 #pragma unroll
             for (int l = 0; l < f; ++l) {
-                const W w = widen(__ldg(trf + (size_t)l * op.SF + no));
+                const W w = widen(trf[(size_t)l * op.SF + no]);
                 jmp[l] = (l & 1) ? fma(-b0, w, jmp[l]) : fma(b0, w, jmp[l]);
                 jmp[f + l] = (l & 1) ? fma(-b1, w, jmp[f + l]) : fma(b1, w, jmp[f + l]);
             }
@@ -861,12 +861,12 @@ __device__ __forceinline__ void fluid_face_jump(const StageArgsT<T>& A, const Ce
     const int slot = c.sbase + j * c.npad + c.lq;
     const int nb = __ldg(op.nb_f + slot);
 #pragma unroll
-    for (int l = 0; l < f; ++l) jmp[l] = __ldg(c.trf_in + (size_t)(f + l) * c.SF + slot);
+    for (int l = 0; l < f; ++l) jmp[l] = c.trf_in[(size_t)(f + l) * c.SF + slot];
     if (nb >= 0) {
         const T be = __ldg(OpData<T>::beta_f(op) + slot);
 #pragma unroll
         for (int l = 0; l < f; ++l) {
-            const T w = __ldg(c.trf_in + (size_t)l * c.SF + nb);
+            const T w = c.trf_in[(size_t)l * c.SF + nb];
             jmp[l] = (l & 1) ? fma(-be, w, jmp[l]) : fma(be, w, jmp[l]);
         }
     } else if (nb < NB_BOUNDARY) {
@@ -876,7 +876,7 @@ __device__ __forceinline__ void fluid_face_jump(const StageArgsT<T>& A, const Ce
         const T bx = __ldg(co + 1), by = __ldg(co + 2);
 #pragma unroll
         for (int l = 0; l < f; ++l) {
-            const T ws = fma(bx, __ldg(c.trs_in + (size_t)l * c.SS + ns), by * __ldg(c.trs_in + (size_t)(f + l) * c.SS + ns));
+            const T ws = fma(bx, c.trs_in[(size_t)l * c.SS + ns], by * c.trs_in[(size_t)(f + l) * c.SS + ns]);
             jmp[l] = (l & 1) ? jmp[l] - ws : jmp[l] + ws;
         }
     }
@@ -1031,7 +1031,7 @@ __device__ __forceinline__ void fluid_rect_traces(const StageArgsT<T>& A, const 
 // k = tau k + da/dX + db/dY.  The flux is loaded here, after the faces, so that
 // the face loop holds neither it nor its derivatives.
 template <class T, int K>
-__device__ __forceinline__ void fp64_rect_div(const T* __restrict__ inp, const CellCtx<T>& c, int fa, int fb, T* k) {
+__device__ __forceinline__ void fp64_rect_div(const T* inp, const CellCtx<T>& c, int fa, int fb, T* k) {
     constexpr int n = Dims<K>::n;
     T a[n], b[n], d[n];
     load_state<n>(inp, c.N, c.q, fa, a);
@@ -1164,15 +1164,15 @@ __device__ __forceinline__ void solid_face_jump(const StageArgsT<T>& A, const Ce
     const int nb = __ldg(op.nb_s + slot);
 #pragma unroll
     for (int l = 0; l < f; ++l) {
-        jx[l] = __ldg(c.trs_in + (size_t)(2 * f + l) * c.SS + slot);
-        jy[l] = __ldg(c.trs_in + (size_t)(3 * f + l) * c.SS + slot);
+        jx[l] = c.trs_in[(size_t)(2 * f + l) * c.SS + slot];
+        jy[l] = c.trs_in[(size_t)(3 * f + l) * c.SS + slot];
     }
     if (nb >= 0) {
         const T be = __ldg(OpData<T>::beta_s(op) + slot);
 #pragma unroll
         for (int l = 0; l < f; ++l) {
-            const T wx = __ldg(c.trs_in + (size_t)l * c.SS + nb);
-            const T wy = __ldg(c.trs_in + (size_t)(f + l) * c.SS + nb);
+            const T wx = c.trs_in[(size_t)l * c.SS + nb];
+            const T wy = c.trs_in[(size_t)(f + l) * c.SS + nb];
             jx[l] = (l & 1) ? fma(-be, wx, jx[l]) : fma(be, wx, jx[l]);
             jy[l] = (l & 1) ? fma(-be, wy, jy[l]) : fma(be, wy, jy[l]);
         }
@@ -1183,7 +1183,7 @@ __device__ __forceinline__ void solid_face_jump(const StageArgsT<T>& A, const Ce
         const T b0 = __ldg(co + 4), b1 = __ldg(co + 5);
 #pragma unroll
         for (int l = 0; l < f; ++l) {
-            const T wf = __ldg(c.trf_in + (size_t)l * c.SF + nfs);
+            const T wf = c.trf_in[(size_t)l * c.SF + nfs];
             jx[l] = (l & 1) ? fma(-b0, wf, jx[l]) : fma(b0, wf, jx[l]);
             jy[l] = (l & 1) ? fma(-b1, wf, jy[l]) : fma(b1, wf, jy[l]);
         }

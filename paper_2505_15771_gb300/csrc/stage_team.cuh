@@ -56,11 +56,11 @@ __device__ __forceinline__ void team_jump(const StageArgsT<T>& A, const T* trf, 
     const int nb = __ldg((SOLID ? op.nb_s : op.nb_f) + slot);
     const T be = __ldg((SOLID ? OpData<T>::beta_s(op) : OpData<T>::beta_f(op)) + slot);   // 0 on boundary and interface
 #pragma unroll
-    for (int l = 0; l < f; ++l) jmp[l] = __ldg(om + (size_t)l * S + slot);
+    for (int l = 0; l < f; ++l) jmp[l] = om[(size_t)l * S + slot];
     if (nb >= 0) {
 #pragma unroll
         for (int l = 0; l < f; ++l) {
-            const T w = __ldg(w0 + (size_t)l * S + nb);
+            const T w = w0[(size_t)l * S + nb];
             jmp[l] = (l & 1) ? fma(-be, w, jmp[l]) : fma(be, w, jmp[l]);
         }
     } else if (nb < NB_BOUNDARY) {
@@ -70,11 +70,11 @@ __device__ __forceinline__ void team_jump(const StageArgsT<T>& A, const T* trf, 
 #pragma unroll
         for (int l = 0; l < f; ++l) {
             if constexpr (SOLID) {
-                const T b = __ldg(co + 4 + comp), wf = __ldg(trf + (size_t)l * op.SF + no);
+                const T b = __ldg(co + 4 + comp), wf = trf[(size_t)l * op.SF + no];
                 jmp[l] = (l & 1) ? fma(-b, wf, jmp[l]) : fma(b, wf, jmp[l]);
             } else {
-                const T ws = fma(__ldg(co + 1), __ldg(trs + (size_t)l * op.SS + no),
-                                 __ldg(co + 2) * __ldg(trs + (size_t)(f + l) * op.SS + no));
+                const T ws = fma(__ldg(co + 1), trs[(size_t)l * op.SS + no],
+                                 __ldg(co + 2) * trs[(size_t)(f + l) * op.SS + no]);
                 jmp[l] = (l & 1) ? jmp[l] - ws : jmp[l] + ws;
             }
         }
