@@ -265,7 +265,9 @@ __global__ void record_kernel(DevOps op, int n_rec, const int32_t* __restrict__ 
     int64_t step = 0;
     if (clock && t == 0) {
         step = *(volatile int64_t*)&clock->step;
+        __threadfence();   // the read comes before the ticket that lets the last block write
         if (atomicAdd(&clock->ticket, 1u) == gridDim.x * gridDim.y - 1) {   // every block has read it
+            __threadfence();
             clock->ticket = 0;
             clock->step = step + 1;
         }

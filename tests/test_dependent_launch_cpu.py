@@ -54,3 +54,19 @@ def test_dependent_kernels_take_no_restrict_pointer_to_written_data():
         assert restrict <= TABLE_PARAMS, (k, restrict)
         body = src[f][m.end():]
         assert "wait_for_predecessor" in body or k == "team_kernel"
+
+
+@pytest.mark.parametrize("name,count", [("stage.cu", 1), ("sdirk.cu", 1)])
+def test_ticket_counters_are_fenced_on_both_sides(name, count):
+    """The last block to take a ticket overwrites (the device clock) or reads
+    (the partial sums) what the others read or wrote before theirs: without a
+    fence on each side of the ticket a block's access may pass it."""
+    src = text(name)
+    tickets = list(re.finditer(r"atomicAdd\([^,]*ticket", src))
+    assert len(tickets) == count
+    for m in tickets:
+        kernel = src[src.rindex("__global__", 0, m.start()):]
+        at = m.start() - (len(src) - len(kernel))
+        before = re.split(r"clock->step|A\.partial", kernel[:at])[-1]
+        after = re.split(r"clock->step|A\.partial", kernel[at:])[0]
+        assert "__threadfence()" in before and "__threadfence()" in after
