@@ -16,6 +16,7 @@
 #include "dependent_launch.cuh"
 #include "f2x.cuh"
 #include "hho_internal.h"
+#include "host_buffers.h"
 #include "stage_launch.h"
 
 namespace {
@@ -1414,38 +1415,10 @@ extern "C" int hho_record(hho_ops* ops, const double* d_state, double* d_out, vo
     return check_launch("hho_record");
 }
 
-extern "C" int hho_erk_run_host(hho_ops* ops, const hho_tableau* tab, double t0, double dt, int64_t nsteps,
-                                double* h_canonical, void* stream) {
-    if (!ops || !tab || !h_canonical) {
-        hho_set_error("hho_erk_run_host: null pointer");
-        return HHO_EINVAL;
-    }
-    int64_t wsz = 0;
-    int rc = hho_work_size(ops, tab, &wsz);
-    if (rc) return rc;
-    if (!ops->d_host_state) {
-        if (cudaMalloc((void**)&ops->d_host_state, sizeof(double) * ops->n_state) != cudaSuccess ||
-            cudaMalloc((void**)&ops->d_host_canon, sizeof(double) * ops->n_canonical) != cudaSuccess) {
-            hho_set_error("hho_erk_run_host: device allocation failed");
-            return HHO_ENOMEM;
-        }
-    }
+// The call on buffers that are ready; returns with work queued on st where it fails.
+static int erk_run_host(hho_ops* ops, const hho_tableau* tab, double t0, double dt, int64_t nsteps, double* h_canonical,
+                        void* stream) {
     cudaStream_t st = (cudaStream_t)stream;
-    if (ops->host_work_size < wsz) {
-        if (ops->d_host_work) cudaFree(ops->d_host_work);
-        ops->d_host_work = nullptr;
-        if (cudaMalloc((void**)&ops->d_host_work, sizeof(double) * wsz) != cudaSuccess) {
-            hho_set_error("hho_erk_run_host: device allocation failed");
-            return HHO_ENOMEM;
-        }
-        ops->host_work_size = wsz;
-        // the mapped path leaves padding slots of its states unwritten
-        if (cudaMemsetAsync(ops->d_host_work, 0, sizeof(double) * wsz, st) != cudaSuccess ||
-            cudaMemsetAsync(ops->d_host_state, 0, sizeof(double) * ops->n_state, st) != cudaSuccess) {
-            hho_set_error("hho_erk_run_host: device memset failed");
-            return HHO_ECUDA;
-        }
-    }
     // A pinned host buffer mapped into the device's address space is read
     // and written by the pack kernels directly (over NVLink-C2C on GB300) or,
     // on large meshes, copied in overlapping pieces; any other host memory goes
@@ -1453,7 +1426,7 @@ extern "C" int hho_erk_run_host(hho_ops* ops, const hho_tableau* tab, double t0,
     cudaPointerAttributes pa;
     if (cudaPointerGetAttributes(&pa, h_canonical) == cudaSuccess && pa.type == cudaMemoryTypeHost &&
         pa.devicePointer) {
-        rc = erk_run_mapped(ops, tab, t0, dt, nsteps, h_canonical, (double*)pa.devicePointer, st);
+        const int rc = erk_run_mapped(ops, tab, t0, dt, nsteps, h_canonical, (double*)pa.devicePointer, st);
         if (rc) return rc;
         if (cudaStreamSynchronize(st) != cudaSuccess) {
             hho_set_error("hho_erk_run_host: %s", cudaGetErrorString(cudaGetLastError()));
@@ -1467,7 +1440,7 @@ extern "C" int hho_erk_run_host(hho_ops* ops, const hho_tableau* tab, double t0,
         hho_set_error("hho_erk_run_host: host-to-device copy failed");
         return HHO_ECUDA;
     }
-    rc = hho_state_pack(ops, ops->d_host_canon, ops->d_host_state, stream);
+    int rc = hho_state_pack(ops, ops->d_host_canon, ops->d_host_state, stream);
     if (rc) return rc;
     rc = hho_erk_step(ops, tab, t0, dt, nsteps, ops->d_host_state, ops->d_host_work, stream);
     if (rc) return rc;
@@ -1480,6 +1453,34 @@ extern "C" int hho_erk_run_host(hho_ops* ops, const hho_tableau* tab, double t0,
         return HHO_ECUDA;
     }
     return HHO_OK;
+}
+
+extern "C" int hho_erk_run_host(hho_ops* ops, const hho_tableau* tab, double t0, double dt, int64_t nsteps,
+                                double* h_canonical, void* stream) {
+    if (!ops || !tab || !h_canonical) {
+        hho_set_error("hho_erk_run_host: null pointer");
+        return HHO_EINVAL;
+    }
+    int64_t wsz = 0;
+    int rc = hho_work_size(ops, tab, &wsz);
+    if (rc) return rc;
+    cudaStream_t st = (cudaStream_t)stream;
+    rc = grow_host_buffers(
+        ops, wsz,
+        [](size_t n) {
+            double* p = nullptr;
+            if (cudaMalloc((void**)&p, sizeof(double) * std::max<size_t>(n, 1)) == cudaSuccess) return p;
+            cudaGetLastError();   // reported here; not for the next launch to find
+            return (double*)nullptr;
+        },
+        [](double* p) { cudaFree(p); },
+        [&](double* p, size_t n) { return cudaMemsetAsync(p, 0, sizeof(double) * n, st) == cudaSuccess; });
+    if (rc == HHO_ENOMEM) hho_set_error("hho_erk_run_host: device allocation failed");
+    if (rc == HHO_ECUDA) hho_set_error("hho_erk_run_host: device memset failed");
+    if (rc) return rc;
+    rc = erk_run_host(ops, tab, t0, dt, nsteps, h_canonical, stream);
+    if (rc) cudaStreamSynchronize(st);   // the next call may come on another stream; the buffers are free for it
+    return rc;
 }
 
 extern "C" int hho_cfl_bracket(hho_ops* ops, const hho_tableau* tab, const double* d_state0, double T_f,
