@@ -527,7 +527,8 @@ def measure_adjoint(a, torch, hho):
            "gradient_finite": bool(np.isfinite(grad).all()), "dtype": "f64",
            "fp32": {"gradient_ms": adj32_ms, "value": ndof * 4 * nsteps / (adj32_ms * 1e-3),
                     "rel_diff_vs_fp64": float(np.linalg.norm(grad32 - grad) / np.linalg.norm(grad)),
-                    "note": "hho_adjoint_vjp_f32: FP32 stage kernels and adjoint vectors, FP64 gradient sums"}}
+                    "note": "hho_adjoint_vjp_f32: FP32 stage kernels and adjoint vectors, a cell's products in "
+                            "double-float, FP64 sums over the stages"}}
     hho.hho_ops_destroy(ops)
     return out
 

@@ -528,8 +528,10 @@ int hho_adjoint_vjp(hho_ops* ops, const hho_tableau* tab, double t0, double dt, 
  * stage kernels (the batched FP32 path with one shot) for the forward
  * checkpoints, the segment recompute and the transposed stages; states,
  * traces, adjoint vectors, d_state0 and d_cotangent ([nsteps][n_rec][5]) in
- * FP32; the gradient sums in FP64; outputs as hho_adjoint_vjp.  d_work:
- * hho_adjoint_work_size_f32 floats. */
+ * FP32.  A cell's products of one backward stage are double-float sums (48
+ * bits) of values scaled by powers of two, so that products outside FP32's
+ * exponents count; the sums over stages and steps are FP64.  Outputs as
+ * hho_adjoint_vjp.  d_work: hho_adjoint_work_size_f32 floats. */
 int hho_adjoint_work_size_f32(const hho_ops* ops, const hho_tableau* tab, int64_t nsteps, int64_t checkpoint_every,
                               int64_t* n_floats);
 int hho_adjoint_vjp_f32(hho_ops* ops, const hho_tableau* tab, double t0, double dt, int64_t nsteps,

@@ -49,8 +49,9 @@
 //
 // Arithmetic: the driver and its kernels are templates on the state type,
 // FP64 (hho_adjoint_vjp) or FP32 (hho_adjoint_vjp_f32: the FP32 stage
-// kernels, states, traces and adjoint vectors in FP32); the gradient sums
-// are accumulated in FP64 in both.
+// kernels, states, traces and adjoint vectors in FP32).  A cell's products of one
+// backward stage are FP64 sums, or in FP32 scaled double-float ones
+// (stage_kernels.cuh, Range); the sums over stages and steps are FP64 in both.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -580,9 +580,11 @@ __device__ __forceinline__ T shot_src_value(const StageArgsT<T>& A) {
 }
 
 // ---- adjoint gradients (MODE_GRAD) ---------------------------------------------------
-// Sums of products in at least FP64 accuracy for FP64 values, and exact
-// products with double-float sums for FP32 values (FP32 pipes; an FP64 sum of
-// FP32 products would spend most of its time in conversions on the FP64 pipe).
+// A cell's sums of products: FP64 for FP64 values; for FP32 values double-float
+// (48 bits, on the FP32 pipes: an FP64 sum of FP32 products would spend most of its
+// time in conversions on the FP64 pipe) of values that are first divided by a
+// power of two near their largest (Range), which is put back in FP64: a pair has
+// FP32's exponents, and the product of two FP32 values needs FP64's.
 template <class T>
 struct Wide {
     using type = double;
@@ -591,6 +593,43 @@ template <>
 struct Wide<float> {
     using type = f2x;
 };
+// The largest magnitude of the values shown to it as a power of two: factor()
+// brings them to 4 or less (below 2^-125, to 2 or less), exponent() undoes that.
+template <class T>
+struct Range;
+template <>
+struct Range<double> {   // FP64 products stay in range unscaled
+    __device__ void add(double) {}
+    __device__ double factor() const { return 1.0; }
+    __device__ int exponent() const { return 0; }
+};
+template <>
+struct Range<float> {
+    uint32_t m = 0;
+    __device__ void add(float x) { m = max(m, __float_as_uint(x) & 0x7fffffffu); }
+    __device__ int biased() const { return min(max((int)(m >> 23), 1), 253); }
+    __device__ float factor() const { return __uint_as_float((uint32_t)(254 - biased()) << 23); }
+    __device__ int exponent() const { return biased() - 127; }
+};
+// x[0..N) divided by a power of two near the largest; returns its exponent
+template <int N, class T>
+__device__ __forceinline__ int to_unit(T* x) {
+    Range<T> r;
+#pragma unroll
+    for (int i = 0; i < N; ++i) r.add(x[i]);
+    const T s = r.factor();
+#pragma unroll
+    for (int i = 0; i < N; ++i) x[i] *= s;
+    return r.exponent();
+}
+// x 2^e, |e| < 512, for x zero, not finite, or a double-float value (no FP64 instruction)
+__device__ __forceinline__ double times_pow2(double x, int e) {
+    const int h = __double2hiint(x);
+    const uint32_t b = ((uint32_t)h >> 20) & 0x7ffu;
+    return b - 1u < 0x7feu ? __hiloint2double(h + e * (1 << 20), __double2loint(x)) : x;
+}
+__device__ __forceinline__ double leading(double x) { return x; }
+__device__ __forceinline__ float leading(f2x x) { return x.hi; }
 __device__ __forceinline__ double widen(double x) { return x; }
 __device__ __forceinline__ f2x widen(float x) { return f2x(x, 0.0f); }
 template <class T>
@@ -641,20 +680,26 @@ __device__ __forceinline__ W coef_dot(const T* x, const W* y) {
     return s;
 }
 
-// acc + z^T M0 g in the wide type for one field of a cell (z with stride N):
-// the source cells of the wavelet gradient only.
-template <class T, int K>
-__device__ __noinline__ typename Wide<T>::type wide_form(const DevOps& op, const int* ci, const T* z, int N,
-                                                         const T* g, typename Wide<T>::type acc) {
+// sum over NC fields of z^T M0 g of a cell (z with stride N): the source cells
+// of the wavelet gradient only.
+template <class T, int K, int NC>
+__device__ __noinline__ double wide_form(const DevOps& op, const int* ci, const T* z, int N, const T* g) {
     using W = typename Wide<T>::type;
     constexpr int n = Dims<K>::n;
     const W* M0 = WideData<T>::cls(op) + __ldg(ci + CI_DOFF);
-    for (int i = 0; i < n; ++i) {
-        W y(0);
-        for (int j = 0; j < n; ++j) y = fma(M0[i * n + j], widen(z[(size_t)j * N]), y);
-        acc = fma(y, widen(g[i]), acc);
+    Range<T> rz, rg;
+    for (int i = 0; i < NC * n; ++i) {
+        rz.add(z[(size_t)i * N]);
+        rg.add(g[i]);
     }
-    return acc;
+    W acc(0);
+    for (int e = 0; e < NC; ++e)
+        for (int i = 0; i < n; ++i) {
+            W y(0);
+            for (int j = 0; j < n; ++j) y = fma(M0[i * n + j], widen(z[(size_t)(e * n + j) * N] * rz.factor()), y);
+            acc = fma(y, widen(g[e * n + i] * rg.factor()), acc);
+        }
+    return times_pow2(to_f64(acc), rz.exponent() + rg.exponent());
 }
 
 // The integral over a face of unit length of the product of two functions
@@ -690,44 +735,70 @@ __device__ __forceinline__ W face_inner(const W* a, const W* b, W acc) {
 // Jump of the primal trace on local face j in the wide type, from the
 // published traces tr (fluid part then solid part) and interface
 // coefficients `co6`; NC = 1 component in a fluid cell, 2 in a solid cell.
+// Returns the exponent of the power of two that jmp is divided by (Range).
 template <class T, int K, int NC, class W>
-__device__ __forceinline__ void wide_jump(const DevOps& op, const T* tr, const double* co6,
-                                          int slot, int nb, W* jmp) {
+__device__ __forceinline__ int wide_jump(const DevOps& op, const T* tr, const double* co6, int slot, int nb, W* jmp) {
     constexpr int f = Dims<K>::f;
     const size_t S = NC == 1 ? op.SF : op.SS;
     const T* trf = tr;
     const T* trs = tr + (size_t)2 * f * op.SF;
     const T* own = NC == 1 ? trf : trs;
+    Range<T> range;
+    T om[NC * f];
 #pragma unroll
-    for (int i = 0; i < NC * f; ++i) jmp[i] = widen(own[(NC * f + i) * S + slot]);
+    for (int i = 0; i < NC * f; ++i) range.add(om[i] = own[(NC * f + i) * S + slot]);
+    auto start = [&](T s) {
+#pragma unroll
+        for (int i = 0; i < NC * f; ++i) jmp[i] = widen(om[i] * s);
+        return s;
+    };
     if (nb >= 0) {
         const W be = __ldg((NC == 1 ? WideData<T>::beta_f(op) : WideData<T>::beta_s(op)) + slot);
+        T w[NC * f];
 #pragma unroll
-        for (int i = 0; i < NC * f; ++i) {
-            const W w = widen(own[i * S + nb]);
-            jmp[i] = ((i % f) & 1) ? fma(-be, w, jmp[i]) : fma(be, w, jmp[i]);
-        }
+        for (int i = 0; i < NC * f; ++i) range.add(leading(be) * (w[i] = own[i * S + nb]));
+        const T s = start(range.factor());
+#pragma unroll
+        for (int i = 0; i < NC * f; ++i) jmp[i] = ((i % f) & 1) ? fma(-be, widen(w[i] * s), jmp[i]) : fma(be, widen(w[i] * s), jmp[i]);
     } else if (nb < NB_BOUNDARY) {
         const int r = -2 - nb;
         const int no = __ldg(op.if_nb + r);
         const double* co = co6 + 6 * r;
         if constexpr (NC == 1) {
             const W bx(__ldg(co + 1)), by(__ldg(co + 2));
+            T wx[f], wy[f];
 #pragma unroll
             for (int l = 0; l < f; ++l) {
-                const W ws = fma(bx, widen(trs[(size_t)l * op.SS + no]), by * widen(trs[(size_t)(f + l) * op.SS + no]));
+                range.add(leading(bx) * (wx[l] = trs[(size_t)l * op.SS + no]));
+                range.add(leading(by) * (wy[l] = trs[(size_t)(f + l) * op.SS + no]));
+            }
+            const T s = start(range.factor());
+#pragma unroll
+            for (int l = 0; l < f; ++l) {
+                const W ws = fma(bx, widen(wx[l] * s), by * widen(wy[l] * s));
                 jmp[l] = (l & 1) ? jmp[l] - ws : jmp[l] + ws;
             }
         } else {
             const W b0(__ldg(co + 4)), b1(__ldg(co + 5));
+            T wf[f];
 #pragma unroll
             for (int l = 0; l < f; ++l) {
-                const W w = widen(trf[(size_t)l * op.SF + no]);
+                wf[l] = trf[(size_t)l * op.SF + no];
+                range.add(leading(b0) * wf[l]);
+                range.add(leading(b1) * wf[l]);
+            }
+            const T s = start(range.factor());
+#pragma unroll
+            for (int l = 0; l < f; ++l) {
+                const W w = widen(wf[l] * s);
                 jmp[l] = (l & 1) ? fma(-b0, w, jmp[l]) : fma(b0, w, jmp[l]);
                 jmp[f + l] = (l & 1) ? fma(-b1, w, jmp[f + l]) : fma(b1, w, jmp[f + l]);
             }
         }
+    } else {
+        start(range.factor());
     }
+    return range.exponent();
 }
 
 // Stabilisation-weight part of one backward stage: gstab += w sum_F |F|/h
@@ -745,12 +816,12 @@ __device__ __forceinline__ void tau_grad(const StageArgsT<T>& A, const GradArgsT
         const int slot = c.sbase + j * c.npad + c.lq;
         const int nb = __ldg((NC == 1 ? op.nb_f : op.nb_s) + slot);
         W jy[NC * f], jz[NC * f];
-        wide_jump<T, K, NC, W>(op, A.tr_in, op.if_coef, slot, nb, jy);
-        wide_jump<T, K, NC, W>(op, G.tr_z, G.if_coef_z, slot, nb, jz);
+        const int ey = wide_jump<T, K, NC, W>(op, A.tr_in, op.if_coef, slot, nb, jy);
+        const int ez = wide_jump<T, K, NC, W>(op, G.tr_z, G.if_coef_z, slot, nb, jz);
         W sum(0);
 #pragma unroll
         for (int e = 0; e < NC; ++e) sum = face_inner<K, W>(jy + e * f, jz + e * f, sum);
-        acc = fma(__ldg(cd + j * FS + 2), double(sum), acc);   // |F| / h
+        acc = fma(__ldg(cd + j * FS + 2), times_pow2(to_f64(sum), ey + ez), acc);   // |F| / h
     }
     G.gstab[g] = fma(G.w, acc, G.gstab[g]);
 }
@@ -764,27 +835,27 @@ __device__ __forceinline__ void fluid_grad(const StageArgsT<T>& A, const GradArg
     using W = typename Wide<T>::type;
     const int q = c.q;
     const W* M0 = WideData<T>::cls(A.op) + __ldg(ci + CI_DOFF);
-    W qf[3];
+    double qf[3];
 #pragma unroll
     for (int fld = 0; fld < 3; ++fld) {
         T u[n], z[n];
         W y[n];
 #pragma unroll
         for (int i = 0; i < n; ++i) u[i] = U[fld * n + i];
+        const int eu = to_unit<n>(u);
         mass_apply<T, K>(M0, rect, u, y);
         load_state<n>(G.z, c.N, q, fld * n, z);
-        qf[fld] = coef_dot<T, K, W>(z, y);
+        const int ez = to_unit<n>(z);
+        qf[fld] = times_pow2(to_f64(coef_dot<T, K, W>(z, y)), eu + ez);
     }
     const double cm = G.mass_f[q], cp = G.mass_f[c.N + q];
-    G.grad_f[q] = fma(-G.w * cm, double(qf[0]) + double(qf[1]), G.grad_f[q]);
-    G.grad_f[c.N + q] = fma(G.w * cp, double(qf[2]), G.grad_f[c.N + q]);
+    G.grad_f[q] = fma(-G.w * cm, qf[0] + qf[1], G.grad_f[q]);
+    G.grad_f[c.N + q] = fma(G.w * cp, qf[2], G.grad_f[c.N + q]);
     if (G.wgrad)
         for (int s = 0; s < A.n_src; ++s)
-            if (A.src_dom[s] == 0 && A.src_q[s] == q) {
-                const W acc = wide_form<T, K>(A.op, ci, G.z + (size_t)2 * n * c.N + q, c.N,
-                                              A.src_g + (size_t)s * 2 * n, W(0));
-                G.wgrad[s] = G.w * cp * double(acc);
-            }
+            if (A.src_dom[s] == 0 && A.src_q[s] == q)
+                G.wgrad[s] = G.w * cp * wide_form<T, K, 1>(A.op, ci, G.z + (size_t)2 * n * c.N + q, c.N,
+                                                           A.src_g + (size_t)s * 2 * n);
 }
 
 // Gradients of one solid cell: U holds the raw rates [e_xx, e_yy, e_xy, div s (2)].
@@ -797,55 +868,56 @@ __device__ __forceinline__ void solid_grad(const StageArgsT<T>& A, const GradArg
     const size_t N = c.N;
     const W* M0 = WideData<T>::cls(A.op) + __ldg(ci + CI_DOFF);
     const T* zb = G.z + (size_t)3 * n * A.op.Nf;
-    W q00, q01, q10, q11, q22, qv;   // q_ab = z_a^T M0 raw_b
+    double q00, q01, q10, q11;   // q_ab = z_a^T M0 raw_b
     {
         T u[n], z[n];
         W y0[n], y1[n];
 #pragma unroll
         for (int i = 0; i < n; ++i) u[i] = U[i];
+        const int e0 = to_unit<n>(u);
         mass_apply<T, K>(M0, rect, u, y0);
 #pragma unroll
         for (int i = 0; i < n; ++i) u[i] = U[n + i];
+        const int e1 = to_unit<n>(u);
         mass_apply<T, K>(M0, rect, u, y1);
         load_state<n>(zb, c.N, q, 0, z);
-        q00 = coef_dot<T, K, W>(z, y0);
-        q01 = coef_dot<T, K, W>(z, y1);
+        int ez = to_unit<n>(z);
+        q00 = times_pow2(to_f64(coef_dot<T, K, W>(z, y0)), ez + e0);
+        q01 = times_pow2(to_f64(coef_dot<T, K, W>(z, y1)), ez + e1);
         load_state<n>(zb, c.N, q, n, z);
-        q10 = coef_dot<T, K, W>(z, y0);
-        q11 = coef_dot<T, K, W>(z, y1);
+        ez = to_unit<n>(z);
+        q10 = times_pow2(to_f64(coef_dot<T, K, W>(z, y0)), ez + e0);
+        q11 = times_pow2(to_f64(coef_dot<T, K, W>(z, y1)), ez + e1);
     }
-    W qs[3];
+    double qs[3];
 #pragma unroll
     for (int fld = 2; fld < 5; ++fld) {
         T u[n], z[n];
         W y[n];
 #pragma unroll
         for (int i = 0; i < n; ++i) u[i] = U[fld * n + i];
+        const int eu = to_unit<n>(u);
         mass_apply<T, K>(M0, rect, u, y);
         load_state<n>(zb, c.N, q, fld * n, z);
-        qs[fld - 2] = coef_dot<T, K, W>(z, y);
+        const int ez = to_unit<n>(z);
+        qs[fld - 2] = times_pow2(to_f64(coef_dot<T, K, W>(z, y)), eu + ez);
     }
-    q22 = qs[0];
-    qv = qs[1] + qs[2];
+    const double q22 = qs[0], qv = qs[1] + qs[2];
     const double d0 = G.mass_s[q], d1 = G.mass_s[N + q], d2 = G.mass_s[2 * N + q], rv = G.mass_s[3 * N + q];
     const double c1 = A.op.scal_s[SS_C1 * N + q], r = A.op.scal_s[SS_R * N + q];
     // mu_xx = -(d0 z_xx + d1 z_yy), mu_yy = -(d1 z_xx + d0 z_yy), mu_xy = -d2 z_xy (times M0 and w)
-    const double xx_xx = d0 * double(q00) + d1 * double(q10), xx_yy = d0 * double(q01) + d1 * double(q11);
-    const double yy_xx = d1 * double(q00) + d0 * double(q10), yy_yy = d1 * double(q01) + d0 * double(q11);
+    const double xx_xx = d0 * q00 + d1 * q10, xx_yy = d0 * q01 + d1 * q11;
+    const double yy_xx = d1 * q00 + d0 * q10, yy_yy = d1 * q01 + d0 * q11;
     const double w = G.w;
     G.grad_s[q] = fma(-w, xx_xx + r * xx_yy + yy_yy + r * yy_xx, G.grad_s[q]);          // d/dc1
     G.grad_s[N + q] = fma(-w * c1, xx_yy + yy_xx, G.grad_s[N + q]);                     // d/dr
-    G.grad_s[2 * N + q] = fma(-w * d2, double(q22), G.grad_s[2 * N + q]);               // d/dc3
-    G.grad_s[3 * N + q] = fma(w * rv, double(qv), G.grad_s[3 * N + q]);                 // d/d(1/(rho h))
+    G.grad_s[2 * N + q] = fma(-w * d2, q22, G.grad_s[2 * N + q]);               // d/dc3
+    G.grad_s[3 * N + q] = fma(w * rv, qv, G.grad_s[3 * N + q]);                 // d/d(1/(rho h))
     if (G.wgrad)
         for (int s = 0; s < A.n_src; ++s)
-            if (A.src_dom[s] == 1 && A.src_q[s] == q) {
-                W acc(0);
-                for (int e = 0; e < 2; ++e)
-                    acc = wide_form<T, K>(A.op, ci, zb + (size_t)(3 + e) * n * N + q, c.N,
-                                          A.src_g + ((size_t)s * 2 + e) * n, acc);
-                G.wgrad[s] = w * rv * double(acc);
-            }
+            if (A.src_dom[s] == 1 && A.src_q[s] == q)
+                G.wgrad[s] = w * rv * wide_form<T, K, 2>(A.op, ci, zb + (size_t)3 * n * N + q, c.N,
+                                                         A.src_g + (size_t)s * 2 * n);
 }
 
 // ---- fluid cells -------------------------------------------------------------------
