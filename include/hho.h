@@ -313,9 +313,9 @@ int hho_erk_step_record(hho_ops* ops, const hho_tableau* tab, double t0, double 
  * directly or, on large meshes (4096 warps of 32 cells and more), copied in
  * pieces that overlap the first and the last stage; other host memory is
  * staged through one device copy.  All give the same bits as
- * hho_state_pack, hho_erk_step and hho_state_unpack.  The device buffers,
- * the copy stream and the events it needs are made on the first call and
- * kept with ops. */
+ * hho_state_pack, hho_erk_step and hho_state_unpack.  The device buffers
+ * are made on the first call, which takes one piece, the copy stream and the
+ * events on the first call in pieces; all are kept with ops. */
 int hho_erk_run_host(hho_ops* ops, const hho_tableau* tab, double t0, double dt, int64_t nsteps,
                      double* h_canonical, void* stream);
 

@@ -807,11 +807,6 @@ void free_host_pipe(HostPipe* p) {
     delete p;
 }
 
-static int host_pieces(const hho_ops* ops, int64_t nsteps) {
-    if (nsteps < 1 || ops->prof_on || uses_graph(ops)) return 1;
-    return ops->host_pieces.n;
-}
-
 static HostPipe* host_pipe(hho_ops* ops) {
     if (ops->host_pipe) return ops->host_pipe;
     std::unique_ptr<HostPipe, void (*)(HostPipe*)> p(new HostPipe, free_host_pipe);
@@ -826,16 +821,17 @@ static HostPipe* host_pipe(hho_ops* ops) {
 // hho_erk_run_host on a pinned host buffer: the state is packed into the
 // arithmetic's device state (the double-float pair copy, or the FP64 state),
 // stepped and unpacked.  Small meshes: the pack kernels read and write the
-// mapped buffer themselves.  Large ones: in pieces (HostPieces) through the
-// device's canonical buffer by the copy engine, which moves the same bytes a
-// second (209 GB/s in, 191 out) without holding SM resources.
+// mapped buffer themselves.  Large ones, but for buffers made in the call: in
+// pieces (HostPieces) through the device's canonical buffer by the copy engine,
+// which moves the same bytes a second (209 GB/s in, 191 out) without holding SM
+// resources.
 template <class T>
 static int erk_run_pinned(hho_ops* ops, const hho_tableau* tab, double t0, double dt, int64_t nsteps,
-                          double* h_canonical, double* m_canonical, T* dst, cudaStream_t st) {
+                          double* h_canonical, double* m_canonical, T* dst, bool made, cudaStream_t st) {
     const char* who = "hho_erk_run_host";
     const int nc = (int)ops->nc;
     if (nc == 0) return HHO_OK;
-    const int blocks = (nc + STAGED_CELLS - 1) / STAGED_CELLS, np = host_pieces(ops, nsteps);
+    const int blocks = (nc + STAGED_CELLS - 1) / STAGED_CELLS, np = host_pieces(ops, nsteps, uses_graph(ops), made);
     if (np == 1) {
         int rc = launch_host_pack<T>(ops, m_canonical, dst, 0, blocks, st);
         if (!rc) rc = erk_run<T>(ops, tab, t0, dt, nsteps, 1, dst, (T*)ops->d_host_work, nullptr, st, who);
@@ -880,7 +876,7 @@ static int erk_run_pinned(hho_ops* ops, const hho_tableau* tab, double t0, doubl
 }
 
 static int erk_run_mapped(hho_ops* ops, const hho_tableau* tab, double t0, double dt, int64_t nsteps,
-                          double* h_canonical, double* m_canonical, cudaStream_t st) {
+                          double* h_canonical, double* m_canonical, bool made, cudaStream_t st) {
     std::vector<StagePlan> plan;
     int nb = 0;
     if (build_plan(tab, plan, &nb) != HHO_OK) {
@@ -889,8 +885,8 @@ static int erk_run_mapped(hho_ops* ops, const hho_tableau* tab, double t0, doubl
     }
     if (ops->arith == HHO_F32X2)
         return erk_run_pinned<f2x>(ops, tab, t0, dt, nsteps, h_canonical, m_canonical,
-                                   (f2x*)(ops->d_host_work + work_f64_part(ops, nb)), st);
-    return erk_run_pinned<double>(ops, tab, t0, dt, nsteps, h_canonical, m_canonical, ops->d_host_state, st);
+                                   (f2x*)(ops->d_host_work + work_f64_part(ops, nb)), made, st);
+    return erk_run_pinned<double>(ops, tab, t0, dt, nsteps, h_canonical, m_canonical, ops->d_host_state, made, st);
 }
 
 extern "C" int hho_set_launch_mode(hho_ops* ops, int32_t mode) {
@@ -1417,7 +1413,7 @@ extern "C" int hho_record(hho_ops* ops, const double* d_state, double* d_out, vo
 
 // The call on buffers that are ready; returns with work queued on st where it fails.
 static int erk_run_host(hho_ops* ops, const hho_tableau* tab, double t0, double dt, int64_t nsteps, double* h_canonical,
-                        void* stream) {
+                        bool made, void* stream) {
     cudaStream_t st = (cudaStream_t)stream;
     // A pinned host buffer mapped into the device's address space is read
     // and written by the pack kernels directly (over NVLink-C2C on GB300) or,
@@ -1426,7 +1422,7 @@ static int erk_run_host(hho_ops* ops, const hho_tableau* tab, double t0, double 
     cudaPointerAttributes pa;
     if (cudaPointerGetAttributes(&pa, h_canonical) == cudaSuccess && pa.type == cudaMemoryTypeHost &&
         pa.devicePointer) {
-        const int rc = erk_run_mapped(ops, tab, t0, dt, nsteps, h_canonical, (double*)pa.devicePointer, st);
+        const int rc = erk_run_mapped(ops, tab, t0, dt, nsteps, h_canonical, (double*)pa.devicePointer, made, st);
         if (rc) return rc;
         if (cudaStreamSynchronize(st) != cudaSuccess) {
             hho_set_error("hho_erk_run_host: %s", cudaGetErrorString(cudaGetLastError()));
@@ -1465,6 +1461,7 @@ extern "C" int hho_erk_run_host(hho_ops* ops, const hho_tableau* tab, double t0,
     int rc = hho_work_size(ops, tab, &wsz);
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
+    bool made = false;
     rc = grow_host_buffers(
         ops, wsz,
         [](size_t n) {
@@ -1474,11 +1471,11 @@ extern "C" int hho_erk_run_host(hho_ops* ops, const hho_tableau* tab, double t0,
             return (double*)nullptr;
         },
         [](double* p) { cudaFree(p); },
-        [&](double* p, size_t n) { return cudaMemsetAsync(p, 0, sizeof(double) * n, st) == cudaSuccess; });
+        [&](double* p, size_t n) { return cudaMemsetAsync(p, 0, sizeof(double) * n, st) == cudaSuccess; }, &made);
     if (rc == HHO_ENOMEM) hho_set_error("hho_erk_run_host: device allocation failed");
     if (rc == HHO_ECUDA) hho_set_error("hho_erk_run_host: device memset failed");
     if (rc) return rc;
-    rc = erk_run_host(ops, tab, t0, dt, nsteps, h_canonical, stream);
+    rc = erk_run_host(ops, tab, t0, dt, nsteps, h_canonical, made, stream);
     if (rc) cudaStreamSynchronize(st);   // the next call may come on another stream; the buffers are free for it
     return rc;
 }

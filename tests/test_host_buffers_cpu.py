@@ -18,6 +18,7 @@ PROGRAM = r"""
 static std::set<double*> live;
 static int countdown;   // the allocation that fails
 static bool memset_ok;
+static bool made;   // a buffer is new
 static int grow(hho_ops* o, int64_t size) {
     return grow_host_buffers(
         o, size,
@@ -31,7 +32,7 @@ static int grow(hho_ops* o, int64_t size) {
             if (!live.erase(p)) abort();   // freed twice, or never allocated
             free(p);
         },
-        [](double* p, size_t) { return live.count(p) && memset_ok; });
+        [](double* p, size_t) { return live.count(p) && memset_ok; }, &made);
 }
 static bool ready(const hho_ops& o, int64_t size) {
     return live.count(o.d_host_state) && live.count(o.d_host_canon) && live.count(o.d_host_work) &&
@@ -63,7 +64,13 @@ int main(int argc, char** argv) {
     if (grow(&o, 30) != HHO_OK || !ready(o, 30)) return 3;   // a smaller tableau afterwards
     if (grow(&o, 40) != HHO_OK || !ready(o, 40)) return 4;
     const double* w = o.d_host_work;
-    if (grow(&o, 20) != HHO_OK || o.d_host_work != w) return 5;
+    if (!made || grow(&o, 20) != HHO_OK || o.d_host_work != w || made) return 5;
+    // pieces: not on buffers just made, for no steps, step graphs or stage profiling
+    o.host_pieces.n = 4;
+    if (host_pieces(&o, 1, false, true) != 1 || host_pieces(&o, 1, false, false) != 4) return 6;
+    if (host_pieces(&o, 0, false, false) != 1 || host_pieces(&o, 1, true, false) != 1) return 7;
+    o.prof_on = true;
+    if (host_pieces(&o, 1, false, false) != 1) return 8;
     return 0;
 }
 """
