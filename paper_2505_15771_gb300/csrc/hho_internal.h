@@ -246,7 +246,7 @@ void launch_bj(const hho_ops* ops, const double* bj, const double* x, const doub
 constexpr int STAGED_CELLS = 64;   // cells of a block of the host pack kernels
 struct HostPieces {
     static constexpr int MAX = 8, WARPS = 2048;
-    int n = 1;
+    int n = 0;   // 0: not cut yet (cut_host_pieces, under the GPU's work of the first pinned call)
     int blocks[MAX + 1], warps[MAX + 1];   // host pieces in blocks of STAGED_CELLS cells, compute pieces in warps
     int64_t off[MAX + 1];                  // host pieces in values
     int own[MAX], need[MAX];               // the last host piece that compute piece d's traces / first stage wait for

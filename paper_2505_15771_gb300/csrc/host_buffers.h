@@ -26,13 +26,3 @@ int grow_host_buffers(hho_ops* ops, int64_t work_size, Alloc alloc, Release rele
     ops->host_work_size = work_size;
     return HHO_OK;
 }
-
-// The pieces (HostPieces) of a call that runs `graph` replays or not, on buffers
-// `made` in the same call or not.  New buffers: one piece.  A copy by the copy
-// engine into memory that was allocated just before waits 0.5 to 8 ms, while
-// kernels run at full speed on it; the first call of an operator, 1024 x 512, k =
-// 2, one FP64 step, took 2.2 to 10 ms in pieces and takes 2.5 to 3.7 in one (later
-// calls 1.75 and 2.04).
-inline int host_pieces(const hho_ops* ops, int64_t nsteps, bool graph, bool made) {
-    return nsteps < 1 || ops->prof_on || graph || made ? 1 : ops->host_pieces.n;
-}

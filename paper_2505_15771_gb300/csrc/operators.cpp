@@ -204,46 +204,6 @@ bool point_in_cell(const std::vector<double>& xy, const int64_t* vtx, int nv, do
     return true;
 }
 
-// The pieces of a host-buffer call (HostPieces): where the cells of each are and
-// which pieces their face neighbours lie in.
-void cut_host_pieces(hho_ops* ops) {
-    HostPieces& p = ops->host_pieces;
-    const int Nf = ops->dev.Nf, warps = (Nf + ops->dev.Ns) / 32;
-    const int64_t nc = ops->nc, blocks = (nc + STAGED_CELLS - 1) / STAGED_CELLS;
-    const int n = p.n = std::max(1, std::min<int>(HostPieces::MAX, warps / HostPieces::WARPS));
-    if (n == 1) return;
-    std::vector<uint8_t> warp_piece(warps), cell_piece(nc);
-    for (int c = 0; c <= n; ++c) {
-        p.blocks[c] = (int)(blocks * c / n);
-        p.off[c] = c == n ? ops->n_canonical : ops->canon_off[(int64_t)p.blocks[c] * STAGED_CELLS];
-        p.warps[c] = c == n ? warps : (int)((int64_t)warps * c / n) & ~3;   // whole thread blocks
-        if (c > 0) std::fill(warp_piece.begin() + p.warps[c - 1], warp_piece.begin() + p.warps[c], (uint8_t)(c - 1));
-    }
-    std::fill(p.own, p.own + n, 0);
-    for (int h = 0; h < n; ++h)
-        for (int64_t c = (int64_t)p.blocks[h] * STAGED_CELLS; c < std::min(nc, (int64_t)p.blocks[h + 1] * STAGED_CELLS); ++c) {
-            const int d = warp_piece[((ops->cell_dom[c] == 0 ? 0 : Nf) + ops->cell_pos[c]) / 32];
-            cell_piece[c] = (uint8_t)d;
-            p.own[d] = h;   // h grows
-        }
-    std::copy(p.own, p.own + n, p.need);
-    for (size_t F = 0; F + 1 < ops->face_cells.size(); F += 2) {
-        const int64_t a = ops->face_cells[F], b = ops->face_cells[F + 1];
-        if (a < 0 || b < 0) continue;
-        const int da = cell_piece[a], db = cell_piece[b];
-        p.need[da] = std::max(p.need[da], p.own[db]);
-        p.need[db] = std::max(p.need[db], p.own[da]);
-    }
-    int pos[HostPieces::MAX];
-    for (int d = 0; d < n; ++d) p.order[d] = d;
-    std::stable_sort(p.order, p.order + n, [&](int a, int b) { return p.need[a] < p.need[b]; });
-    for (int i = 0; i < n; ++i) pos[p.order[i]] = i;
-    std::fill(p.last, p.last + n, 0);
-    for (int h = 0; h < n; ++h)
-        for (int64_t c = (int64_t)p.blocks[h] * STAGED_CELLS; c < std::min(nc, (int64_t)p.blocks[h + 1] * STAGED_CELLS); ++c)
-            p.last[h] = std::max(p.last[h], pos[cell_piece[c]]);
-}
-
 // Bucket grid for locate(): about one bucket per cell over the mesh's
 // bounding box; each cell is listed in every bucket its bounding box
 // (enlarged by 1e-9 of its size, beyond point_in_cell's tolerance) meets.
@@ -982,7 +942,6 @@ extern "C" int hho_operators_build_tau(const hho_mesh* m, int32_t k, const doubl
     ops->h_cls_int = cls_int;
     ops->h_nb_f = nb_f;
     ops->h_nb_s = nb_s;
-    cut_host_pieces(ops);
     ops->h_if_nb = if_nb;
     ops->n_state = (int64_t)3 * n * Nf + (int64_t)5 * n * Ns;
     ops->trace_doubles = (int64_t)2 * f * SF + (int64_t)4 * f * SS;

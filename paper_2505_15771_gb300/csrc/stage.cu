@@ -17,6 +17,7 @@
 #include "f2x.cuh"
 #include "hho_internal.h"
 #include "host_buffers.h"
+#include "host_pieces.h"
 #include "stage_launch.h"
 
 namespace {
@@ -835,7 +836,9 @@ static int erk_run_pinned(hho_ops* ops, const hho_tableau* tab, double t0, doubl
     if (np == 1) {
         int rc = launch_host_pack<T>(ops, m_canonical, dst, 0, blocks, st);
         if (!rc) rc = erk_run<T>(ops, tab, t0, dt, nsteps, 1, dst, (T*)ops->d_host_work, nullptr, st, who);
-        return rc ? rc : launch_host_unpack<T>(ops, dst, m_canonical, 0, blocks, st);
+        if (!rc) rc = launch_host_unpack<T>(ops, dst, m_canonical, 0, blocks, st);
+        if (!rc && ops->host_pieces.n == 0) cut_host_pieces(ops);   // while the GPU works
+        return rc;
     }
     const HostPieces& cut = ops->host_pieces;
     HostPipe* p = host_pipe(ops);

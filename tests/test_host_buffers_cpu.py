@@ -65,12 +65,6 @@ int main(int argc, char** argv) {
     if (grow(&o, 40) != HHO_OK || !ready(o, 40)) return 4;
     const double* w = o.d_host_work;
     if (!made || grow(&o, 20) != HHO_OK || o.d_host_work != w || made) return 5;
-    // pieces: not on buffers just made, for no steps, step graphs or stage profiling
-    o.host_pieces.n = 4;
-    if (host_pieces(&o, 1, false, true) != 1 || host_pieces(&o, 1, false, false) != 4) return 6;
-    if (host_pieces(&o, 0, false, false) != 1 || host_pieces(&o, 1, true, false) != 1) return 7;
-    o.prof_on = true;
-    if (host_pieces(&o, 1, false, false) != 1) return 8;
     return 0;
 }
 """
