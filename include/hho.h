@@ -310,8 +310,8 @@ int hho_erk_step_record(hho_ops* ops, const hho_tableau* tab, double t0, double 
  * stepped, unpacked back into h_canonical, and the stream is synchronised.
  * Pinned host memory (cudaHostAlloc, or a pinned torch tensor) mapped into
  * the device's address space is read and written by the pack kernels
- * directly or, on large meshes (4096 warps of 32 cells and more), copied in
- * pieces that overlap the first and the last stage; other host memory is
+ * directly or, on large meshes (from 40 MB), copied in pieces that overlap
+ * the first and the last stage; other host memory is
  * staged through one device copy.  All give the same bits as
  * hho_state_pack, hho_erk_step and hho_state_unpack.  The device buffers
  * are made on the first call, which takes one piece, the copy stream and the

@@ -238,14 +238,30 @@ void launch_bj(const hho_ops* ops, const double* bj, const double* x, const doub
 // the traces of its face neighbours too.  The order only decides what overlaps:
 // a mesh whose device order is unrelated to its cell order runs one after the other.
 //
-// From 4096 warps of cells (131 K cells, 15 to 25 MB each way at k = 2), a piece
-// for every 2048 of them: smaller pieces leave the SMs idle between them for
-// longer than the copies they hide.  One FP64 step of the k = 2 bilayer, us, by
-// pieces 1 | 2 | 4 | 8 | 16: 1024 x 512 2038 | 1889 | 1823 | 1719 | 1815; 724 x 362
-// 1083 | 1035 | 999 | 1023 | 1312; 512 x 272 590 | 575 | 591 | 690 | 946.
+// Two, four or eight pieces of 2000 warps of cells and more (smaller ones leave the
+// SMs idle between them for longer than the copies they hide; three cut a piece at
+// the domains' border), from BYTES on each way, and one where not even the traces
+// of a piece can start before the last one has arrived: the second pass over memory
+// and the smaller grids then cost more than overlaps.  One step of ERK4, us, by
+// pieces 1 | 2 | 4 | 8, FP64 and double-float:
+//   1024 x 512, k = 2, 100 MB         2032 | 1916 | 1847 | 1745    1829 | 1745 | 1711 | 1661
+//   1024 x 512, k = 1, 50 MB          1066 | 1014 | 1006 |  981     972 |  933 |  922 |  954
+//   724 x 362, k = 2, 50 MB           1106 | 1057 | 1032 | 1050    1049 |  996 | 1023 |  969
+//   512 x 272, k = 3, 45 MB            991 |  942 |  962 | 1075     924 |  883 |  901 |  992
+//   512 x 272, k = 2, 27 MB            610 |  599 |  610 |  717     551 |  576 |  569 |  635
+//   724 x 362, k = 1, 25 MB            602 |  588 |  600 |  658     520 |  503 |  556 |  574
+//   512 x 512 triangles, k = 2, 100 MB 2796 | 2598 | 2663 | 2597   1940 | 1843 | 1845 | 1804
+// and where two pieces both wait for the last arrival, and with four every stage does:
+//   400 x 400 hybrid, k = 3, 63 MB    1556 | 1654 | 1590 | 1630    1291 | 1380 | 1258 | 1281
+//   300 x 300 triangles, k = 3, 58 MB 1782 | 1923 | 1935 | 1895    1239 | 1324 | 1281 | 1291
+//   400 x 400 hanging, k = 3, 52 MB   1201 | 1326 | 1342 | 1320    1112 | 1183 | 1093 | 1123
+//   680 x 340 hybrid, k = 3, 91 MB    2173 | 2262 | 2190 | 2193    1773 | 1901 | 1734 | 1692
+//   800 x 600 hanging, k = 2, 91 MB   2066 | 2173 | 2078 | 1974    1759 | 1856 | 1862 | 1718
+//   1000 x 700 hybrid, k = 2, 175 MB  3835 | 3959 | 3596 | 3404    3046 | 3173 | 2931 | 2776
 constexpr int STAGED_CELLS = 64;   // cells of a block of the host pack kernels
 struct HostPieces {
-    static constexpr int MAX = 8, WARPS = 2048;
+    static constexpr int MAX = 8, WARPS = 2000;
+    static constexpr int64_t BYTES = 40000000;
     int n = 0;   // 0: not cut yet (cut_host_pieces, under the GPU's work of the first pinned call)
     int blocks[MAX + 1], warps[MAX + 1];   // host pieces in blocks of STAGED_CELLS cells, compute pieces in warps
     int64_t off[MAX + 1];                  // host pieces in values

@@ -19,8 +19,9 @@ inline void cut_host_pieces(hho_ops* ops) {
     const int Nf = ops->dev.Nf, warps = (Nf + ops->dev.Ns) / 32;
     const int64_t nc = ops->nc, blocks = (nc + STAGED_CELLS - 1) / STAGED_CELLS;
     p.n = 1;
-    const int n = std::min<int>(HostPieces::MAX, warps / HostPieces::WARPS);
-    if (n <= 1) return;
+    int n = 1;
+    while (n < HostPieces::MAX && warps / HostPieces::WARPS >= 2 * n) n *= 2;
+    if (n == 1 || (int64_t)sizeof(double) * ops->n_canonical < HostPieces::BYTES) return;
     std::unique_ptr<uint8_t[]> warp_piece(new (std::nothrow) uint8_t[warps]), cell_piece(new (std::nothrow) uint8_t[nc]);
     if (!warp_piece || !cell_piece) return;   // one piece
     for (int c = 0; c <= n; ++c) {
@@ -62,6 +63,7 @@ inline void cut_host_pieces(hho_ops* ops) {
             if ((meets[d] >> e) & 1) p.need[d] = std::max(p.need[d], p.own[e]);
     }
     std::stable_sort(p.order, p.order + n, [&](int a, int b) { return p.need[a] < p.need[b]; });
+    if (*std::min_element(p.own, p.own + n) == n - 1) return;   // nothing starts before the last arrival
     for (int h = 0; h < n; ++h) {
         p.last[h] = 0;
         for (int i = 0; i < n; ++i)

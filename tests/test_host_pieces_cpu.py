@@ -18,7 +18,7 @@ PROGRAM = r"""
 
 int main(int argc, char** argv) {
     const int nx = atoi(argv[1]), ny = atoi(argv[2]), k = atoi(argv[3]);
-    const char order = argv[4][0];   // o: as the cells; i: two classes interleaved; r: random
+    const char order = argv[4][0];   // o: as the cells; i: two classes interleaved; r: random; x: domains too
     const int n = (k + 1) * (k + 2) / 2;
     hho_ops o;
     o.nc = (int64_t)nx * ny;
@@ -27,7 +27,7 @@ int main(int argc, char** argv) {
     o.cell_dom.resize(o.nc), o.cell_pos.resize(o.nc);
     int64_t count[2] = {};
     for (int64_t c = 0; c < o.nc; ++c) {   // upper half fluid
-        o.cell_dom[c] = c < o.nc / 2;
+        o.cell_dom[c] = order == 'x' ? c & 1 : c < o.nc / 2;
         o.canon_off.push_back(o.n_canonical);
         o.n_canonical += (o.cell_dom[c] ? 5 : 3) * n;
         count[o.cell_dom[c]]++;
@@ -37,7 +37,7 @@ int main(int argc, char** argv) {
         for (int64_t c = 0; c < o.nc; ++c)
             if (o.cell_dom[c] == d) cells.push_back(c);
         if (order == 'i') std::stable_partition(cells.begin(), cells.end(), [](int64_t c) { return c & 1; });
-        if (order == 'r') std::shuffle(cells.begin(), cells.end(), rng);
+        if (order == 'r' || order == 'x') std::shuffle(cells.begin(), cells.end(), rng);
         for (size_t i = 0; i < cells.size(); ++i) o.cell_pos[cells[i]] = (int32_t)i;
     }
     o.dev.Nf = (int)((count[0] + 31) / 32 * 32);
@@ -104,9 +104,11 @@ def program(tmp_path_factory):
     return exe
 
 
+# the last ones: cells of both domains all over the canonical order, where nothing can start early
 @pytest.mark.parametrize("nx,ny,k,order,pieces", [
     (1024, 512, 2, "o", 8), (1024, 512, 1, "o", 8), (723, 363, 2, "o", 4), (512, 272, 3, "o", 2),
-    (64, 64, 2, "o", 1), (1000, 700, 2, "i", 8), (1023, 513, 3, "r", 8)])
+    (512, 272, 2, "o", 1), (64, 64, 2, "o", 1), (1000, 700, 2, "i", 8), (1023, 513, 3, "r", 8), (723, 363, 3, "r", 4),
+    (1023, 513, 2, "x", 1), (723, 363, 3, "x", 1)])
 def test_pieces_follow_their_definition(program, nx, ny, k, order, pieces):
     r = subprocess.run([program, str(nx), str(ny), str(k), order], capture_output=True, text=True)
     assert r.returncode == 0 and int(r.stdout) == pieces
