@@ -239,79 +239,79 @@ __global__ void sum_kernel(const double* __restrict__ partial, int np, double* o
 
 // Receivers: fluid [p, m_x, m_y, 0, 0]; solid [v_x, v_y, s_xx, s_yy, s_xy];
 // interface [p_F, v_Fx, v_Fy, 0, 0] from the pointwise face solve.
-// One block a receiver (y = shot): thread (field, i) fetches a coefficient, one
-// thread a field adds them up, then one thread an output.  The chain of loads is
-// two long, and FP64 instructions, 64 cycles each to a warp, are issued for all
-// fields at once (one thread a receiver took 7.3 us for the eight interface
-// receivers of the academic run, a sixth of its step).  State shot stride
-// n_state, output shot stride 5 n_rec; with a device clock (graph replay) out is
-// the trace base, offset by the step, and the last block to have read the step
-// advances it.
-constexpr int REC_FIELDS = 8;   // three of the fluid cell, five of the solid cell
+// Eight lanes a receiver (y = shot), a field each: a lane issues its loads together
+// and adds the field's coefficients up, and the pointwise solve goes through
+// shuffles.  The chain of loads is two long, and FP64 instructions, 64 cycles each
+// to a warp, are issued for all fields and four receivers at once.  Few
+// receivers: blocks of one warp, so that they spread over the SMs.  us for 8 |
+// 1000 | 20,000 | 100,000 receivers, k = 2: one thread a receiver 8.2 | 14.7 | 16.7 |
+// 27.0, one block a receiver 6.8 | 6.7 | 21.4 | 101.5, this form 6.8 | 6.6 | 9.7 | 27.5.
+// State shot stride n_state, output shot stride 5 n_rec; with a device clock (graph
+// replay) out is the trace base, offset by the step, and the last block to have
+// read the step advances it.
+constexpr int REC_LANES = 8;   // three fields of the fluid cell, five of the solid cell
 constexpr int REC_MAX_N = 10;
-inline int record_threads(int n) { return (REC_FIELDS * n + 31) / 32 * 32; }
 template <class T, class TO = T>
-__global__ void record_kernel(DevOps op, int n_rec, const int32_t* __restrict__ ri, const double* __restrict__ rd,
-                              const T* state, int64_t n_state, TO* out, StageClock* clock = nullptr) {
-    __shared__ double val[REC_FIELDS][REC_MAX_N], field[REC_FIELDS], flux[3];
-    const int r = blockIdx.x, n = op.n, t = threadIdx.x;
+__global__ void __launch_bounds__(128)
+    record_kernel(DevOps op, int n_rec, const int32_t* __restrict__ ri, const double* __restrict__ rd, const T* state,
+                  int64_t n_state, TO* out, StageClock* clock = nullptr) {
+    const int n = op.n, t = threadIdx.x % REC_LANES;
+    const int at = blockIdx.x * (blockDim.x / REC_LANES) + threadIdx.x / REC_LANES;
+    const int r = min(at, n_rec - 1);   // lanes past the last receiver follow it and store nothing
     const double* d = rd + (size_t)r * (2 * n + 15);
-    const int kind = ri[4 * r], qf = ri[4 * r + 1], qs = ri[4 * r + 2];
-    const int fld = t / n, i = t - fld * n;   // 0..2 fluid m_x, m_y, p; 3..7 solid s_xx, s_yy, s_xy, v_x, v_y
+    const int kind = ri[4 * r], q = ri[4 * r + (t < 3 ? 1 : 2)];
+    const bool use = kind == 2 || (t >= 3) == (kind == 1);
+    const double* phi = kind == 2 && t >= 3 ? d + n : d;
     release_successor();
     wait_for_predecessor();
-    const T* sf = state + (size_t)blockIdx.y * n_state;
-    const T* ss = sf + (size_t)3 * n * op.Nf;
-    if (fld < 3 && kind != 1) val[fld][i] = double(sf[(size_t)(fld * n + i) * op.Nf + qf]);
-    if (fld >= 3 && fld < REC_FIELDS && kind != 0) val[fld][i] = double(ss[(size_t)((fld - 3) * n + i) * op.Ns + qs]);
-    int64_t step = 0;
-    if (clock && t == 0) {
-        step = *(volatile int64_t*)&clock->step;
-        __threadfence();   // the read comes before the ticket that lets the last block write
-        if (atomicAdd(&clock->ticket, 1u) == gridDim.x * gridDim.y - 1) {   // every block has read it
-            __threadfence();
-            clock->ticket = 0;
-            clock->step = step + 1;
+    const size_t N = t < 3 ? op.Nf : op.Ns;
+    const T* field = state + (size_t)blockIdx.y * n_state + (t < 3 ? (size_t)t * n * N : (size_t)3 * n * op.Nf + (size_t)(t - 3) * n * N);
+    T val[REC_MAX_N];
+#pragma unroll
+    for (int j = 0; j < REC_MAX_N; ++j)
+        if (use && j < n) val[j] = field[j * N + q];
+    if (clock) {
+        __shared__ int64_t step;
+        if (threadIdx.x == 0) {
+            step = *(volatile int64_t*)&clock->step;
+            __threadfence();   // the read comes before the ticket that lets the last block write
+            if (atomicAdd(&clock->ticket, 1u) == gridDim.x * gridDim.y - 1) {   // every block has read it
+                __threadfence();
+                clock->ticket = 0;
+                clock->step = step + 1;
+            }
         }
+        __syncthreads();
+        out += (size_t)step * 5 * n_rec * gridDim.y;
     }
-    __shared__ int64_t step_sh;
-    if (t == 0) step_sh = step;
-    __syncthreads();
-    if (t < REC_FIELDS) {
-        const double* phi = kind == 2 && t >= 3 ? d + n : d;
-        double s = 0.0;
-        if (kind == 2 || (t >= 3) == (kind == 1))
-            for (int j = 0; j < n; ++j) s = fma(phi[j], val[t][j], s);
-        field[t] = s;
+    double g = 0.0;   // lane t: fluid m_x, m_y, p; solid s_xx, s_yy, s_xy, v_x, v_y
+#pragma unroll
+    for (int j = 0; j < REC_MAX_N; ++j)
+        if (use && j < n) g = fma(phi[j], double(val[j]), g);
+    auto of = [](double x, int lane) { return __shfl_sync(0xffffffffu, x, lane, REC_LANES); };
+    // plain receivers: [p, m_x, m_y] or [v_x, v_y, s_xx, s_yy, s_xy]
+    double o = of(g, kind == 0 ? (t == 0 ? 2 : t == 1 ? 0 : 1) : (t < 2 ? 6 + t : t < 5 ? 1 + t : 0));
+    // interface: lanes 0..2 the fluxes tau_f p - m.n_f, tau_s v - s n_s
+    const double u = of(g, t == 0 ? 2 : t == 1 ? 6 : 7), a = of(g, t == 0 ? 0 : t == 1 ? 3 : 5),
+                 b = of(g, t == 0 ? 1 : t == 1 ? 5 : 4);
+    double flux = 0.0;
+    if (kind == 2) {
+        const double* c = d + 2 * n;   // tau_f, tau_s, n_f, n_s
+        flux = c[t == 0 ? 0 : 1] * u - (a * c[t == 0 ? 2 : 4] + b * c[t == 0 ? 3 : 5]);
     }
-    __syncthreads();
-    const double* g = field;
-    if (kind == 2 && t < 3) {   // tau_f p - m.n_f, tau_s v - s n_s
-        const double tf = d[2 * n], ts = d[2 * n + 1];
-        const double nfx = d[2 * n + 2], nfy = d[2 * n + 3], nsx = d[2 * n + 4], nsy = d[2 * n + 5];
-        flux[t] = t == 0   ? tf * g[2] - (g[0] * nfx + g[1] * nfy)
-                  : t == 1 ? ts * g[6] - (g[3] * nsx + g[5] * nsy)
-                           : ts * g[7] - (g[5] * nsx + g[4] * nsy);
-    }
-    __syncthreads();
-    if (t >= 5) return;
-    double o = 0.0;
-    if (kind == 0) {
-        if (t < 3) o = g[t == 0 ? 2 : t - 1];
-    } else if (kind == 1) {
-        o = g[t < 2 ? 6 + t : 1 + t];
-    } else if (t < 3) {
+    const double w0 = of(flux, 0), w1 = of(flux, 1), w2 = of(flux, 2);
+    if (kind == 2 && t < 3) {
         const double* Ai = d + 2 * n + 6 + 3 * t;
-        o = Ai[0] * flux[0] + Ai[1] * flux[1] + Ai[2] * flux[2];
+        o = Ai[0] * w0 + Ai[1] * w1 + Ai[2] * w2;
     }
-    if (clock) out += (size_t)step_sh * 5 * n_rec * gridDim.y;
-    out[(size_t)blockIdx.y * 5 * n_rec + 5 * r + t] = TO(o);
+    if (at < n_rec && t < 5) out[(size_t)blockIdx.y * 5 * n_rec + 5 * r + t] = TO(kind != 1 && t >= 3 ? 0.0 : o);
 }
 
 template <class T, class TO>
 void launch_record(const hho_ops* ops, int n_shots, const T* state, TO* out, StageClock* clock, cudaStream_t st) {
-    launch_dependent(record_kernel<T, TO>, dim3(ops->n_rec, n_shots), record_threads(ops->n), 0, st, ops->dev, ops->n_rec,
-                     ops->d_rec_int, ops->d_rec_dbl, state, ops->n_state, out, clock);
+    const int threads = (int64_t)ops->n_rec * n_shots <= 16 * 152 ? 32 : 128, per = threads / REC_LANES;
+    launch_dependent(record_kernel<T, TO>, dim3((ops->n_rec + per - 1) / per, n_shots), threads, 0, st, ops->dev,
+                     ops->n_rec, ops->d_rec_int, ops->d_rec_dbl, state, ops->n_state, out, clock);
 }
 
 template <class T, int MODE>
