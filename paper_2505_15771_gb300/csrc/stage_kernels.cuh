@@ -1758,37 +1758,54 @@ struct TeamTag {};
 
 // Where the team form (stage_team.cuh) is the faster one: up to so many groups
 // of 32 cells (times shots), by arithmetic, degree, mode (stage, application,
-// traces alone) and mesh (at least a quarter of the groups not rectangles: gen).
-// Small grids take W warps a block, larger ones four (fewer idle warps, more
+// traces alone) and mesh (rectangles, or at least a quarter of the groups others:
+// gen).  Up to 600 groups take W warps a block, more four (fewer idle warps, more
 // blocks an SM) but for the 8-byte types at k = 3, whose ten rows fit ten warps.
-// Both forms give the same bits, so the choice is free.  Measured on GB300, us
-// a stage, thread form / team form:
-//                               512 groups    1024          2048          4096
-//   FP64 k = 2 squares          18.9 / 17.1   21.4 / 26.7   31.7 / 44.3   68.7 / 87.8
-//   FP64 k = 3 hanging          68.2 / 28.2   74.6 / 46.0   107 / 91.2    165 / 174
-//   double-float k = 2 squares  19.5 / 8.3    20.6 / 12.6   22.5 / 23.0   52.3 / 54.9
-//   double-float k = 3 squares  31.2 / 12.9   36.5 / 20.4   68.3 / 46.7   113 / 88.3
-//   FP32 k = 2 squares          8.9 / 5.5     9.7 / 7.7     10.5 / 13.8   14.8 / 25.2
-// Large FP64 grids are bound by the FP64 pipe, and the thread form issues the
-// fewer FP64 instructions; large FP32 ones by memory, where its coalesced rows
-// of one warp do as well with less code.
+// Both forms give the same bits, so the choice is free.  The lines lie where both
+// forms, timed at 128 to 8192 groups of squares and of triangles, cross (us a
+// launch on GB300, thread form / team form):
+//                                 512 groups    1048          2048          4200
+//   stage, squares    FP64 k = 1  11.3 / 9.7    13.4 / 14.6   18.2 / 23.0   36.9 / 46.8
+//                     FP64 k = 2  18.6 / 17.3   21.9 / 27.2   32.5 / 44.9   72.9 / 92.2
+//                     FP64 k = 3  29.7 / 21.6   37.0 / 37.0   58.0 / 74.2   118 / 147
+//                     pairs k = 1 9.6 / 6.5     10.2 / 7.9    11.5 / 13.2   20.4 / 31.0
+//                     pairs k = 2 19.6 / 8.3    20.1 / 12.6   22.9 / 23.5   53.9 / 57.6
+//                     pairs k = 3 31.7 / 12.7   33.2 / 19.9   69.7 / 46.7   120 / 94.2
+//                     FP32 k = 1  5.7 / 4.3     6.7 / 5.5     6.9 / 9.1     8.9 / 16.2
+//                     FP32 k = 2  8.7 / 5.3     9.7 / 7.6     10.0 / 13.6   15.4 / 25.5
+//                     FP32 k = 3  11.0 / 8.4    11.9 / 10.5   12.7 / 18.8   31.3 / 45.9
+//   stage, triangles  FP64 k = 2  31.1 / 22.3   33.9 / 35.0   56.2 / 57.9   113 / 118
+//                     FP64 k = 3  51.0 / 33.5   60.7 / 57.1   103 / 106     202 / 211
+//                     pairs k = 3 49.9 / 15.0   52.0 / 24.9   92.4 / 48.0   134 / 97.5
+//                     FP32 k = 3  13.1 / 8.8    12.6 / 11.0   15.0 / 19.9   33.7 / 43.5
+//   traces, triangles FP64 k = 2  13.3 / 11.7   15.0 / 17.0   26.1 / 28.7   52.1 / 58.5
+//                     pairs k = 3 21.8 / 9.8    30.8 / 15.6   39.5 / 32.3   56.4 / 61.5
+//                     FP32 k = 3  4.8 / 6.6     5.0 / 7.6     6.1 / 11.9    11.3 / 24.5
+//   application, tri. pairs k = 3 22.7 / 9.3    38.7 / 15.0   43.8 / 26.2   70.7 / 55.6
+// and pairs at 16,384 | 33,000 groups: squares k = 2 179 / 194 | 332 / 376, k = 3 368 /
+// 341 | 660 / 676; triangles k = 2 196 / 201 | 383 / 399, k = 3 456 / 357 | 894 / 715.
+// (1216 groups are one wave of the four-warp team, eight blocks an SM.)  Large
+// FP64 grids are bound by the FP64 pipe, and the thread form issues the fewer FP64
+// instructions; large FP32 ones by memory, where its coalesced rows of one warp do
+// as well with less code.
 template <class T, int K>
 struct TeamRule;
 constexpr int TEAM_ALL = 1 << 30;
-#define HHO_TEAM_RULE(T_, K_, W_, rect_, gen_, app_, tr_rect_, tr_gen_)                                        \
-    template <>                                                                                               \
-    struct TeamRule<T_, K_> {                                                                                 \
-        static constexpr int W = W_, rect = rect_, gen = gen_, app = app_, tr_rect = tr_rect_, tr_gen = tr_gen_; \
+#define HHO_TEAM_RULE(T_, K_, W_, rect_, gen_, app_rect_, app_gen_, tr_rect_, tr_gen_)                      \
+    template <>                                                                                             \
+    struct TeamRule<T_, K_> {                                                                               \
+        static constexpr int W = W_, rect = rect_, gen = gen_, app_rect = app_rect_, app_gen = app_gen_,     \
+                             tr_rect = tr_rect_, tr_gen = tr_gen_;                                          \
     }
-HHO_TEAM_RULE(double, 1, 8, 800, 2500, 1300, 128, 900);
-HHO_TEAM_RULE(double, 2, 8, 650, 2100, 1100, 200, 900);
-HHO_TEAM_RULE(double, 3, 10, 1050, 3200, 1500, 300, 1500);
-HHO_TEAM_RULE(f2x, 1, 8, 1800, 3200, 2500, 1300, 3000);
-HHO_TEAM_RULE(f2x, 2, 8, 2000, TEAM_ALL, 4000, 700, 4000);
-HHO_TEAM_RULE(f2x, 3, 10, TEAM_ALL, TEAM_ALL, 3000, 1500, 5500);
-HHO_TEAM_RULE(float, 1, 8, 1300, 1900, 0, 200, 900);
-HHO_TEAM_RULE(float, 2, 8, 1400, 1900, 0, 200, 850);
-HHO_TEAM_RULE(float, 3, 10, 1250, 1700, 0, 200, 1200);
+HHO_TEAM_RULE(double, 1, 8, 720, 1500, 1216, 1300, 400, 700);
+HHO_TEAM_RULE(double, 2, 8, 650, 1000, 1100, 1216, 350, 680);
+HHO_TEAM_RULE(double, 3, 10, 1050, 2000, 1216, 3500, 480, 850);
+HHO_TEAM_RULE(f2x, 1, 8, 1300, 1900, 3700, 1500, 1216, 1216);
+HHO_TEAM_RULE(f2x, 2, 8, 2000, 12000, 4000, 5500, 700, 1700);
+HHO_TEAM_RULE(f2x, 3, 10, 24000, TEAM_ALL, 2900, 24000, 1300, 3500);
+HHO_TEAM_RULE(float, 1, 8, 1216, 1216, 0, 0, 640, 600);
+HHO_TEAM_RULE(float, 2, 8, 1216, 1216, 0, 0, 500, 300);
+HHO_TEAM_RULE(float, 3, 10, 1216, 1216, 0, 0, 300, 250);
 #undef HHO_TEAM_RULE
 
 // Warps of a team block for this launch, 0 for the thread form.
@@ -1797,7 +1814,9 @@ int team_warps(const DevOps& op, int warps, int n_shots) {
     using R = TeamRule<T, K>;
     const int64_t cells = op.n_warps_f + op.n_warps_s, groups = (int64_t)warps * n_shots;
     const bool gen = 4 * (cells - op.n_warps_rect) >= cells;
-    const int limit = MODE == MODE_TRACES ? (gen ? R::tr_gen : R::tr_rect) : MODE == MODE_APPLY ? R::app : gen ? R::gen : R::rect;
+    const int limit = MODE == MODE_TRACES  ? (gen ? R::tr_gen : R::tr_rect)
+                      : MODE == MODE_APPLY ? (gen ? R::app_gen : R::app_rect)
+                                           : (gen ? R::gen : R::rect);
     if (groups > limit || op.max_nf > 32 || sizeof(T) * team_smem_elems<T, K>(op.max_nf) > 200 * 1024) return 0;
     return groups <= 600 || (K == 3 && sizeof(T) == 8) ? R::W : 4;
 }
