@@ -167,11 +167,8 @@ __device__ __forceinline__ double to_f64(double v) { return v; }
 __device__ __forceinline__ double to_f64(float v) { return f32_to_f64(v); }
 __device__ __forceinline__ double to_f64(f2x v) { return pair_to_f64(v); }
 
-// Comparisons of class-matrix entries (FP64 ones on the bits: a DSETP would
-// take an FP64 slot).
-__device__ __forceinline__ bool is_zero(double x) { return (__double_as_longlong(x) << 1) == 0; }
-__device__ __forceinline__ bool is_zero(float x) { return x == 0.0f; }
-__device__ __forceinline__ bool is_zero(f2x x) { return x.hi == 0.0f; }
+// Signs of class-matrix entries (FP64 ones on the bits: a DSETP would take an FP64
+// slot).
 __device__ __forceinline__ bool is_negative(double x) { return __double2hiint(x) < 0; }
 __device__ __forceinline__ bool is_negative(float x) { return x < 0.0f; }
 __device__ __forceinline__ bool is_negative(f2x x) { return x.hi < 0.0f; }

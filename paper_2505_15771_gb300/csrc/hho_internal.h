@@ -55,8 +55,8 @@ struct hho_mesh {
 };
 
 // Per-class integer record on the device (stride CI_STRIDE ints).
-// CI_HOR, CI_VER: bit j set where local face j < 32 is horizontal (n_x = 0) or
-// vertical (n_y = 0).
+// CI_HOR, CI_VER: bit j set where local face j (a cell has at most 32,
+// hho_mesh_create) is horizontal (n_x = 0) or vertical (n_y = 0).
 enum { CI_DOMAIN = 0, CI_NF, CI_START, CI_COUNT, CI_NPAD, CI_SLOT, CI_DOFF, CI_KIND, CI_HOR, CI_VER, CI_STRIDE };
 
 // Class kinds: generic polygon (dense class matrices) or axis-aligned
@@ -225,8 +225,7 @@ int erk_steps_f32(hho_ops* ops, const hho_tableau* tab, double t0, double dt, in
 int check_cuda(const char* what);
 // y = *scale P^-1 x (scale null: 1; bj null: P = I; accumulate: y += ..., not with
 // traces), P^-1 the inverse cell blocks of hho_ops::d_bj; with tr, the FP64
-// face traces of y too, where bj_traces_fit (sdirk_bj.cu).
-bool bj_traces_fit(const hho_ops* ops);
+// face traces of y too.
 void launch_bj(const hho_ops* ops, const double* bj, const double* x, const double* scale, double* y, bool accumulate,
                double* tr, void* stream);
 

@@ -631,11 +631,10 @@ int gmres(hho_ops* ops, const SdirkWork& W, const double* b, double* x, double a
     double* S1 = W.sums;
     double* S2 = W.sums + (m + 1);
     double* S3 = W.sums + 2 * (m + 1);
-    const bool fused = bj_traces_fit(ops);
     // V_{l + 1} = A P^-1 V_l / ||V_l||
     auto apply_vector = [&](int l) {
-        launch_bj(ops, bj, W.V + (size_t)l * W.n, W.inv + l, W.PZ, false, fused ? W.tr : nullptr, (void*)st);
-        apply_op(ops, W.PZ, W.V + (size_t)(l + 1) * W.n, W.tr, a_dt, false, 0.0, st, fused);
+        launch_bj(ops, bj, W.V + (size_t)l * W.n, W.inv + l, W.PZ, false, W.tr, (void*)st);
+        apply_op(ops, W.PZ, W.V + (size_t)(l + 1) * W.n, W.tr, a_dt, false, 0.0, st, true);
     };
     KrylovArgs N;
     N.V = W.W;

@@ -104,8 +104,6 @@ void launch(const DevOps& op, const double* bj, const double* x, const double* s
 
 }  // namespace
 
-bool bj_traces_fit(const hho_ops* ops) { return ops->dev.max_nf <= 32; }
-
 void launch_bj(const hho_ops* ops, const double* bj, const double* x, const double* scale, double* y, bool accumulate,
                double* tr, void* stream) {
     if (ops->dev.n_warps_f + ops->dev.n_warps_s == 0) return;

@@ -488,7 +488,7 @@ __device__ __forceinline__ void for_faces(const CellCtx<T>& c, H hor, V ver, O o
         const uint32_t done = c.hor | c.ver;
 #pragma unroll 1
         for (int j = 0; j < c.nF; ++j)
-            if (j >= 32 || !((done >> j) & 1)) other(j);
+            if (!((done >> j) & 1)) other(j);
     } else {
 #pragma unroll 1
         for (int j = 0; j < c.nF; ++j) other(j);
@@ -1817,7 +1817,7 @@ int team_warps(const DevOps& op, int warps, int n_shots) {
     const int limit = MODE == MODE_TRACES  ? (gen ? R::tr_gen : R::tr_rect)
                       : MODE == MODE_APPLY ? (gen ? R::app_gen : R::app_rect)
                                            : (gen ? R::gen : R::rect);
-    if (groups > limit || op.max_nf > 32 || sizeof(T) * team_smem_elems<T, K>(op.max_nf) > 200 * 1024) return 0;
+    if (groups > limit || sizeof(T) * team_smem_elems<T, K>(op.max_nf) > 200 * 1024) return 0;
     return groups <= 600 || (K == 3 && sizeof(T) == 8) ? R::W : 4;
 }
 

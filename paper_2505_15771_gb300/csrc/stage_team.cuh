@@ -247,7 +247,7 @@ __device__ __forceinline__ void team_cells(const StageArgsT<T>& A, int gw, int s
         float4* dst = reinterpret_cast<float4*>(cd);
         for (int e = threadIdx.x; e < nF * FS * (int)sizeof(T) / 16; e += 32 * W) dst[e] = __ldg(src + e);
     }
-    // faces by orientation: horizontal, vertical, other (at most 32 faces, see team_warps)
+    // faces by orientation: horizontal, vertical, other (a cell has at most 32)
     const uint32_t faces_h = (uint32_t)__ldg(ci + CI_HOR), faces_v = (uint32_t)__ldg(ci + CI_VER);
     const uint32_t faces_g = (nF >= 32 ? 0xffffffffu : (1u << nF) - 1u) & ~(faces_h | faces_v);
     const T* inp = A.inp + soff + q;
