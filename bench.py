@@ -191,14 +191,48 @@ def replica_reduce(ms_local, units_local, world, dist=None, device=None):
     return float(t.item()), float(u.item())
 
 
+def stage_sources():
+    """The stage kernels' source files: what their translation units include of
+    csrc, directly or not."""
+    import re
+    csrc = os.path.join(ROOT, "paper_2505_15771_gb300", "csrc")
+    todo, seen = ["stage_f64.cu", "stage_f32.cu", "stage_f2x.cu"], set()
+    while todo:
+        f = todo.pop()
+        if f in seen or not os.path.exists(os.path.join(csrc, f)):
+            continue
+        seen.add(f)
+        todo += re.findall(r'#include "([^"]+)"', open(os.path.join(csrc, f)).read())
+    return [os.path.join(csrc, f) for f in sorted(seen)]
+
+
 def stage_source_sha():
-    """sha256 of the stage kernel sources (stage_kernels.cuh, f2x.cuh, then the
-    tuning table stage_tuning.h)."""
+    """sha256 of the stage kernel sources."""
     import hashlib
     h = hashlib.sha256()
-    for f in ("stage_kernels.cuh", "f2x.cuh", "stage_tuning.h"):
-        h.update(open(os.path.join(ROOT, "paper_2505_15771_gb300", "csrc", f), "rb").read())
+    for f in stage_sources():
+        h.update(open(f, "rb").read())
     return h.hexdigest()
+
+
+STAGE_KERNEL = r"(stage|team)_kernel<(\w+), ?(?:\(int\))?(\d), ?(?:\(int\))?1(?:, ?(?:\(int\))?(\d+))?>"
+
+
+def stage_kernel_name(torch, run):
+    """The ERK stage kernel that run() launches, from the device's activity list:
+    stage_kernel<T,k,1> (one thread a cell) or team_kernel<T,k,1,W> (W warps for 32
+    cells).  "stage kernel" where the profiler reports no kernels."""
+    import re
+    from torch.profiler import ProfilerActivity, profile
+    for _ in range(2):   # a process's first profile may report nothing
+        with profile(activities=[ProfilerActivity.CUDA]) as p:
+            run()
+            torch.cuda.synchronize()
+        for e in p.events():
+            g = re.search(STAGE_KERNEL, e.name)
+            if g:
+                return "%s_kernel<%s,%s,1%s>" % (g.group(1), g.group(2), g.group(3), "," + g.group(4) if g.group(4) else "")
+    return "stage kernel"
 
 
 def measured_traffic(k, cell_dofs, arith="f64"):
@@ -235,14 +269,14 @@ def write_traffic_record(captures, out_path=None):
     ``captures``: (csv path, nx, ny, k) of each capture on the nx x ny
     bilayer.  Per arithmetic (the kernel's template type: double -> k<k>,
     f2x -> f32x2_k<k>, float -> f32_k<k>) and k, the mean over the captured
-    ERK stage launches (stage_kernel<T, k, 1>) divided by the captured case's
+    ERK stage launches (stage_kernel<T, k, 1> or team_kernel<T, k, 1, W>) divided by the captured case's
     cell DOFs, keyed by the current stage sources."""
     import csv
     import collections
     import re
     scale = {"byte": 1.0, "Kbyte": 1e3, "Mbyte": 1e6, "Gbyte": 1e9, "ns": 1e-3, "us": 1.0, "usecond": 1.0,
              "msecond": 1e3, "ms": 1e3}
-    pat = re.compile(r"stage_kernel<(\w+), ?(?:\(int\))?(\d), ?(?:\(int\))?1>")
+    pat = re.compile(STAGE_KERNEL)
     out = {}
     for path, nx, ny, k in captures:
         nx, ny, k = int(nx), int(ny), int(k)
@@ -256,8 +290,8 @@ def write_traffic_record(captures, out_path=None):
         by_key = collections.defaultdict(list)
         for (_, name), m in per.items():
             g = pat.search(name)
-            if g and int(g.group(2)) == k and g.group(1) in TRAFFIC_KEYS:
-                by_key[TRAFFIC_KEYS[g.group(1)] % k].append(m)
+            if g and int(g.group(3)) == k and g.group(2) in TRAFFIC_KEYS:
+                by_key[TRAFFIC_KEYS[g.group(2)] % k].append(m)
         for key, ms in by_key.items():
             b = [m["dram__bytes_read.sum"] + m["dram__bytes_write.sum"] for m in ms]
             t = [m["gpu__time_duration.sum"] for m in ms]
@@ -266,9 +300,9 @@ def write_traffic_record(captures, out_path=None):
                         "dram_bytes_per_launch_per_cell_dof": sum(b) / len(b) / dofs,
                         "kernel_time_us_mean_under_ncu": sum(t) / len(t)}
     rec = {"stage_sources_sha256": stage_source_sha(),
-           "note": "ncu dram__bytes_read.sum + dram__bytes_write.sum of the ERK stage launches (stage_kernel<T,k,1>), "
+           "note": "ncu dram__bytes_read.sum + dram__bytes_write.sum of the ERK stage launches (either form), "
                    "mean over the captured launches, divided by the cell DOFs of the captured case; bench.py scales "
-                   "by the workload's cell DOFs (one thread per cell, class-sorted SoA: traffic grows in "
+                   "by the workload's cell DOFs (class-sorted SoA: traffic grows in "
                    "proportion). Keys: k<k> FP64 kernel, f32x2_k<k> double-float kernel, f32_k<k> FP32 kernel. "
                    "Written by bench.py --traffic-record."}
     rec.update(out)
@@ -443,6 +477,7 @@ def measure_batched(a, torch, hho, solver, hbm_peak):
     elt = 4 if prec in (hho.HHO_F32, hho.HHO_BF16X3) else 8
     per_launch = bytes_min / 8 * elt * S / 4
     avg = stage_ms * 1e-3 / max(nl, 1)
+    kern = stage_kernel_name(torch, lambda: P.batch_step(state, work, S, 4, 0.0, dt, 1, precision=prec))
     out = {"metric": "shot-cell-DOF updates/s per ERK stage", "value": value, "unit": "shot-cell-DOF-stage/s",
            "precision": a.batch_precision, "shots": S, "steps": steps, "ms_per_step": ms / steps,
            "workload": desc,
@@ -454,8 +489,7 @@ def measure_batched(a, torch, hho, solver, hbm_peak):
            "roofline": {"bound": "hbm", "achieved": per_launch / avg / 1e9, "peak": hbm_peak, "unit": "GB/s",
                         "frac": per_launch / avg / 1e9 / hbm_peak,
                         "algorithmic_bytes_per_launch": per_launch, "avg_launch_ms": avg * 1e3,
-                        "kernel": "stage_kernel<%s,%d,1>" % ({hho.HHO_F32: "float", hho.HHO_F64: "double",
-                                                               hho.HHO_F32X2: "f2x"}[prec], kk)}}
+                        "kernel": kern}}
     P.close()
     return out
 
@@ -679,7 +713,8 @@ def measure_arith(a, torch, hho, P, tab, dt, state, work, seis, stream, U0, arit
     avg_launch_s = stage_ms * 1e-3 / max(n_launch, 1)
     ops_per_launch = fp64_ops / a.stages
     name = "f64" if arith == hho.HHO_F64 else "f32x2"
-    kern = "stage_kernel<%s,%d,1>" % ("double" if arith == hho.HHO_F64 else "f2x", a.k)
+    kern = stage_kernel_name(torch, lambda: hho.hho_erk_step(P.ops, tab, 0.0, dt, 1, x0.data_ptr(), work.data_ptr(),
+                                                             stream.cuda_stream))
     hbm = {"bound": "hbm", "achieved": bytes_min / a.stages / avg_launch_s / 1e9, "peak": hbm_peak, "unit": "GB/s",
            "frac": bytes_min / a.stages / avg_launch_s / 1e9 / hbm_peak,
            "algorithmic_bytes_per_launch": bytes_min / a.stages,
