@@ -114,6 +114,8 @@ enum { SS_C1 = 0, SS_R, SS_C3, SS_AV, SS_TAU, SCS };
 // <= -2 interface record (-2 - r).
 constexpr int32_t NB_BOUNDARY = -1;
 
+constexpr int GB300_SMS = 152;
+
 constexpr int MAX_TARGETS = 6;        // of a stage launch: the adjoint of an accepted tableau may need six
 constexpr int MAX_PLAN_TARGETS = 4;   // of a forward tableau's stage (build_plan)
 constexpr int MAX_SOURCES = 8;

@@ -52,7 +52,7 @@ constexpr int MAX_RESTART = 64;
 // eight levels and a launch for every set of partials took 104 us of the 190 us
 // per vector on 786,432 values.
 enum { KR_DOT, KR_UPDATE, KR_UPDATE_DOT, KR_UPDATE_NORM, KR_NORM, KR_RESIDUAL };
-constexpr int KR_THREADS = 256, KR_MAX_BLOCKS = 3 * 152, KR_CHUNK = 12;
+constexpr int KR_THREADS = 256, KR_MAX_BLOCKS = 3 * GB300_SMS, KR_CHUNK = 12;
 
 struct KrylovArgs {
     const double* V;
@@ -198,7 +198,7 @@ __global__ void terms_kernel(double* y, Terms T, int64_t n) {   // y may be one 
     }
 }
 
-int grid_for(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 8)); }
+int grid_for(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, GB300_SMS * 8)); }
 
 }  // namespace
 
@@ -339,7 +339,7 @@ void apply_op(hho_ops* ops, const double* v, double* out, double* tr, double a_d
 // that colour is column i of its block, because no two cells of a colour
 // share a face (nor an interface face).  The blocks are inverted in place
 // (Gauss-Jordan with partial pivoting, one CTA per cell) and applied as
-// y = P^-1 x, one thread per (row, cell), coalesced over cells.
+// y = P^-1 x, a block of warps for 32 cells (bj_kernel, sdirk_bj.cu).
 
 // Greedy colouring of the cells (fluid slots 0..Nf-1, solid Nf..Nf+Ns-1;
 // padding slots -1) so that face neighbours, across an interface too,

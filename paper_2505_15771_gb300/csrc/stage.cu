@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(128)
 
 template <class T, class TO>
 void launch_record(const hho_ops* ops, int n_shots, const T* state, TO* out, StageClock* clock, cudaStream_t st) {
-    const int threads = (int64_t)ops->n_rec * n_shots <= 16 * 152 ? 32 : 128, per = threads / REC_LANES;
+    const int threads = (int64_t)ops->n_rec * n_shots <= 16 * GB300_SMS ? 32 : 128, per = threads / REC_LANES;
     launch_dependent(record_kernel<T, TO>, dim3((ops->n_rec + per - 1) / per, n_shots), threads, 0, st, ops->dev,
                      ops->n_rec, ops->d_rec_int, ops->d_rec_dbl, state, ops->n_state, out, clock);
 }
@@ -752,7 +752,7 @@ __global__ void from_pairs_kernel(const f2x* __restrict__ x, double* __restrict_
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         y[i] = pair_to_f64(x[i]);
 }
-int pairs_grid(int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, 152 * 16); }
+int pairs_grid(int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, GB300_SMS * 16); }
 }  // namespace
 
 // Single-shot stepping: FP64, or double-float on a pair copy of the state

@@ -1694,8 +1694,8 @@ __device__ __forceinline__ void tau_cell(const StageArgsT<T>& A, const GradArgsT
 // forward stage value, taken straight into the gradient sums instead of being
 // stored.  y = 0: the mass part, y = 1: the tau part, which share nothing but the
 // traces they read; side by side they halve the chain of a thread and fill a
-// grid of one wave (65,536 cells, k = 2: FP64 44.4 -> 42.8 us, FP32 30.1 -> 20.8; 40.8 and 19.2
-// with the block counts of stage_tuning.h).
+// grid of one wave (65,536 cells, k = 2: FP64 44.4 -> 42.8 us, FP32 30.1 -> 20.8; 42.9 and
+// 21.6 since values are brought to unit size first, Range).
 template <class T, int K>
 __global__ void __launch_bounds__(128, MinBlocks<T, K>::value)
     grad_stage_kernel(const StageArgsT<T> A, const GradArgsT<T> G) {
@@ -1745,13 +1745,13 @@ namespace hho_stage {
 
 // Threads of a stage block (the kernels use no block-wide barrier).  128 for
 // large grids.  A grid of at most 20 warps per SM runs in one wave, where
-// blocks of one warp spread the cells evenly over the SMs: with 128 threads
-// the 65,536 cells of the 256 x 256 adjoint leave SMs with 3 or 4 blocks, and
-// a stage took 49.0 us against 41.6 when that was measured (its gradients 55.0
-// against 46.7).  With
-// several waves the smaller blocks cost 1 to 10 % (21 FP32 shots: 354 us
-// against 321, whose shared memory per block leaves fewer resident warps).
-inline int stage_threads(int64_t warps) { return warps <= 20 * 152 ? 32 : 128; }
+// blocks of one warp spread the cells evenly over the SMs, while blocks of four
+// leave some SMs with one more than others.  us a launch with 32 | 64 | 128 threads:
+// 2048 warps, FP64, squares k = 2 32.3 | 34.8 | 39.9, triangles k = 3 102 | 112 | 126,
+// FP32 triangles k = 3 14.8 | 15.5 | 16.9, gradients (k = 2) FP64 42.9 | 42.1 | 44.5, FP32
+// 21.6 | 20.3 | 20.8; 4200 warps, FP64 squares k = 2 73.2 | 73.8 | 72.2; 8192 warps
+// 121.1 | 121.1 | 121.3.
+inline int stage_threads(int64_t warps) { return warps <= 20 * GB300_SMS ? 32 : 128; }
 
 template <class T, int K, int MODE, int W>
 struct TeamTag {};

@@ -11,9 +11,11 @@
 //               orientation looped over its two faces (compact code, fewer
 //               live registers); 0: four unrolled bodies with constant signs.
 // tune.py (beside the package) rewrites these tables from timings of
-// candidate builds on the target GPU; the values here are the fastest it
-// and the earlier sweeps found on GB300 for the 1024 x 512 bilayer (FP64,
-// double-float) and the batched hybrid and basin meshes (FP32).
+// candidate builds on the target GPU, over values that include all of these.
+// The values here are the fastest found on GB300 for the 1024 x 512 bilayer
+// (FP64, double-float), 16 shots of the 680 x 340 hybrid mesh (FP32, k = 3) and 21
+// shots of the 331 x 167 hanging mesh (FP32, k = 2); the figures stand at
+// MinBlocks, L2Prefetch and AccSmem in stage_kernels.cuh.
 #pragma once
 
 struct StageTuning {

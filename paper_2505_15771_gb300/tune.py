@@ -23,7 +23,7 @@ win with them).  This tool measures it:
     python -m paper_2505_15771_gb300.tune --arith f32 --k 3 --workload hybrid --write
 
 Workloads: bilayer (the 1024 x 512 two-layer mesh, one shot, FP64 or
-double-float, hho_erk_step), hybrid (the 1.2 M-cell quad/triangle mesh, 16
+double-float, hho_erk_step; 1536 x 768 for double-float at k = 3), hybrid (the 1.2 M-cell quad/triangle mesh, 16
 shots, batched FP32) and basin (the 3.3 M-cell basin with hanging nodes, 32
 shots, batched FP32).  The library must have been built in-tree first.
 """
@@ -40,7 +40,7 @@ from . import build as B
 
 HEADER = os.path.join(B.CSRC, "stage_tuning.h")
 TABLE = {"f64": "TUNED_F64", "f32": "TUNED_F32", "f2x": "TUNED_F2X"}
-AXES = {"min_blocks": [4, 5, 6, 8, 10, 12], "acc_smem": [0, 1], "prefetch": [0, 16, 48, 50], "rect_loop": [0, 1]}
+AXES = {"min_blocks": [4, 5, 6, 8, 10, 12], "acc_smem": [0, 1], "prefetch": [0, 16, 34, 48, 50, 51], "rect_loop": [0, 1]}
 FIELDS = ("min_blocks", "acc_smem", "prefetch", "rect_loop")
 _TABLE_RE = r"constexpr StageTuning %s = \{\{([^}]*)\}, \{([^}]*)\}, \{([^}]*)\}, \{([^}]*)\}\};"
 
@@ -84,7 +84,9 @@ def time_workload(arith, k, workload, steps, warmup):
     # stage operator on squares, and a margin below it on the right-triangle
     # grids
     if workload == "bilayer":
-        w = synth.bilayer_c2(nx=1024, ny=512, k=k)
+        # the tables set the one thread a cell form, which double-float k = 3 takes from 24,000 warps of cells on
+        scale = 3 if (arith, k) == ("f2x", 3) else 2
+        w = synth.bilayer_c2(nx=512 * scale, ny=256 * scale, k=k)
         P = solver.Problem(w["mesh"], w["media"], k)
         P.set_sources([w["source"]], [(0.0, 1.0)], 10.0)
         P.set_arithmetic(hho.HHO_F64 if arith == "f64" else hho.HHO_F32X2)
