@@ -43,6 +43,7 @@
 #include "dependent_launch.cuh"
 #include "f2x.cuh"
 #include "hho_internal.h"
+#include "smem_opt_in.h"
 #include "stage_launch.h"
 #include "stage_tuning.h"
 
@@ -1721,20 +1722,16 @@ __global__ void __launch_bounds__(128, MinBlocks<T, K>::value)
 // register budget allows.  `Tag` makes one state per kernel.
 template <class Tag, class F>
 void stage_smem_attributes(F* kernel, size_t smem, bool carve) {
-    static size_t opted[64] = {};
-    static bool carved[64] = {};
+    static SmemOptIn state;
     int dev = 0;
     cudaGetDevice(&dev);
-    const bool known = dev >= 0 && dev < 64;
-    if (smem > 48 * 1024 && (!known || opted[dev] < smem)) {
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (known) opted[dev] = smem;
-    }
-    if (carve && (!known || !carved[dev])) {
-        cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-        if (known) carved[dev] = true;
-    }
+    state.require(
+        dev, smem, carve,
+        [&](size_t n) { cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n); },
+        [&] {
+            cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 (int)cudaSharedmemCarveoutMaxShared);
+        });
 }
 template <class T, int K, int MODE>
 struct StageTag {};

@@ -6,6 +6,11 @@ namespace {
 #include "stage_tc.cuh"
 }  // namespace
 
+namespace {
+template <int K, int MODE>
+struct TcTag {};
+}  // namespace
+
 namespace hho_stage {
 
 // The tensor-core stage (HHO_BF16X3): 32 consecutive cells of one class
@@ -26,13 +31,7 @@ void launch_tc(const hho_ops* ops, const StageArgsT<float>& a, int n_shots, cuda
     T.cols = ops->tc_cols;
     T.error = ops->d_tc_err;
     const size_t smem = (size_t)2 * 2 * 128 * ops->tc_kmax + (size_t)ops->tc_bmax;
-    static size_t opted[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (smem > 48 * 1024 && (dev < 0 || dev >= 64 || opted[dev] < smem)) {
-        cudaFuncSetAttribute(stage_tc_kernel<K, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (dev >= 0 && dev < 64) opted[dev] = smem;
-    }
+    stage_smem_attributes<TcTag<K, MODE>>(stage_tc_kernel<K, MODE>, smem, false);
     stage_tc_kernel<K, MODE><<<grid, 128, smem, s>>>(a, T);
 }
 
