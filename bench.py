@@ -421,6 +421,7 @@ def measure_batched(a, torch, hho, solver, hbm_peak):
     torch.cuda.synchronize()
     graph_ms = g0.elapsed_time(g1)
     P.set_launch_mode(hho.HHO_LAUNCH_AUTO)
+    kern = stage_kernel_name(torch, lambda: P.batch_step(state, work, S, 4, 0.0, dt, 1, precision=prec))
     # the same shots with the dense local products on the tcgen05 tensor
     # cores (split BF16, FP32 accumulation), from the same start
     tensor_core = None
@@ -477,7 +478,6 @@ def measure_batched(a, torch, hho, solver, hbm_peak):
     elt = 4 if prec in (hho.HHO_F32, hho.HHO_BF16X3) else 8
     per_launch = bytes_min / 8 * elt * S / 4
     avg = stage_ms * 1e-3 / max(nl, 1)
-    kern = stage_kernel_name(torch, lambda: P.batch_step(state, work, S, 4, 0.0, dt, 1, precision=prec))
     out = {"metric": "shot-cell-DOF updates/s per ERK stage", "value": value, "unit": "shot-cell-DOF-stage/s",
            "precision": a.batch_precision, "shots": S, "steps": steps, "ms_per_step": ms / steps,
            "workload": desc,
