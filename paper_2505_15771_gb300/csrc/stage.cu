@@ -531,8 +531,8 @@ struct HostPipe {
 // Whether erk_run replays the step as a graph.  AUTO does not: consecutive stages
 // of a stream are dependent launches that overlap across steps too, while a graph
 // ends with its step, and the host launches a stage in less time than the
-// smallest one runs (512 triangles, k = 1, four stages and a record: 28.2 us a
-// step launched, 34.9 replayed).
+// smallest one runs (512 triangles, k = 1, four stages and a record: 28.3 us a
+// step launched, 36.9 replayed).
 static bool uses_graph(const hho_ops* ops) {
     return !ops->prof_on && ops->d_clock && !ops->src_sampled && ops->launch_mode == HHO_LAUNCH_GRAPH;
 }
